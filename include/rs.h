@@ -602,7 +602,9 @@ typedef enum rs_debug_knob {
   RS_DEBUG_TRACE_PTR = 3,         /* device u64 buffer [tiles][16] for onesweep phase data; 0 off */
   RS_DEBUG_TRACE_TILES = 4,       /* number of tiles the trace buffer holds */
   RS_DEBUG_TRACE_PASS = 5,        /* the digit pass whose tiles are traced */
-  RS_DEBUG_LB_SMALL = 6,          /* look-back windows of 8 status words instead of 32 */
+  RS_DEBUG_LB_SMALL = 6,          /* accepted, without effect */
+  RS_DEBUG_MIRROR_LANES = 8,      /* 1: lanes take their keys in reverse, so that equal digits
+                                     draw their ranks out of turn and every tile needs repair */
   RS_DEBUG_BAD_INDEX_TILE = 7     /* debug build only (else RS_ERR_INVALID): this tile of
                                      digit pass 0 of a multi-launch sort computes scatter
                                      indices past the array, so that the bounds checks of

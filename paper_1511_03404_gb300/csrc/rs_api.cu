@@ -99,7 +99,7 @@ static std::atomic<long long> g_drop_pass{-1};
 static std::atomic<long long> g_trace_ptr{0};
 static std::atomic<long long> g_trace_tiles{0};
 static std::atomic<long long> g_trace_pass{0};
-static std::atomic<long long> g_lb_small{0};
+static std::atomic<long long> g_mirror{0};
 static std::atomic<long long> g_dbg_bad_tile{-1};
 
 bool pdl_enabled() {
@@ -133,7 +133,7 @@ Knobs knobs_now() {
   k.trace = reinterpret_cast<uint64_t*>(g_trace_ptr.load());
   k.trace_tiles = uint32_t(g_trace_tiles.load());
   k.trace_pass = int32_t(g_trace_pass.load());
-  k.lb_small = int32_t(g_lb_small.load());
+  k.mirror = int32_t(g_mirror.load() != 0);
   k.dbg_bad_tile = int32_t(g_dbg_bad_tile.load());
   return k;
 }
@@ -681,7 +681,9 @@ rs_status rs_debug_set(rs_debug_knob knob, long long value) {
       g_trace_pass.store(value);
       return RS_OK;
     case RS_DEBUG_LB_SMALL:
-      g_lb_small.store(value);
+      return RS_OK;  // accepted, without effect
+    case RS_DEBUG_MIRROR_LANES:
+      g_mirror.store(value);
       return RS_OK;
     case RS_DEBUG_BAD_INDEX_TILE:
 #ifdef RS_DEBUG

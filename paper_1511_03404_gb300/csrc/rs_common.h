@@ -17,13 +17,21 @@ constexpr uint32_t kValueMask = (1u << kFlagShift) - 1u;
 
 constexpr int kMaxPasses = 16;  // 64-bit keys at 4-bit digits
 
-// Look-back groups: every kGroupTiles consecutive tiles of a pass also sum
-// their digit counts into one group word per digit (count in the low 24 bits,
-// number of tiles that added in the high 8), and the group's last tile
-// publishes the inclusive prefix through the group's end.
-constexpr int kGroupTiles = 32;
+// Look-back of a whole-array pass, per digit.  A tile publishes its count in a
+// 16-bit word (bit 15: published) and adds it to its group's (8 tiles) and its
+// super's (64 tiles): count in the low 24 bits, tiles that added in the high
+// 8.  The last tile of a super publishes the inclusive prefix through it.
+constexpr uint32_t kTilePublished = 0x8000u;
+constexpr int kGroupTiles = 8;
+constexpr int kSuperGroups = 8;
+constexpr int kSuperTiles = kGroupTiles * kSuperGroups;
 constexpr uint32_t kGroupOne = 1u << 24;
 constexpr uint32_t kGroupCountMask = kGroupOne - 1u;
+
+// The look-back words of one pass.
+struct LookBackWords {
+  uint32_t *status, *gagg, *sagg, *sinc;
+};
 
 // Device status codes (the values of rs_status).
 constexpr uint32_t kDevOk = 0;
@@ -58,7 +66,8 @@ struct Knobs {
   uint64_t* trace;         // device [trace_tiles][16] phase timestamps (ns) and counters, or null
   uint32_t trace_tiles;    // tiles 0 .. trace_tiles-1 of trace_pass are recorded
   int32_t trace_pass;
-  int32_t lb_small;        // test-only: look-back windows of 8 instead of 32 words
+  int32_t mirror;          // test-only: every warp's lanes take their keys in reverse, so that
+                           // equal digits draw their ranks out of turn
   int32_t dbg_bad_tile;    // debug builds only: this tile of pass 0 computes scatter
                            // indices past the array, which the bounds checks drop (-1: off)
 };
@@ -124,30 +133,48 @@ __host__ __device__ __forceinline__ size_t lb_index(uint32_t t, uint32_t d) {
 //   [0, 256)            Ctrl
 //   counts   u32 [passes][radix]    digit histograms (atomics; zeroed per call)
 //   offsets  u32 [passes][radix]    exclusive scans of the histograms
-//   status   u32 [passes][tiles/4][radix][4]   look-back words of the tiles
-//   gagg     u32 [passes][groups/4][radix][4]  group digit counts (+ tiles added)
-//   ginc     u32 [passes][groups/4][radix][4]  group inclusive prefixes
-// Four consecutive tiles (groups) of one digit are adjacent, so a look-back
-// thread fetches four of them with one 16-byte load, and a warp's loads (32
-// digits) are one contiguous 512-byte block.  status, gagg and ginc are one
-// range, zeroed by the upsweep; tile and group counts are rounded up to 4.
+//   status   u16 [passes][tiles][radix]   look-back words of the tiles
+//   gagg     u32 [passes][groups][radix]  group counts (+ tiles added)
+//   sagg     u32 [passes][supers][radix]  super counts (+ tiles added)
+//   sinc     u32 [passes][supers][radix]  super inclusive prefixes
+// A warp's 32 digits are side by side in all of them, so that each of its
+// stores, atomics and loads is one line.  (Four groups of one digit side by
+// side, fetched by one 16-byte load, took 2.5 times the sectors.)  The words
+// are one range, zeroed by the upsweep.  The size asked of the caller is what
+// 32-bit tile words with two words per 32 tiles would take: somewhat more.
 struct Layout {
-  size_t counts, offsets, status, gagg, ginc, status_bytes, total, memset_bytes;
-  size_t tiles, groups;
+  size_t counts, offsets, status, gagg, sagg, sinc, status_bytes, total, memset_bytes;
+  size_t tiles, groups, supers;  // rounded up
+  size_t radix;
+
+  // the words of pass p
+  __host__ __device__ LookBackWords words(void* ws, int p) const {
+    char* w = static_cast<char*>(ws);
+    auto at = [&](size_t off, size_t words_per_pass) {
+      return reinterpret_cast<uint32_t*>(w + off) + size_t(p) * words_per_pass;
+    };
+    return LookBackWords{at(status, tiles * radix / 2), at(gagg, groups * radix),
+                         at(sagg, supers * radix), at(sinc, supers * radix)};
+  }
 };
 
 inline Layout onesweep_layout(int passes, int radix_bits, size_t tiles) {
   Layout L;
   const size_t radix = size_t(1) << radix_bits;
-  L.tiles = align_up(tiles, 4);
+  L.radix = radix;
+  L.tiles = align_up(tiles, 8);
   L.groups = align_up((tiles + kGroupTiles - 1) / kGroupTiles, 4);
+  L.supers = align_up((tiles + kSuperTiles - 1) / kSuperTiles, 4);
   L.counts = 256;
   L.offsets = align_up(L.counts + size_t(passes) * radix * 4, 256);
   L.status = align_up(L.offsets + size_t(passes) * radix * 4, 256);
-  L.gagg = L.status + size_t(passes) * L.tiles * radix * 4;
-  L.ginc = L.gagg + size_t(passes) * L.groups * radix * 4;
-  L.status_bytes = align_up(L.ginc + size_t(passes) * L.groups * radix * 4 - L.status, 256);
-  L.total = L.status + L.status_bytes;
+  L.gagg = L.status + size_t(passes) * L.tiles * radix * 2;
+  L.sagg = L.gagg + size_t(passes) * L.groups * radix * 4;
+  L.sinc = L.sagg + size_t(passes) * L.supers * radix * 4;
+  L.status_bytes = align_up(L.sinc + size_t(passes) * L.supers * radix * 4 - L.status, 256);
+  const size_t asked = size_t(passes) * radix * 4 *
+                       (align_up(tiles, 4) + 2 * align_up((tiles + 31) / 32, 4));
+  L.total = L.status + (asked > L.status_bytes ? align_up(asked, 256) : L.status_bytes);
   L.memset_bytes = L.offsets;  // Ctrl + counts
   return L;
 }

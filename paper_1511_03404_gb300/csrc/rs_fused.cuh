@@ -22,16 +22,16 @@
 
 namespace rs {
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 struct FusedSmem {
-  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS>;
+  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   static constexpr int RADIX = 1 << RADIX_BITS;
   static constexpr int MAXP = (8 * int(sizeof(K)) + RADIX_BITS - 1) / RADIX_BITS;
   static constexpr int OFF = (S::BYTES + 15) / 16 * 16;  // u32 [MAXP][RADIX] digit offsets
   static constexpr int FLAG = OFF + MAXP * RADIX * 4;    // u32: barrier outcome
   static constexpr int BYTES = FLAG + 16;
   // the histograms of step 1 use the warp-counter region of the tile
-  static_assert(MAXP * RADIX <= S::WARPS * RADIX, "histograms fit the warp counters");
+  static_assert(MAXP <= S::WARPS, "histograms fit the warp counters");
 };
 
 // All CTAs of the grid meet; false if the wait ran out or an error was
@@ -50,16 +50,14 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* ctrl, uint32_t gen, uint64_t 
   return *s_flag != 0u;
 }
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB, bool INDEX>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_fused(K* __restrict__ k0, K* __restrict__ k1, ValT<VB>* __restrict__ v0,
             ValT<VB>* __restrict__ v1, uint32_t n, int begin_bit, int end_bit, int passes,
-            uint32_t* __restrict__ counts, uint32_t* __restrict__ status,
-            uint32_t* __restrict__ gagg, uint32_t* __restrict__ ginc, uint32_t tiles,
-            uint32_t tiles_pad, uint32_t groups_pad, uint4* __restrict__ zero_base,
-            uint64_t zero_vec4, Ctrl* __restrict__ ctrl, Knobs knobs, KeyXf<K> xf,
+            uint32_t* __restrict__ counts, Layout lay, uint32_t tiles,
+            uint4* __restrict__ zero_base, uint64_t zero_vec4, Ctrl* __restrict__ ctrl, Knobs knobs, KeyXf<K> xf,
             uint32_t shape) {
-  using F = FusedSmem<K, VB, RADIX_BITS, THREADS, ITEMS>;
+  using F = FusedSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   using S = typename F::S;
   constexpr int RADIX = F::RADIX, MAXP = F::MAXP;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -123,28 +121,15 @@ __global__ void __launch_bounds__(THREADS, MINB)
   // ---- 3. the passes that move data
   for (int p = 0; p < passes; ++p) {
     if (!((exec >> p) & 1u)) continue;
-    const bool from_alt = (__popc(exec & ((1u << p) - 1u)) & 1) != 0;
-    TileArgs<K, VB> t;
-    t.ksrc = from_alt ? k1 : k0;
-    t.kdst = from_alt ? k0 : k1;
-    t.vsrc = from_alt ? v1 : v0;
-    t.vdst = from_alt ? v0 : v1;
-    t.n = n;
-    const int lo = begin_bit + p * RADIX_BITS;
-    t.shift = uint32_t(lo);
-    t.mask = (1u << min(RADIX_BITS, end_bit - lo)) - 1u;
-    t.pass_offsets = s_off + p * RADIX;
-    t.status = status + size_t(p) * tiles_pad * RADIX;
-    t.tile0 = 0u;
-    t.gagg = gagg + size_t(p) * groups_pad * RADIX;
-    t.ginc = ginc + size_t(p) * groups_pad * RADIX;
-    t.tiles = tiles;
-    t.lb_words = uint64_t(tiles_pad) * RADIX;
-    t.g_words = uint64_t(groups_pad) * RADIX;
-    t.lb_small = knobs.lb_small != 0;
-    t.xf = xf;
-    t.xin = xf.on && p == __ffs(int(exec)) - 1;
-    t.xout = xf.on && p == 31 - __clz(exec);
+    if (tid == 0) {
+      const int lo = begin_bit + p * RADIX_BITS;
+      auto* t = reinterpret_cast<TileArgs<K, VB>*>(smem + S::ARGS);
+      pass_args<K, VB, RADIX>(t, k0, k1, v0, v1, n, p, exec, uint32_t(lo),
+                              (1u << min(RADIX_BITS, end_bit - lo)) - 1u, s_off + p * RADIX,
+                              lay.words(ctrl, p), tiles, xf, knobs);
+      t->trace = nullptr;
+      t->bad_tile = -1;
+    }
     if (rec) ctrl->t_pass[p][0] = stat_now(ctrl);
     for (;;) {
       __syncthreads();  // the previous tile is done with s_misc
@@ -155,11 +140,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
       __syncthreads();
       const uint32_t tile = s_misc[0];
       if (tile >= tiles) break;  // CTA-uniform
-      t.tile = tile;
-      t.silent = (int(tile) == knobs.drop_tile) && (p == knobs.drop_pass);
-      t.dbg_bad = false;
-      t.trace = nullptr;
-      onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, true>(t, ctrl, knobs.timeout_ns, smem);
+      onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, true>(tile, ctrl, knobs.timeout_ns,
+                                                                    smem);
     }
     ++gen;
     if (!grid_barrier(ctrl, gen, knobs.timeout_ns, s_flag)) return;

@@ -14,15 +14,15 @@ const Variant* variants_k32(int* count) {
       OnesweepSort<uint32_t, 0, 7, 256, 16, 4>::describe(),
       SmallSort<uint32_t, 0, 8, 256, 16>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 16, 4, true>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 16, 5>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 256, 8, 4>::describe(),
       FusedSort<uint32_t, 0, 8, 256, 16, 4>::describe(),
       FusedSort<uint32_t, 0, 8, 256, 8, 4>::describe(),
       ClusterSort<uint32_t, 0, 8, 512, 16, 8>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 15, 4, true, 16>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 17, 4, true, 16>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 37, 2, true, 16, true>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 37, 2, true, 16>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 256, 33, 2, true, 16>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 256, 22, 4, true>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 256, 45, 2, true>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 256, 31, 3, true>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 384, 31, 2, true>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 512, 23, 2, true>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

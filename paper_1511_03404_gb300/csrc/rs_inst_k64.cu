@@ -14,11 +14,11 @@ const Variant* variants_k64(int* count) {
       OnesweepSort<uint64_t, 0, 8, 256, 12, 3, true>::describe(),
       FusedSort<uint64_t, 0, 8, 256, 12, 3>::describe(),
       ClusterSort<uint64_t, 0, 8, 512, 16, 8>::describe(),
-      OnesweepSort<uint64_t, 0, 8, 256, 13, 3, true, 16>::describe(),
-      OnesweepSort<uint64_t, 0, 8, 256, 11, 3, true, 16>::describe(),
-      OnesweepSort<uint64_t, 0, 8, 256, 15, 3, true, 16, true>::describe(),
-      OnesweepSort<uint64_t, 0, 8, 256, 27, 2, true, 16, true>::describe(),
-      OnesweepSort<uint64_t, 0, 8, 256, 23, 2, true, 16>::describe(),
+      OnesweepSort<uint64_t, 0, 8, 256, 16, 3, true>::describe(),
+      OnesweepSort<uint64_t, 0, 8, 256, 25, 2, true>::describe(),
+      OnesweepSort<uint64_t, 0, 8, 384, 16, 2, true>::describe(),
+      OnesweepSort<uint64_t, 0, 8, 256, 11, 4, true>::describe(),
+      OnesweepSort<uint64_t, 0, 8, 512, 11, 2, true>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

@@ -17,11 +17,11 @@ const Variant* variants_kv32(int* count) {
       FusedSort<uint32_t, 4, 8, 256, 16, 4>::describe(),
       FusedSort<uint32_t, 4, 8, 256, 8, 4>::describe(),
       ClusterSort<uint32_t, 4, 8, 512, 16, 8>::describe(),
-      OnesweepSort<uint32_t, 4, 8, 256, 15, 4, true, 16>::describe(),
-      OnesweepSort<uint32_t, 4, 8, 256, 17, 4, true, 16>::describe(),
-      OnesweepSort<uint32_t, 4, 8, 256, 33, 2, true, 16>::describe(),
-      OnesweepSort<uint32_t, 4, 8, 256, 41, 2, true, 16>::describe(),
-      OnesweepSort<uint32_t, 4, 8, 256, 45, 2, true, 16>::describe(),
+      OnesweepSort<uint32_t, 4, 8, 256, 18, 4, true>::describe(),
+      OnesweepSort<uint32_t, 4, 8, 256, 41, 2, true>::describe(),
+      OnesweepSort<uint32_t, 4, 8, 256, 26, 3, true>::describe(),
+      OnesweepSort<uint32_t, 4, 8, 384, 26, 2, true>::describe(),
+      OnesweepSort<uint32_t, 4, 8, 512, 19, 2, true>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

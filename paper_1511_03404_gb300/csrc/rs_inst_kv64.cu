@@ -14,10 +14,10 @@ const Variant* variants_kv64(int* count) {
       OnesweepSort<uint64_t, 8, 8, 256, 12, 2, true>::describe(),
       FusedSort<uint64_t, 8, 8, 256, 12, 2>::describe(),
       ClusterSort<uint64_t, 8, 8, 512, 8, 8>::describe(),
-      OnesweepSort<uint64_t, 8, 8, 256, 13, 2, false, 16>::describe(),
-      OnesweepSort<uint64_t, 8, 8, 256, 11, 2, false, 16>::describe(),
-      OnesweepSort<uint64_t, 8, 8, 256, 23, 2, true, 16>::describe(),
-      OnesweepSort<uint64_t, 8, 8, 256, 19, 2, true, 16>::describe(),
+      OnesweepSort<uint64_t, 8, 8, 256, 14, 3, true>::describe(),
+      OnesweepSort<uint64_t, 8, 8, 256, 23, 2, true>::describe(),
+      OnesweepSort<uint64_t, 8, 8, 384, 14, 2, true>::describe(),
+      OnesweepSort<uint64_t, 8, 8, 512, 10, 2, true>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

@@ -6,8 +6,7 @@
 //               takes the exclusive scan of each histogram (the "prefix"
 //               step) and decides which passes move data.
 //   k_onesweep  one digit pass: the tile's keys are ranked within the tile
-//               (stable: ranking-unit-major, a unit being a warp or half a
-//               warp, then item, then lane order), the tile's
+//               (stable: warp-major, then item, then lane order), the tile's
 //               digit counts are published for the following tiles, the
 //               tile's global digit offsets come from a decoupled look-back
 //               over the preceding tiles, and the tile is scattered through
@@ -48,6 +47,16 @@ __device__ __forceinline__ uint4 ld_relaxed_v4(const uint32_t* p) {
                : "l"(p)
                : "memory");
   return v;
+}
+
+__device__ __forceinline__ uint32_t ld_relaxed_u16(const uint16_t* p) {
+  uint16_t v;
+  asm volatile("ld.relaxed.gpu.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_relaxed_u16(uint16_t* p, uint16_t v) {
+  asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(p), "h"(v) : "memory");
 }
 
 __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
@@ -123,34 +132,6 @@ __device__ __forceinline__ void warp_rank_packed(uint32_t (&dp)[ITEMS], uint32_t
     }
     __syncwarp();
     dp[j] = (d << 16) | (__shfl_sync(kFull, before, leader) + uint32_t(__popc(peers & lt)));
-  }
-}
-
-// Rank within half-warp units: lanes 0-15 and lanes 16-31 of a warp rank
-// their items separately, each half against its own counter words.  A word
-// holds the half's running count of the digit in its upper 16 bits and the
-// peer mask of the current item (one bit per lane of the half) in its lower
-// 16 bits, so an item costs a shared atomic OR, a load and the leader's store
-// (the leader's store clears the mask and advances the count at once).  wh
-// points at the half's own [RADIX] words; dp as in warp_rank_packed.
-template <int ITEMS>
-__device__ __forceinline__ void half_rank_packed(uint32_t (&dp)[ITEMS], uint32_t* wh, int lane) {
-  static_assert(ITEMS * 16 < 65536, "counts fit 16 bits");
-  const uint32_t sub = uint32_t(lane & 15);
-  const uint32_t bit = 1u << sub;
-  const uint32_t lt = bit - 1u;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const uint32_t d = dp[j];
-    atomicOr(&wh[d], bit);
-    __syncwarp();
-    const uint32_t v = wh[d];
-    __syncwarp();
-    const uint32_t peers = v & 0xffffu;
-    const uint32_t before = v >> 16;
-    if (sub == uint32_t(31 - __clz(peers))) wh[d] = (before + uint32_t(__popc(peers))) << 16;
-    __syncwarp();  // the next item's atomics come after the leader's store
-    dp[j] = (d << 16) | (before + uint32_t(__popc(peers & lt)));
   }
 }
 
@@ -258,24 +239,6 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* s
   }
   __syncthreads();
   return inc - x + s_tot[warp];
-}
-
-// Wait (bounded) until a look-back status word has a flag.  Returns the word,
-// or kFlagErr when the wait ran out or another CTA already reported an error.
-static __device__ __noinline__ uint32_t wait_status(const uint32_t* p, Ctrl* ctrl, uint64_t timeout_ns,
-                                             uint32_t tile) {
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    const uint32_t s = ld_relaxed(p);
-    if (s & kFlagMask) return s;
-    if ((it & 63u) == 0u) {
-      if (ld_relaxed(&ctrl->error) != 0u) return kFlagErr;
-      if (global_ns() - t0 > timeout_ns) {
-        report_error(ctrl, kDevTimeout, tile);
-        return kFlagErr;
-      }
-    }
-  }
 }
 
 // --------------------------------------------------------------- upsweep
@@ -425,70 +388,62 @@ __global__ void __launch_bounds__(THREADS, 1)
 // -------------------------------------------------------------- onesweep
 
 // Words of the zero source of the counter-clearing bulk copies: the counters
-// of up to 32 half-warp units (512 threads) x 256 digits.
-constexpr int kZeroWords = 8192;
+// of up to 16 warps x 256 digits.
+constexpr int kZeroWords = 4096;
 
-// UNIT: lanes per ranking unit, 32 (a warp, warp_rank_packed) or 16 (half a
-// warp, half_rank_packed).
-// INPLACE (keys only, half-warp units): the keys are staged in (digit, input)
-// order in the key buffer itself, which is free once every thread holds its
-// keys in registers; there is no separate stage, so the tile costs its keys'
-// bytes of shared memory once instead of twice.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int UNIT = 32,
-          bool INPLACE = false>
+// INDEX: the stage holds 16-bit tile slots, and keys and values stay in the
+// buffers they were loaded into until the scatter gathers them (10 bytes of
+// shared memory for a 32-bit pair).  Otherwise (keys only) it holds the keys,
+// and the next tile's keys can land in the key buffer from then on.
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 struct OnesweepSmem {
-  static_assert(UNIT == 32 || UNIT == 16, "warp or half-warp ranking units");
-  static_assert(!INPLACE || (VB == 0 && UNIT == 16), "in-place stage: keys only, half-warp units");
   static constexpr int RADIX = 1 << RADIX_BITS;
   static constexpr int WARPS = THREADS / 32;
-  static constexpr int UNITS = THREADS / UNIT;
   static constexpr int TILE = THREADS * ITEMS;
-  static constexpr int ELEM = (int(sizeof(K)) > VB) ? int(sizeof(K)) : VB;
-  static constexpr int WH = 0;                              // u32 [UNITS][RADIX] unit counters
-  // half-warp units: the counters are cleared by a bulk copy with each tile's keys
-  static constexpr uint32_t ZERO_BYTES = UNIT == 16 ? uint32_t(UNITS * RADIX * 4) : 0u;
+  static constexpr int WH = 0;                             // u32 [WARPS][RADIX] warp counters
+  // the counters are cleared by a bulk copy with each tile's keys
+  static constexpr uint32_t ZERO_BYTES = uint32_t(WARPS * RADIX * 4);
   static_assert(ZERO_BYTES <= kZeroWords * 4 && ZERO_BYTES % 16 == 0, "one bulk copy of zeros");
-  static constexpr int CNT = WH + UNITS * RADIX * 4;       // u32 [RADIX] tile counts
-  static constexpr int TSTART = CNT + RADIX * 4;           // u32 [RADIX] tile digit starts
-  static constexpr int GBASE = TSTART + RADIX * 4;         // u32 [RADIX] global base
+  static constexpr int GBASE = WH + WARPS * RADIX * 4;     // u32 [RADIX] global base
   static constexpr int TOT = GBASE + RADIX * 4;            // u32 [32]
-  static constexpr int MISC = TOT + 32 * 4;                // u32 [8]: tile, abort, next tile, ...
+  static constexpr int MISC = TOT + 32 * 4;                // u32 [8]: [0] tile, [2] error,
+                                                           // [3] next tile, [5..6] check sums
   static constexpr int MBAR = MISC + 32;                   // u64 [2] mbarriers: keys, values
-  // the tile's keys as loaded (+16 B skew); once they are staged in OUT, the
-  // tile's values are loaded here
-  static constexpr int KIN = (MBAR + 16 + 15) / 16 * 16;
-  // the tile in (digit, input) order: keys, then values; during the rank of
-  // warp units it holds the warps' peer masks (u32 [WARPS][RADIX])
-  static constexpr int OUT = INPLACE ? KIN : KIN + TILE * ELEM + 16;
-  static constexpr int MM = OUT;
-  static constexpr int OUT_BYTES =
-      TILE * ELEM > WARPS * RADIX * 4 ? TILE * ELEM : WARPS * RADIX * 4;
-  static constexpr int BYTES = INPLACE ? KIN + TILE * ELEM + 16 : OUT + OUT_BYTES;
+  static constexpr int ARGS = MBAR + 16;                   // TileArgs
+  static constexpr int KIN = ARGS + 208;   // the tile's keys as loaded (+16 B skew)
+  static constexpr int VIN = KIN + TILE * int(sizeof(K)) + 16;    // the tile's values as loaded
+  static constexpr int OUT = VIN + (VB > 0 ? TILE * VB + 16 : 0); // the stage and an end mark
+  static constexpr int BYTES = OUT + (INDEX ? (TILE + 8) * 2 : (TILE + 2) * int(sizeof(K)));
 };
 
-// Operands of one tile of one digit pass over one array (or one segment).
+// Operands of the tiles of one digit pass over one array (or one segment).
+// They lie in shared memory (written by one thread before a barrier): held in
+// registers over the resident CTAs' loop, they and what the compiler derives
+// from them cost up to 60 registers a thread, most of them spilled.
 template <class K, int VB>
 struct TileArgs {
   const K* ksrc;
   K* kdst;
   const ValT<VB>* vsrc;
   ValT<VB>* vdst;
-  uint32_t n;                   // elements of the array / segment
-  uint32_t tile;                // tile index inside the array / segment
-  uint32_t shift, mask;         // digit of this pass: (key >> shift) & mask
   const uint32_t* pass_offsets; // [RADIX] global digit offsets of this pass
-  uint32_t* status;             // [tiles/4][RADIX][4] look-back words of this pass
-  uint32_t tile0;               // index of this array's tile 0 in status (a segment's first tile)
-  uint32_t* gagg;               // [groups/4][RADIX][4] group counts of this pass, or null (flat walk)
-  uint32_t* ginc;               // [groups/4][RADIX][4] group inclusive prefixes of this pass
-  uint32_t tiles;               // tiles of this array
+  // look-back words of this pass.  Whole arrays: status u16 [tiles][RADIX],
+  // gagg [groups][RADIX], sagg and sinc [supers][RADIX].  Segments: status u32
+  // [tiles/4][RADIX][4] alone.
+  uint32_t *status, *gagg, *sagg, *sinc;
   uint64_t lb_words;            // words in status (debug bounds checks only)
-  uint64_t g_words;             // words in gagg / ginc (debug bounds checks only)
-  bool silent;                  // test-only: publish nothing for this tile
-  bool lb_small;                // test-only: 8-word look-back windows
-  bool dbg_bad;                 // debug builds, test-only: scatter indices pushed past n
-  uint64_t* trace;              // test-only: 16 phase stamps / counters of this tile, or null
+  uint64_t g_words, s_words;    // words in gagg; in sagg and in sinc (the same)
+  uint64_t* trace;              // test-only: [tiles][16] phase stamps and counters, or null
   KeyXf<K> xf;                  // order-preserving key transform of the sort
+  uint32_t n;                   // elements of the array / segment
+  uint32_t shift, mask;         // digit of this pass: (key >> shift) & mask
+  uint32_t tile0;               // index of this array's tile 0 in status (a segment's first tile)
+  uint32_t tiles;               // tiles of this array
+  uint32_t trace_tiles;         // test-only: tiles the trace holds
+  int32_t drop_tile;            // test-only: this tile publishes nothing (-1: none)
+  int32_t bad_tile;             // debug builds, test-only: this tile's scatter indices are
+                                // pushed past n (-1: none)
+  bool mirror;                  // test-only: lanes take their keys in reverse
   bool xin;                     // the source holds untransformed keys: apply xf on load
   bool xout;                    // write untransformed keys (apply xf's inverse)
 };
@@ -504,79 +459,211 @@ __device__ __forceinline__ void stamp(uint64_t* tr, int k) {
   if (tr != nullptr && threadIdx.x == 0) tr[k] = global_ns();
 }
 
-// ---- look-back walks (one thread per digit)
-
-// Bounded wait until a group word reports `need` contributing tiles.
-static __device__ __noinline__ uint32_t wait_group(const uint32_t* p, uint32_t need, Ctrl* ctrl,
-                                                   uint64_t timeout_ns, uint32_t tile, bool* ok) {
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    const uint32_t w = ld_relaxed(p);
-    if ((w >> 24) >= need) {
-      *ok = true;
-      return w;
-    }
-    if ((it & 63u) == 0u) {
-      if (ld_relaxed(&ctrl->error) != 0u) break;
-      if (global_ns() - t0 > timeout_ns) {
-        report_error(ctrl, kDevTimeout, tile);
-        break;
-      }
-    }
-  }
-  *ok = false;
-  return 0u;
-}
-
 // test-only counters of digit 0's look-back (thread 0)
 __device__ __forceinline__ void trace_add(uint64_t* tr, int k, uint64_t v) {
   if (tr != nullptr && threadIdx.x == 0) tr[k] += v;
 }
 
-// Walk the tiles from, from-1, ..., lo (indices into status) of one digit,
-// nearest first, adding their published counts to excl until an inclusive
-// prefix (done).  NB 16-byte L2 loads fetch a window of 4*NB tiles at once;
-// a warp's load is one contiguous 512-byte block (32 digits x 4 tiles).
-template <int RADIX, int NB>
-__device__ __forceinline__ void walk_tiles(const uint32_t* status, uint32_t d, int32_t from,
-                                           int32_t lo, uint32_t& excl, bool& done, bool& gave_up,
-                                           Ctrl* ctrl, uint64_t timeout_ns, uint32_t tile,
-                                           uint64_t* tr) {
-  int32_t hi = from;
-  while (!done && !gave_up && hi >= lo) {
-    trace_add(tr, 10, 1);
-    const int32_t b0 = hi >> 2;
-    uint4 v[NB];
+// The look-back of one digit (one thread): the sum of the counts of the
+// earlier tiles, in steps that a caller can put between other work.  issue()
+// starts the L2 loads, consume() adds what has arrived; finish() does both
+// until nothing is missing, every wait without progress bounded.
+//
+// Whole arrays: every tile adds its counts to its group's (8 tiles) and its
+// super's (64 tiles) when it publishes them, so the sum is at most 7 tiles, 7
+// groups and the earlier supers, nearest first: complete counts (go on) or an
+// inclusive prefix (stop; the last tile of each super publishes it).  All
+// levels are fetched at once, 18 words a thread at most, a warp's 32 digits
+// side by side.  Under load such a round trip takes 1-2 us, and how many
+// follow one another is what a look-back costs: a walk over groups of 32
+// tiles, 8 tiles at a time, took 3.8 of them a tile (5.9 of its 10.5 us, keys
+// alone at 2^26); this one takes 1.7, the first under the stage, and leaves
+// 2.8 of 9.2 us.
+template <class K, int VB, int RADIX>
+struct TreeLookBack {
+  uint32_t excl = 0u;
+  uint32_t missing = 0u;        // bit l: level l (tiles, groups, supers) is not summed yet
+  uint32_t at_tile = 0u;
+  int32_t super = -1;           // the next super to add
+  uint32_t w[kGroupTiles - 1], g[kSuperGroups - 1], agg[2], inc[2];
+
+  __device__ __forceinline__ void start(const TileArgs<K, VB>&, uint32_t tile) {
+    at_tile = tile;
+    super = int32_t(tile / kSuperTiles) - 1;
+    missing = (tile % kGroupTiles ? 1u : 0u) | (tile / kGroupTiles % kSuperGroups ? 2u : 0u) |
+              (super >= 0 ? 4u : 0u);
+  }
+
+  __device__ __forceinline__ bool done() const { return missing == 0u; }
+
+  __device__ __forceinline__ void issue(const TileArgs<K, VB>& t, uint32_t d) {
+    if (missing & 1u) {
+      const uint16_t* p = reinterpret_cast<const uint16_t*>(t.status) +
+                          size_t(at_tile / kGroupTiles * kGroupTiles) * RADIX + d;
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      const int32_t b = b0 - k;
-      v[k] = (4 * b + 3 >= lo)
-                 ? __ldcg(reinterpret_cast<const uint4*>(status + (size_t(b) * RADIX + d) * 4))
-                 : make_uint4(0u, 0u, 0u, 0u);
+      for (uint32_t c = 0; c < kGroupTiles - 1; ++c)
+        if (c < at_tile % kGroupTiles) w[c] = ld_relaxed_u16(p + c * RADIX);
     }
+    if (missing & 2u) {
+      const uint32_t* p = t.gagg + size_t(at_tile / kSuperTiles * kSuperGroups) * RADIX + d;
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
+      for (uint32_t c = 0; c < kSuperGroups - 1; ++c)
+        if (c < at_tile / kGroupTiles % kSuperGroups) g[c] = ld_relaxed(p + c * RADIX);
+    }
+    if (missing & 4u) {
 #pragma unroll
-      for (int c = 3; c >= 0; --c) {
-        const int32_t a = 4 * (b0 - k) + c;
-        if (done || gave_up || a > hi || a < lo) continue;
-        uint32_t sw = c == 0 ? v[k].x : c == 1 ? v[k].y : c == 2 ? v[k].z : v[k].w;
-        if ((sw & kFlagMask) == 0u) {
-          trace_add(tr, 12, 1);
-          sw = wait_status(status + lb_index<RADIX>(uint32_t(a), d), ctrl, timeout_ns, tile);
+      for (int c = 0; c < 2; ++c)
+        if (super >= c) {
+          agg[c] = ld_relaxed(t.sagg + size_t(super - c) * RADIX + d);
+          inc[c] = ld_relaxed(t.sinc + size_t(super - c) * RADIX + d);
         }
-        const uint32_t f = sw & kFlagMask;
-        if (f == kFlagErr) {
-          gave_up = true;
-        } else {
-          excl += sw & kValueMask;
-          if (f == kFlagInc) done = true;
+    }
+  }
+
+  __device__ __forceinline__ void consume(uint64_t* tr) {
+    if (missing != 0u) trace_add(tr, 10, 1);
+    if (missing & 1u) {
+      uint32_t sum = 0u, all = kTilePublished;
+#pragma unroll
+      for (uint32_t c = 0; c < kGroupTiles - 1; ++c)
+        if (c < at_tile % kGroupTiles) {
+          sum += w[c] & ~kTilePublished;
+          all &= w[c];
+        }
+      if (all) {
+        excl += sum;
+        missing &= ~1u;
+      }
+    }
+    if (missing & 2u) {
+      uint32_t sum = 0u;
+      bool whole = true;
+#pragma unroll
+      for (uint32_t c = 0; c < kSuperGroups - 1; ++c)
+        if (c < at_tile / kGroupTiles % kSuperGroups) {
+          sum += g[c] & kGroupCountMask;
+          whole = whole && (g[c] >> 24) == uint32_t(kGroupTiles);
+        }
+      if (whole) {
+        excl += sum;
+        missing &= ~2u;
+      }
+    }
+    if (missing & 4u) {
+      const int32_t s0 = super;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (super != s0 - c || super < 0 || !(missing & 4u)) continue;
+        if (inc[c] & kFlagMask) {
+          excl += inc[c] & kValueMask;
+          missing &= ~4u;
+        } else if ((agg[c] >> 24) == uint32_t(kSuperTiles)) {
+          excl += agg[c] & kGroupCountMask;
+          --super;
+        }
+      }
+      if (super < 0) missing &= ~4u;  // every super summed
+    }
+  }
+
+  __device__ __forceinline__ bool finish(const TileArgs<K, VB>& t, uint32_t d, Ctrl* ctrl,
+                                         uint64_t timeout_ns, uint32_t tile, uint64_t* tr) {
+    uint64_t t0 = 0;
+    for (uint32_t idle = 0; missing != 0u;) {
+      const uint32_t m0 = missing;
+      const int32_t s0 = super;
+      issue(t, d);
+      consume(tr);
+      if (missing != m0 || super != s0) {
+        idle = 0;
+        continue;
+      }
+      trace_add(tr, 12, 1);
+      if (idle == 0) t0 = global_ns();
+      if ((++idle & 63u) == 0u) {
+        if (ld_relaxed(&ctrl->error) != 0u) return false;
+        if (global_ns() - t0 > timeout_ns) {
+          report_error(ctrl, kDevTimeout, tile);
+          return false;
         }
       }
     }
-    hi = 4 * (b0 - NB + 1) - 1;
+    return true;
   }
-}
+};
+
+// Segments: a walk over the segment's tiles, nearest first, 8 at a time, down
+// to an inclusive prefix (every tile publishes its own once it has it).
+template <class K, int VB, int RADIX>
+struct FlatLookBack {
+  uint32_t excl = 0u;
+  int32_t at = -1, lo = 0;  // next tile to add; the segment's first
+  uint4 w[2];
+
+  __device__ __forceinline__ void start(const TileArgs<K, VB>& t, uint32_t tile) {
+    lo = int32_t(t.tile0);
+    at = tile ? lo + int32_t(tile) - 1 : lo - 1;
+  }
+
+  __device__ __forceinline__ bool done() const { return at < lo; }
+
+  __device__ __forceinline__ void issue(const TileArgs<K, VB>& t, uint32_t d) {
+    if (done()) return;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int32_t b = (at >> 2) - k;
+      w[k] = 4 * b + 3 >= lo ? ld_relaxed_v4(t.status + (size_t(b) * RADIX + d) * 4)
+                             : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+
+  __device__ __forceinline__ void consume(uint64_t* tr) {
+    if (done()) return;
+    trace_add(tr, 10, 1);
+    const int32_t b0 = at >> 2;
+    bool go = true;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int c = 3; c >= 0; --c) {
+        if (!go || 4 * (b0 - k) + c != at || at < lo) continue;
+        const uint32_t sw = c == 0 ? w[k].x : c == 1 ? w[k].y : c == 2 ? w[k].z : w[k].w;
+        const uint32_t f = sw & kFlagMask;
+        if (f == 0u) {
+          go = false;
+        } else {
+          excl += sw & kValueMask;
+          at = f == kFlagInc ? lo - 1 : at - 1;
+          go = f != kFlagInc;
+        }
+      }
+    }
+  }
+
+  __device__ __forceinline__ bool finish(const TileArgs<K, VB>& t, uint32_t d, Ctrl* ctrl,
+                                         uint64_t timeout_ns, uint32_t tile, uint64_t* tr) {
+    uint64_t t0 = 0;
+    for (uint32_t idle = 0; !done();) {
+      const int32_t at0 = at;
+      issue(t, d);
+      consume(tr);
+      if (at != at0) {
+        idle = 0;
+        continue;
+      }
+      trace_add(tr, 12, 1);
+      if (idle == 0) t0 = global_ns();
+      if ((++idle & 63u) == 0u) {
+        if (ld_relaxed(&ctrl->error) != 0u) return false;
+        if (global_ns() - t0 > timeout_ns) {
+          report_error(ctrl, kDevTimeout, tile);
+          return false;
+        }
+      }
+    }
+    return true;
+  }
+};
 
 // ---- bulk (TMA engine) copies global -> shared, completed on an mbarrier
 
@@ -638,6 +725,14 @@ __device__ __noinline__ static bool mbar_wait_bounded(uint64_t* bar, uint32_t pa
   }
 }
 
+// The same with the first try in line: a call's saved registers then cost
+// only the waits that need it.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Ctrl* ctrl,
+                                          uint64_t timeout_ns, uint32_t info) {
+  return mbar_try_wait(bar, parity) || mbar_wait_bounded(bar, parity, ctrl, timeout_ns, info) ||
+         mbar_wait_bounded(bar, parity, ctrl, timeout_ns, info);
+}
+
 // Shared-memory staging of elements [0, len) of src: element i lands at byte
 // (skew + i * sizeof(T)) of `buf`, skew = src address mod 16, so that the
 // 16-byte aligned middle ("body") goes by one bulk copy while the few head
@@ -679,8 +774,8 @@ __device__ __align__(128) uint32_t g_zero_words[kZeroWords];
 }
 
 // Start staging the keys of tile `tile` of an array of n keys into the key
-// buffer: one bulk copy issued by thread 0 on `bar`, head/tail elements and
-// the past-the-end sentinels written by every thread.  zero_dst (optional):
+// buffer: one bulk copy issued by thread 0 on `bar`, head and tail elements
+// loaded by the other threads.  zero_dst (optional):
 // zero_bytes (a multiple of 16, at most kZeroWords words) of shared memory cleared by a
 // second bulk copy on the same barrier, so that the tile's counters are zero
 // once its keys have landed, without a store loop on the shared-memory pipe.
@@ -704,10 +799,34 @@ __device__ __forceinline__ void stage_keys(unsigned char* kin, const K* ksrc, ui
     if (zero_bytes) bulk_load(zero_dst, g_zero_words, zero_bytes, bar);
   }
   sk.edges(kin, gk, tile_len);
-  // past the end: the largest digit, so these items rank after every key of
-  // the tile and are never written out
-  K* s_kin = sk.at(kin);
-  for (uint32_t i = tile_len + threadIdx.x; i < uint32_t(TILE); i += THREADS) s_kin[i] = ~K(0);
+}
+
+// Start loading tile `tile`'s keys and the cleared counters, on the keys'
+// barrier.  Every thread of the CTA calls it.
+template <class S, class K, int VB, int THREADS, bool CG>
+__device__ __forceinline__ void stage_tile(unsigned char* smem, uint32_t tile) {
+  const TileArgs<K, VB>& t = *reinterpret_cast<const TileArgs<K, VB>*>(smem + S::ARGS);
+  stage_keys<K, THREADS, S::TILE, CG>(smem + S::KIN, t.ksrc, t.n, tile,
+                                      reinterpret_cast<uint64_t*>(smem + S::MBAR), smem + S::WH,
+                                      S::ZERO_BYTES);
+}
+
+// The same for its values, on theirs.
+template <class S, class K, int VB, bool CG>
+__device__ __forceinline__ void stage_values(unsigned char* smem, uint32_t tile) {
+  const TileArgs<K, VB>& t = *reinterpret_cast<const TileArgs<K, VB>*>(smem + S::ARGS);
+  uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + S::MBAR);
+  const uint32_t base = tile * uint32_t(S::TILE);
+  const uint32_t len = min(uint32_t(S::TILE), t.n - base);
+  const ValT<VB>* gv = t.vsrc + base;
+  const Stage<ValT<VB>> sv(gv, len);
+  if (threadIdx.x == 0) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if constexpr (CG) asm volatile("fence.proxy.async.global;" ::: "memory");
+    mbar_arrive_expect_tx(&s_bar[1], sv.body);
+    sv.issue(smem + S::VIN, gv, &s_bar[1]);
+  }
+  sv.edges(smem + S::VIN, gv, len);
 }
 
 // Persistent CTAs: where the next tile id comes from.
@@ -716,45 +835,80 @@ struct Prefetch {
   uint32_t tiles;
 };
 
-// One tile of one counting-sort pass (Sec. 2.6): stage the tile's keys in
-// shared memory, rank them, publish the tile's digit counts, look back, and
-// scatter stably; the values are fetched into the freed key buffer while the
-// look-back and the key scatter run.  Every thread of the CTA calls it.
-// Returns false (CTA-uniform) when a bounded wait gave up, in which case
-// nothing of this tile was written and no copy into shared memory is pending.
+// One tile of one counting-sort pass (Sec. 2.6), its operands at S::ARGS in
+// shared memory.  Every thread of the CTA calls it.  Returns false
+// (CTA-uniform) when a bounded wait gave up, in which case no copy into shared
+// memory is pending.
+//
+//   1. count: every warp counts its keys' digits (shared atomics);
+//   2. per digit, the sum over the warps is the tile's count, published at
+//      once, before anything is ranked; the counters become the warps' first
+//      slots in the tile;
+//   3. stage, in (digit, input) order: each warp takes its keys item by item
+//      and draws a slot from its counter of the key's digit (one returning
+//      atomicAdd); into the slot goes the key itself, or (INDEX) its 16-bit
+//      place in the tile.  The look-back's first round trip runs meanwhile;
+//   4. the rest of the look-back, then the scatter in stage order: contiguous
+//      stores inside each digit run.  With INDEX the keys are gathered from
+//      the buffer they were loaded into, then the values from theirs.
+//
+// The order of equal digits inside one warp's atomicAdd is the hardware's: on
+// sm_103a it went by lane in every pair measured (0.9e9), which is the input
+// order, but nothing promises it.  So the scatter checks what it reads:
+//   - INDEX: places ascend inside every digit run, i.e. the stage has no
+//     descents but those at the starts of runs;
+//   - keys (only sorts of whole keys, where no pass looks below or above the
+//     key's bits): the bits up to this digit ascend over the whole stage.
+//     Keys that agree in all of them need no order: later passes tell them
+//     apart, or they are equal.
+// A tile that fails is put in order (a slot drawn out of turn is less than a
+// warp away from its place) and scattered again to the same destinations.
+//
+// What bounds it: the shared-memory pipe.  Each of the accesses by a random
+// digit or slot costs 3.1-3.6 wavefronts a warp: the count, the draw, the
+// stage store and (INDEX) the gathers.  A rank by peer masks (atomicOr, its
+// load, the leader's store, then the offset's load) took two more and, item
+// after item, a chain of three of them; the returning atomic ranks 2.58e12
+// digits a second on the whole GPU, the masks 0.91e12 (random digits in
+// registers; all 32 lanes on one digit: 0.297e12 and 0.267e12).  Measured at
+// 2^26, a whole sort, before -> now, ms: u32 keys 1.09 -> 0.777, u32 pairs
+// 1.31 -> 1.075, u64 keys 3.04 -> 2.32, u64 pairs 4.08 -> 3.74; pipe busy
+// (2^24) 68 % -> 68 % (keys), 79 % (pairs) at 25.5 -> 19.0 and 34 -> 30.5
+// wavefronts per 32 elements.
 //
 // PERSIST: the calling kernel keeps the CTA resident over many tiles.  The
 // barriers are initialised once by the kernel, this tile's keys were staged
 // by the previous call (or the kernel's prologue) on barrier phase `parity`,
-// and as soon as the key buffer is free again this call takes the next tile
-// id (s_misc[3]) and starts staging its keys (s_misc[4] = 1), overlapping the
-// end of this tile.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool CG, bool PERSIST = false,
-          int UNIT = 32, bool INPLACE = false>
-__device__ __forceinline__ bool onesweep_tile(const TileArgs<K, VB>& t, Ctrl* ctrl,
-                                              uint64_t timeout_ns, unsigned char* smem,
-                                              uint32_t parity = 0u,
-                                              const Prefetch* pf = nullptr) {
+// and as soon as the key buffer is free (the keys staged, or with INDEX
+// scattered: under the values' scatter) this call takes the next tile id
+// (*next, at least pf->tiles when there is none) and starts loading it.
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX, bool CG,
+          bool PERSIST = false, bool FLAT = false>
+__device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_t timeout_ns,
+                                              unsigned char* smem, uint32_t parity = 0u,
+                                              const Prefetch* pf = nullptr,
+                                              uint32_t* next = nullptr) {
   using V = ValT<VB>;
-  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, UNIT, INPLACE>;
-  constexpr int RADIX = S::RADIX, WARPS = S::WARPS, UNITS = S::UNITS, TILE = S::TILE;
+  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
+  constexpr int RADIX = S::RADIX, WARPS = S::WARPS, TILE = S::TILE;
   static_assert(RADIX <= THREADS, "one thread per digit");
-  static_assert(TILE <= 65536, "stage slots fit 16 bits");
+  static_assert(TILE < 1 << 15, "a tile's counts fit 15 bits, its slots 16");
+  static_assert(INDEX || VB == 0, "values follow their keys' slots");
   uint32_t* s_wh = reinterpret_cast<uint32_t*>(smem + S::WH);
-  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + S::CNT);
-  uint32_t* s_tstart = reinterpret_cast<uint32_t*>(smem + S::TSTART);
   uint32_t* s_gbase = reinterpret_cast<uint32_t*>(smem + S::GBASE);
   uint32_t* s_tot = reinterpret_cast<uint32_t*>(smem + S::TOT);
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + S::MISC);
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + S::MBAR);  // [0] keys, [1] values
-  uint32_t* s_mm = reinterpret_cast<uint32_t*>(smem + S::MM);
+  static_assert(sizeof(TileArgs<K, VB>) <= S::KIN - S::ARGS, "the operands' place");
+  const TileArgs<K, VB>& t = *reinterpret_cast<const TileArgs<K, VB>*>(smem + S::ARGS);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  const uint32_t tile = t.tile, n = t.n;
   const uint32_t tile_base = tile * uint32_t(TILE);
-  const uint32_t tile_len = min(uint32_t(TILE), n - tile_base);
-  stamp(t.trace, 0);
-  if (t.trace != nullptr && tid == 0) t.trace[7] = sm_id();
+  const uint32_t tile_len = min(uint32_t(TILE), t.n - tile_base);
+  const bool silent = int(tile) == t.drop_tile;
+  auto trace = [&]() { return t.trace && tile < t.trace_tiles ? t.trace + size_t(tile) * 16 : nullptr; };
+  stamp(trace(), 0);
+  if (tid == 0 && trace()) trace()[7] = sm_id();
 
   if constexpr (!PERSIST) {
     if (tid == 0) {
@@ -762,353 +916,398 @@ __device__ __forceinline__ bool onesweep_tile(const TileArgs<K, VB>& t, Ctrl* ct
       if constexpr (VB > 0) mbar_init(&s_bar[1]);
     }
     __syncthreads();
-    // ---- stage the tile's keys (half-warp units: and clear the counters)
-    stage_keys<K, THREADS, TILE, CG>(smem + S::KIN, t.ksrc, n, tile, &s_bar[0],
-                                     smem + S::WH, S::ZERO_BYTES);
+    stage_tile<S, K, VB, THREADS, CG>(smem, tile);
+    if constexpr (VB > 0) stage_values<S, K, VB, CG>(smem, tile);
   }
-  if (tid == 0) s_misc[1] = 0u;
+  const bool landed = mbar_wait(&s_bar[0], parity, ctrl, timeout_ns, tile);
+  auto leave = [&](bool ok, bool values) {
+    if constexpr (VB > 0) {  // the value copy must not land after this call
+      if (!ok && values) {
+        mbar_wait(&s_bar[1], parity, ctrl, timeout_ns, tile);
+        __syncthreads();
+      }
+    }
+    if constexpr (!PERSIST) {
+      if (tid == 0) {
+        mbar_inval(&s_bar[0]);
+        if constexpr (VB > 0) mbar_inval(&s_bar[1]);
+      }
+    }
+    return ok;
+  };
+  if (__syncthreads_or(!landed)) return leave(false, !PERSIST);  // CTA-uniform
+  if constexpr (PERSIST && VB > 0) stage_values<S, K, VB, CG>(smem, tile);
+  stamp(trace(), 1);
+
+  // ---- 1. count.  Warp w owns tile slots [w*ITEMS*32, (w+1)*ITEMS*32); item j
+  // of lane l is slot w*ITEMS*32 + j*32 + l.  mirror (test-only): the lanes
+  // are taken in reverse, so that every repeated digit draws out of turn.
   K* s_kin = Stage<K>(t.ksrc + tile_base, tile_len).at(smem + S::KIN);
-  if constexpr (UNIT == 32) {
-    for (int i = tid; i < WARPS * RADIX; i += THREADS) {
-      s_wh[i] = 0u;
-      s_mm[i] = 0u;
-    }
-  }  // half-warp units: the bulk copy that staged the keys cleared the counters
-  bool landed = mbar_wait_bounded(&s_bar[0], parity, ctrl, timeout_ns, tile);
-  if (!landed) landed = mbar_wait_bounded(&s_bar[0], parity, ctrl, timeout_ns, tile);
-  if (__syncthreads_or(!landed)) {  // CTA-uniform
-    if constexpr (!PERSIST) {
-      if (tid == 0) {
-        mbar_inval(&s_bar[0]);
-        if constexpr (VB > 0) mbar_inval(&s_bar[1]);
-      }
-    }
-    return false;
-  }
-  if (t.xin) {  // the first pass that moves data: from here on the keys are transformed
-    for (uint32_t i = tid; i < tile_len; i += THREADS) s_kin[i] = xf_fwd(s_kin[i], t.xf);
-    __syncthreads();
-  }
-  stamp(t.trace, 1);
-
-  // ---- rank within the unit: unit u owns tile slots [u*ITEMS*UNIT, (u+1)*ITEMS*UNIT),
-  // item j of the unit's lane l is slot u*ITEMS*UNIT + j*UNIT + l.  (With
-  // half-warp units and ITEMS odd, the two halves of a warp read 16 banks
-  // apart.)
-  const int unit = tid / UNIT;
-  const uint32_t slot0 = uint32_t(unit * ITEMS * UNIT + (tid % UNIT));
-  uint32_t dp[ITEMS];  // digit << 16 | rank in the unit
-  K kreg[VB > 0 ? 1 : ITEMS];  // keys only: the keys stay in registers until staged
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const K k = s_kin[slot0 + j * UNIT];
-    if constexpr (VB == 0) kreg[j] = k;
-    dp[j] = digit_of(k, t.shift, t.mask);
-  }
-  if constexpr (UNIT == 32)
-    warp_rank_packed<ITEMS>(dp, s_wh + warp * RADIX, s_mm + warp * RADIX, lane);
-  else
-    half_rank_packed<ITEMS>(dp, s_wh + unit * RADIX, lane);
-  __syncthreads();
-  stamp(t.trace, 2);
-
-  // ---- per digit: tile count, publish it; then the exclusive prefix over
-  // the ranking units, which starts at the digit's first slot in the tile
-  uint32_t my_cnt = 0u;
-  constexpr int CSHIFT = UNIT == 32 ? 0 : 16;  // where the unit counters keep the count
-  if (tid < RADIX) {
-    uint32_t run = 0u;
-#pragma unroll
-    for (int w = 0; w < UNITS; ++w) run += s_wh[w * RADIX + tid] >> CSHIFT;
-    my_cnt = run;
-    if (!t.silent) {
-      if (dbg_ok(lb_index<RADIX>(t.tile0 + tile, tid), t.lb_words, kSiteTileStatus))
-        st_relaxed(&t.status[lb_index<RADIX>(t.tile0 + tile, tid)],
-                   (tile == 0u ? kFlagInc : kFlagAgg) | run);
-      if (t.gagg != nullptr &&
-          dbg_ok(lb_index<RADIX>(tile / kGroupTiles, tid), t.g_words, kSiteGroupAgg))
-        atomicAdd(&t.gagg[lb_index<RADIX>(tile / kGroupTiles, tid)], run | kGroupOne);
-    }
-  }
-  const uint32_t my_start = block_exclusive_scan<THREADS>(my_cnt, s_tot);
-  if (tid < RADIX) {
-    s_cnt[tid] = my_cnt;
-    s_tstart[tid] = my_start;
-    uint32_t run = my_start;
-#pragma unroll
-    for (int w = 0; w < UNITS; ++w) {
-      const uint32_t c = s_wh[w * RADIX + tid] >> CSHIFT;
-      s_wh[w * RADIX + tid] = run;
-      run += c;
-    }
-  }
-  __syncthreads();
-  stamp(t.trace, 3);
-
-  // ---- keys into the stage in (digit, input) order (the peer masks are done)
-  K* s_out = reinterpret_cast<K*>(smem + S::OUT);
-  uint32_t pos[VB > 0 ? ITEMS : 1];  // stage slots, for the values
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const uint32_t p = (dp[j] & 0xffffu) + s_wh[unit * RADIX + (dp[j] >> 16)];
-    if constexpr (VB == 0)
-      s_out[p] = kreg[j];
-    else
-      s_out[p] = s_kin[slot0 + j * UNIT];
-    if constexpr (VB > 0) pos[j] = p;
-  }
-  stamp(t.trace, 8);
-
-  // ---- the values into the key buffer, while the look-back and the key
-  // scatter run
-  V* s_vin = nullptr;
-  if constexpr (VB > 0) {
-    __syncthreads();  // every key has left the buffer
-    const V* gv = t.vsrc + tile_base;
-    const Stage<V> sv(gv, tile_len);
-    s_vin = sv.at(smem + S::KIN);
-    if (tid == 0) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive_expect_tx(&s_bar[1], sv.body);
-      sv.issue(smem + S::KIN, gv, &s_bar[1]);
-    }
-    sv.edges(smem + S::KIN, gv, tile_len);
-  }
-
-  // ---- decoupled look-back: the sum of the counts of the preceding tiles for
-  // my digit.  With groups: the earlier tiles of my group, then earlier
-  // groups nearest first, each giving either its inclusive prefix (stop) or
-  // its complete count (go on).  The walk then no longer grows with the
-  // number of tiles in flight.
-  if (tid < RADIX) {
-    uint32_t excl = 0u;
-    bool gave_up = false;
-    if (tile > 0u) {
-      bool done = false;
-      if (t.gagg == nullptr) {
-        walk_tiles<RADIX, 2>(t.status, tid, int32_t(t.tile0 + tile) - 1, int32_t(t.tile0), excl,
-                             done, gave_up, ctrl, timeout_ns, tile, t.trace);
-        if (!done && !gave_up) {  // tile 0 is inclusive: only if words were not cleared
-          report_error(ctrl, kDevIndex, tile);
-          gave_up = true;
-        }
-      } else {
-        const int32_t g = int32_t(tile / kGroupTiles);
-        walk_tiles<RADIX, 1>(t.status, tid, int32_t(tile) - 1, g * kGroupTiles, excl, done,
-                             gave_up, ctrl, timeout_ns, tile, t.trace);
-        stamp(t.trace, 14);
-        // earlier groups, 8 per round trip (two 16-byte loads per array)
-        for (int32_t h = g - 1; !done && !gave_up && h >= 0;) {
-          trace_add(t.trace, 11, 1);
-          const int32_t b0 = h >> 2;
-          uint4 vi[2], va[2];
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const bool in = b0 - k >= 0;
-            const size_t off = (size_t(b0 - k) * RADIX + tid) * 4;
-            vi[k] = in ? __ldcg(reinterpret_cast<const uint4*>(t.ginc + off)) : make_uint4(0, 0, 0, 0);
-            va[k] = in ? __ldcg(reinterpret_cast<const uint4*>(t.gagg + off)) : make_uint4(0, 0, 0, 0);
-          }
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int32_t hh = 4 * b0 + 3 - q;  // groups of this window, nearest first
-            if (hh > h || hh < 0 || done || gave_up) continue;
-            const int c = 3 - (q & 3);
-            const uint4& vq = vi[q >> 2];
-            const uint4& aq = va[q >> 2];
-            const uint32_t wi = c == 0 ? vq.x : c == 1 ? vq.y : c == 2 ? vq.z : vq.w;
-            uint32_t ag = c == 0 ? aq.x : c == 1 ? aq.y : c == 2 ? aq.z : aq.w;
-            const uint32_t fi = wi & kFlagMask;
-            if (fi == kFlagErr) {
-              gave_up = true;
-            } else if (fi == kFlagInc) {
-              excl += wi & kValueMask;
-              done = true;
-            } else {
-              const uint32_t need = min(uint32_t(kGroupTiles), t.tiles - uint32_t(hh) * kGroupTiles);
-              if ((ag >> 24) < need) {
-                trace_add(t.trace, 13, 1);
-                bool ok = false;
-                ag = wait_group(&t.gagg[lb_index<RADIX>(uint32_t(hh), tid)], need, ctrl,
-                                timeout_ns, tile, &ok);
-                if (!ok) gave_up = true;
-              }
-              if (!gave_up) excl += ag & kGroupCountMask;
-            }
-          }
-          h = 4 * b0 - 5;  // below the lowest group of this window (4*b0 - 4)
-        }
-        // a walk that ran past group 0 without an inclusive prefix has summed
-        // every earlier group completely
-      }
-      if (!t.silent && dbg_ok(lb_index<RADIX>(t.tile0 + tile, tid), t.lb_words, kSiteTileStatus))
-        st_relaxed(&t.status[lb_index<RADIX>(t.tile0 + tile, tid)],
-                   gave_up ? kFlagErr : (kFlagInc | ((excl + my_cnt) & kValueMask)));
-    }
-    if (t.ginc != nullptr && !t.silent &&
-        ((tile + 1) % kGroupTiles == 0 || tile + 1 == t.tiles) &&
-        dbg_ok(lb_index<RADIX>(tile / kGroupTiles, tid), t.g_words, kSiteGroupInc))
-      st_relaxed(&t.ginc[lb_index<RADIX>(tile / kGroupTiles, tid)],
-                 gave_up ? kFlagErr : (kFlagInc | ((excl + my_cnt) & kValueMask)));
-    // every key of digit tid goes to [pass offset + excl, ... + its count):
-    // checked here once, so that the scatters below need no per-element
-    // bound.  The past-the-end sentinels of a partial tile were counted under
-    // the largest digit; they are never written.
-    const uint32_t base = t.pass_offsets[tid] + excl;
-    const uint32_t real = my_cnt - (uint32_t(tid) == t.mask ? uint32_t(TILE) - tile_len : 0u);
-    if (!gave_up && (base > n || real > n - base)) {
-      report_error(ctrl, kDevIndex, tile);
-      gave_up = true;
-    }
-    if (gave_up) s_misc[1] = 1u;
-    stamp(t.trace, 9);
-    s_gbase[tid] = base - my_start;
-  }
-  __syncthreads();
-  if (s_misc[1]) {
-    // the output of this call is void (ctrl->error says why); let the value
-    // copy land before leaving
-    if constexpr (VB > 0) {
-      bool ok = mbar_wait_bounded(&s_bar[1], parity, ctrl, timeout_ns, tile);
-      if (!ok) mbar_wait_bounded(&s_bar[1], parity, ctrl, timeout_ns, tile);
-      __syncthreads();
-    }
-    if constexpr (!PERSIST) {
-      if (tid == 0) {
-        mbar_inval(&s_bar[0]);
-        if constexpr (VB > 0) mbar_inval(&s_bar[1]);
-      }
-    }
-    return false;
-  }
-  stamp(t.trace, 4);
-  // keys only: the key buffer is free (keys are staged in OUT) -- start the next tile
-  if constexpr (PERSIST && VB == 0 && !INPLACE) {
-    if (tid == 0) {
-      const uint32_t nxt = atomicAdd(pf->counter, 1u);
-      s_misc[3] = nxt;
-      s_misc[4] = nxt < pf->tiles ? 1u : 0u;
-    }
-    __syncthreads();
-    if (s_misc[4])
-      stage_keys<K, THREADS, TILE, CG>(smem + S::KIN, t.ksrc, n, s_misc[3], &s_bar[0],
-                                       smem + S::WH, S::ZERO_BYTES);
-  }
-
-  // ---- scatter: consecutive threads take consecutive stage slots, which map
-  // to consecutive output addresses inside each digit run
+  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (t.mirror ? 31 - lane : lane));
+  uint32_t* wh = s_wh + warp * RADIX;
+  // a tile's keys are its first tile_len slots; the rest draw nothing
+  const uint32_t lim = tile_len - min(slot0, tile_len);  // item j is a key if j * 32 < lim
   const bool full = tile_len == uint32_t(TILE);
-  uint32_t gidx[VB > 0 ? ITEMS : 1];  // the values' destinations
-  // XO: the last pass that moves data writes the keys back untransformed
-  // debug builds, test-only: every destination of this tile past the array,
-  // so that the bounds checks must drop the stores (0 otherwise)
-  const uint32_t dbg_push = (kDebugChecks && t.dbg_bad) ? n : 0u;
-  auto scatter_keys = [&](auto XO) {
-    auto out = [&](K k) {
-      if constexpr (decltype(XO)::value) return xf_inv(k, t.xf);
-      else return k;
-    };
-    if (full) {
+  // until they are staged: the keys, or (INDEX) their digits, four a word
+  K key[INDEX ? 1 : ITEMS];
+  uint32_t dig[INDEX ? (ITEMS + 3) / 4 : 1];
+  // in batches, so that a batch's loads, atomics and stores each go back to
+  // back: one after another per item they would wait on one another
+  constexpr int BATCH = ITEMS < 9 ? ITEMS : 9;
+  auto count = [&](auto FULL) __attribute__((always_inline)) {
+    const uint32_t shift = t.shift, mask = t.mask;
+    const bool xin = t.xin;
+    const KeyXf<K> xf = t.xf;
 #pragma unroll
-      for (int s = 0; s < ITEMS; ++s) {
-        const uint32_t i = uint32_t(s * THREADS + tid);
-        const K k = s_out[i];
-        const uint32_t g = s_gbase[digit_of(k, t.shift, t.mask)] + i + dbg_push;
-        if (dbg_ok(g, n, kSiteKeyScatter)) t.kdst[g] = out(k);
-        if constexpr (VB > 0) gidx[s] = g;
-      }
-    } else {
+    for (int j0 = 0; j0 < ITEMS; j0 += BATCH) {
+      K k[BATCH];
 #pragma unroll
-      for (int s = 0; s < ITEMS; ++s) {
-        const uint32_t i = uint32_t(s * THREADS + tid);
-        if constexpr (VB > 0) gidx[s] = 0u;
-        if (i < tile_len) {
-          const K k = s_out[i];
-          const uint32_t g = s_gbase[digit_of(k, t.shift, t.mask)] + i + dbg_push;
-          if (dbg_ok(g, n, kSiteKeyScatter)) t.kdst[g] = out(k);
-          if constexpr (VB > 0) gidx[s] = g;
+      for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) k[j - j0] = s_kin[slot0 + j * 32];
+      if (xin) {  // the first pass that moves data: from here on the keys are transformed
+#pragma unroll
+        for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+          k[j - j0] = xf_fwd(k[j - j0], xf);
+          if constexpr (INDEX) s_kin[slot0 + j * 32] = k[j - j0];
         }
+      }
+#pragma unroll
+      for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+        const uint32_t d = digit_of(k[j - j0], shift, mask);
+        if (decltype(FULL)::value || uint32_t(j * 32) < lim) atomicAdd(&wh[d], 1u);
+        if constexpr (INDEX) dig[j / 4] = j % 4 ? dig[j / 4] | d << (8 * (j % 4)) : d;
+        else key[j] = k[j - j0];
       }
     }
   };
-  if (t.xout)
-    scatter_keys(std::true_type{});
+  if (full)
+    count(std::true_type{});
   else
-    scatter_keys(std::false_type{});
-  // in place: the key buffer is free once every staged key has left -- start the next tile
-  if constexpr (PERSIST && INPLACE) {
-    __syncthreads();
-    if (tid == 0) {
-      const uint32_t nxt = atomicAdd(pf->counter, 1u);
-      s_misc[3] = nxt;
-      s_misc[4] = nxt < pf->tiles ? 1u : 0u;
-    }
-    __syncthreads();
-    if (s_misc[4])
-      stage_keys<K, THREADS, TILE, CG>(smem + S::KIN, t.ksrc, n, s_misc[3], &s_bar[0],
-                                       smem + S::WH, S::ZERO_BYTES);
-  }
-  stamp(t.trace, 5);
-  bool ok = true;
-  if constexpr (VB > 0) {
-    ok = mbar_wait_bounded(&s_bar[1], parity, ctrl, timeout_ns, tile);
-    if (!ok) ok = mbar_wait_bounded(&s_bar[1], parity, ctrl, timeout_ns, tile);
-    // every key has left the stage and the value edges are in place
-    if (!__syncthreads_or(!ok)) {
-      V* s_vout = reinterpret_cast<V*>(smem + S::OUT);
+    count(std::false_type{});
+  if (INDEX && tid == 0) s_misc[5] = s_misc[6] = 0u;  // the check's sums, one a round
+  __syncthreads();
+  stamp(trace(), 2);
+
+  // ---- 2. per digit: the tile's count, published; then the exclusive prefix
+  // over the warps from the digit's first slot in the tile
+  typename std::conditional<FLAT, FlatLookBack<K, VB, RADIX>, TreeLookBack<K, VB, RADIX>>::type lb;
+  uint32_t my_cnt = 0u, off0 = 0u;
+  uint32_t c[WARPS];
+  if (tid < RADIX) {
 #pragma unroll
-      for (int j = 0; j < ITEMS; ++j) s_vout[pos[j]] = s_vin[slot0 + j * UNIT];
-      if constexpr (PERSIST) {
-        // the key buffer is free (values are staged in OUT): start the next tile
-        if (tid == 0) {
-          const uint32_t nxt = atomicAdd(pf->counter, 1u);
-          s_misc[3] = nxt;
-          s_misc[4] = nxt < pf->tiles ? 1u : 0u;
+    for (int w = 0; w < WARPS; ++w) {
+      c[w] = s_wh[w * RADIX + tid];
+      my_cnt += c[w];
+    }
+    if (!silent) {
+      if constexpr (FLAT) {
+        if (dbg_ok(lb_index<RADIX>(t.tile0 + tile, tid), t.lb_words, kSiteTileStatus))
+          st_relaxed(&t.status[lb_index<RADIX>(t.tile0 + tile, tid)],
+                     (tile == 0u ? kFlagInc : kFlagAgg) | my_cnt);
+      } else {
+        const size_t at = size_t(tile) * RADIX + tid;
+        if (dbg_ok(at, t.lb_words, kSiteTileStatus))
+          st_relaxed_u16(reinterpret_cast<uint16_t*>(t.status) + at,
+                         uint16_t(kTilePublished | my_cnt));
+        const size_t g = size_t(tile / kGroupTiles) * RADIX + tid;
+        if (dbg_ok(g, t.g_words, kSiteGroupAgg)) atomicAdd(&t.gagg[g], my_cnt | kGroupOne);
+        const size_t s = size_t(tile / kSuperTiles) * RADIX + tid;
+        if (dbg_ok(s, t.s_words, kSiteGroupAgg)) atomicAdd(&t.sagg[s], my_cnt | kGroupOne);
+      }
+    }
+    off0 = t.pass_offsets[tid];
+  }
+  const uint32_t inc = warp_inclusive_scan(my_cnt, lane);
+  if (lane == 31) s_tot[warp] = inc;
+  __syncthreads();
+  const uint32_t my_start =
+      __reduce_add_sync(kFull, lane < WARPS && lane < warp ? s_tot[lane] : 0u) + inc - my_cnt;
+  if (tid < RADIX) {
+    uint32_t run = my_start;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+      s_wh[w * RADIX + tid] = run;
+      run += c[w];
+    }
+    lb.start(t, tile);
+  }
+  __syncthreads();
+  stamp(trace(), 3);
+
+  // ---- 3. stage, the look-back in between
+  K* s_out = reinterpret_cast<K*>(smem + S::OUT);
+  uint16_t* s_idx = reinterpret_cast<uint16_t*>(smem + S::OUT);
+  constexpr int LB_AT = ((ITEMS + BATCH - 1) / BATCH - 1) / 2;
+  auto stage = [&](auto FULL) __attribute__((always_inline)) {
+    [[maybe_unused]] const uint32_t shift = t.shift, mask = t.mask;
+#pragma unroll
+    for (int j0 = 0; j0 < ITEMS; j0 += BATCH) {
+      uint32_t p[BATCH];
+#pragma unroll
+      for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+        uint32_t d;
+        if constexpr (INDEX) d = dig[j / 4] >> (8 * (j % 4)) & 0xffu;
+        else d = digit_of(key[j], shift, mask);
+        p[j - j0] = 0u;
+        if (decltype(FULL)::value || uint32_t(j * 32) < lim) p[j - j0] = atomicAdd(&wh[d], 1u);
+      }
+#pragma unroll
+      for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+        if (decltype(FULL)::value || uint32_t(j * 32) < lim) {
+          if constexpr (INDEX) s_idx[p[j - j0]] = uint16_t(slot0 + j * 32);
+          else s_out[p[j - j0]] = key[j];
+        }
+      }
+      // half-way, so that the tiles just before this one, which publish at
+      // about the same time, mostly have
+      if (j0 / BATCH == LB_AT && tid < RADIX) lb.issue(t, tid);
+    }
+  };
+  if (full)
+    stage(std::true_type{});
+  else
+    stage(std::false_type{});
+  // past the end, and one more: what the scatter may read, and ascends to
+  for (uint32_t i = tile_len + tid; i <= uint32_t(TILE); i += THREADS) {
+    if constexpr (INDEX) s_idx[i] = uint16_t(tile_len - 1u);
+    else s_out[i] = ~K(0);
+  }
+  stamp(trace(), 8);
+  if constexpr (PERSIST) {
+    if (tid == 0) s_misc[3] = atomicAdd(pf->counter, 1u);
+  }
+
+  // ---- 4. the rest of the look-back
+  bool gave_up = false;
+  if (tid < RADIX) {
+    lb.consume(trace());
+    gave_up = !lb.finish(t, tid, ctrl, timeout_ns, tile, trace());
+    const uint32_t excl = lb.excl;
+    if (!gave_up && !silent) {
+      const uint32_t pub = kFlagInc | ((excl + my_cnt) & kValueMask);
+      if constexpr (FLAT) {
+        if (tile > 0u && dbg_ok(lb_index<RADIX>(t.tile0 + tile, tid), t.lb_words, kSiteTileStatus))
+          st_relaxed(&t.status[lb_index<RADIX>(t.tile0 + tile, tid)], pub);
+      } else {
+        const size_t s = size_t(tile / kSuperTiles) * RADIX + tid;
+        if ((tile + 1) % kSuperTiles == 0 && dbg_ok(s, t.s_words, kSiteGroupInc))
+          st_relaxed(&t.sinc[s], pub);
+      }
+    }
+    // every key of digit tid goes to [pass offset + excl, ... + its count):
+    // checked here once, so that the scatters below need no per-element
+    // bound.
+    const uint32_t base = off0 + excl;
+    if (!gave_up && (base > t.n || my_cnt > t.n - base)) {
+      report_error(ctrl, kDevIndex, tile);
+      gave_up = true;
+    }
+    stamp(trace(), 9);
+    s_gbase[tid] = base - my_start;
+  }
+  if constexpr (VB > 0) {
+    if (!mbar_wait(&s_bar[1], parity, ctrl, timeout_ns, tile)) gave_up = true;
+  }
+  // the output of a call that gave up is void (ctrl->error says why)
+  if (__syncthreads_or(gave_up)) return leave(false, true);
+  stamp(trace(), 4);
+  if constexpr (PERSIST) {
+    *next = s_misc[3];
+    if (*next < pf->tiles) {
+      // staged keys: their buffer and the counters are free -- start the next tile
+      if constexpr (!INDEX) stage_tile<S, K, VB, THREADS, CG>(smem, *next);
+    }
+  }
+
+  // consecutive threads take consecutive stage slots, which map to
+  // consecutive output addresses inside each digit run; first the keys
+  const V* s_vin = nullptr;
+  if constexpr (VB > 0) s_vin = Stage<V>(t.vsrc + tile_base, tile_len).at(smem + S::VIN);
+  // the bits that ascend over a stage of keys
+  auto upto_bits = [&]() { return K((K(t.mask) << t.shift) | ((K(1) << t.shift) - K(1))); };
+  // one instance for full and partial tiles, with or without the last pass's
+  // inverse transform: of four, the compiler kept the common loads in
+  // registers across the branch and spilled
+  uint32_t bad = 0u;
+  uint32_t dst[VB > 0 ? ITEMS : 1];  // the values' destinations
+  {
+    const uint32_t shift = t.shift, mask = t.mask;
+    const bool xout = t.xout;
+    [[maybe_unused]] const uint32_t n = t.n;
+    [[maybe_unused]] const K upto = upto_bits();
+    K* kdst = t.kdst;
+    // debug builds, test-only: every destination of this tile past the array,
+    // so that the bounds checks must drop the stores (0 otherwise)
+    const uint32_t dbg_push = (kDebugChecks && int(tile) == t.bad_tile) ? n : 0u;
+#pragma unroll
+    for (int s0 = 0; s0 < ITEMS; s0 += BATCH) {
+      K k[BATCH];
+      uint32_t g[BATCH];
+      [[maybe_unused]] uint32_t at[BATCH];
+#pragma unroll
+      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+        const uint32_t i = uint32_t(s * THREADS + tid);
+        if constexpr (INDEX) {
+          at[s - s0] = s_idx[i];
+          bad += at[s - s0] > uint32_t(s_idx[i + 1]) ? 1u : 0u;
+        } else {
+          k[s - s0] = s_out[i];
+          bad |= (k[s - s0] & upto) > (s_out[i + 1] & upto) ? 1u : 0u;
+        }
+      }
+#pragma unroll
+      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+        if constexpr (INDEX) k[s - s0] = s_kin[at[s - s0]];
+        g[s - s0] = s_gbase[digit_of(k[s - s0], shift, mask)] + uint32_t(s * THREADS + tid) +
+                    dbg_push;
+      }
+      if (xout) {  // the last pass that moves data writes the keys back untransformed
+        const KeyXf<K> xf = t.xf;
+#pragma unroll
+        for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) k[s - s0] = xf_inv(k[s - s0], xf);
+      }
+#pragma unroll
+      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+        const bool in = uint32_t(s * THREADS + tid) < tile_len;
+        if (in && dbg_ok(g[s - s0], n, kSiteKeyScatter)) kdst[g[s - s0]] = k[s - s0];
+        if constexpr (VB > 0) dst[s] = g[s - s0];
+      }
+    }
+  }
+  // the sum of a check over the CTA (a barrier): 0 when the stage is in order
+  auto check = [&](uint32_t bad, int which) {
+    if constexpr (INDEX) {
+      // descents at the starts of digit runs are due: take them off the count
+      if (tid < RADIX && my_cnt > 0u && my_start > 0u &&
+          s_idx[my_start - 1] > s_idx[my_start])
+        bad -= 1u;
+      bad = __reduce_add_sync(kFull, bad);
+      if (lane == 0 && bad != 0u) atomicAdd(&s_misc[which], bad);
+      __syncthreads();
+      return s_misc[which];
+    } else {
+      return uint32_t(__syncthreads_or(bad != 0u));
+    }
+  };
+  bool ok = check(bad, 5) == 0u;
+  const bool repaired = !ok;
+  if (!ok) {
+    // out of turn: at most 31 places off, so 32 rounds of odd-even
+    // transposition put every digit run in order; then the scatter again
+    auto wrong = [&](uint32_t i) {  // stage slots i and i + 1 are out of order
+      if constexpr (INDEX) {
+        const uint32_t a = s_idx[i], b = s_idx[i + 1];
+        return a > b && digit_of(s_kin[a], t.shift, t.mask) == digit_of(s_kin[b], t.shift, t.mask);
+      } else {
+        return (s_out[i] & upto_bits()) > (s_out[i + 1] & upto_bits());
+      }
+    };
+    for (int r = 0; r < 32; ++r) {
+      for (uint32_t i = uint32_t(2 * tid + (r & 1)); i + 1u < tile_len; i += 2 * THREADS) {
+        if (!wrong(i)) continue;
+        if constexpr (INDEX) {
+          const uint16_t a = s_idx[i];
+          s_idx[i] = s_idx[i + 1];
+          s_idx[i + 1] = a;
+        } else {
+          const K a = s_out[i];
+          s_out[i] = s_out[i + 1];
+          s_out[i + 1] = a;
         }
       }
       __syncthreads();
-      if constexpr (PERSIST) {
-        if (s_misc[4])
-          stage_keys<K, THREADS, TILE, CG>(smem + S::KIN, t.ksrc, n, s_misc[3], &s_bar[0],
-                                           smem + S::WH, S::ZERO_BYTES);
-      }
-      if (full) {
-#pragma unroll
-        for (int s = 0; s < ITEMS; ++s)
-          if (dbg_ok(gidx[s], n, kSiteValScatter)) t.vdst[gidx[s]] = s_vout[s * THREADS + tid];
+    }
+    bad = 0u;
+    for (uint32_t i = tid; i < tile_len; i += THREADS) {
+      K k;
+      uint32_t at = 0u;
+      if constexpr (INDEX) {
+        at = s_idx[i];
+        bad += at > uint32_t(s_idx[i + 1]) ? 1u : 0u;
+        k = s_kin[at];
       } else {
-#pragma unroll
-        for (int s = 0; s < ITEMS; ++s) {
-          const uint32_t i = uint32_t(s * THREADS + tid);
-          if (i < tile_len && dbg_ok(gidx[s], n, kSiteValScatter)) t.vdst[gidx[s]] = s_vout[i];
-        }
+        k = s_out[i];
+        bad |= wrong(i) && i + 1u < tile_len ? 1u : 0u;
       }
-    } else {
-      ok = false;
+      const uint32_t g = s_gbase[digit_of(k, t.shift, t.mask)] + i;
+      if (dbg_ok(g, t.n, kSiteKeyScatter)) t.kdst[g] = t.xout ? xf_inv(k, t.xf) : k;
+      if constexpr (VB > 0)
+        if (dbg_ok(g, t.n, kSiteValScatter)) t.vdst[g] = s_vin[at];
+    }
+    ok = check(bad, 6) == 0u;
+  }
+  if (!ok && tid == 0) report_error(ctrl, kDevIndex, tile);
+  // INDEX: every key has left the buffer -- start the next tile, under the
+  // scatter of the values
+  if constexpr (PERSIST && INDEX) {
+    if (ok && *next < pf->tiles) stage_tile<S, K, VB, THREADS, CG>(smem, *next);
+  }
+  if constexpr (VB > 0) {
+    if (!repaired) {  // (a repaired tile's values went with its keys)
+      V* vdst = t.vdst;
+      [[maybe_unused]] const uint32_t n = t.n;
+#pragma unroll
+      for (int s = 0; s < ITEMS; ++s) {
+        const uint32_t i = uint32_t(s * THREADS + tid);
+        const V v = s_vin[s_idx[i]];
+        if (i < tile_len && dbg_ok(dst[s], n, kSiteValScatter)) vdst[dst[s]] = v;
+      }
     }
   }
-  if constexpr (!PERSIST) {
-    if (tid == 0) {
-      mbar_inval(&s_bar[0]);
-      if constexpr (VB > 0) mbar_inval(&s_bar[1]);
+  stamp(trace(), 6);
+  if (!ok) {
+    // (keys, resident: the next tile's copy is in flight and must land first)
+    if constexpr (PERSIST && !INDEX) {
+      if (*next < pf->tiles) mbar_wait(&s_bar[0], parity ^ 1u, ctrl, timeout_ns, tile);
+      __syncthreads();
     }
   }
-  stamp(t.trace, 6);
-  return ok;
+  return leave(ok, true);
+}
+
+// The operands of a whole-array pass (one thread; a barrier follows).
+template <class K, int VB, int RADIX>
+__device__ __forceinline__ void pass_args(
+    TileArgs<K, VB>* t, K* k0, K* k1, ValT<VB>* v0, ValT<VB>* v1, uint32_t n, int pass,
+    uint32_t exec, uint32_t shift, uint32_t mask, const uint32_t* pass_offsets,
+    const LookBackWords& lbw, uint32_t tiles, const KeyXf<K>& xf, const Knobs& knobs) {
+  const bool from_alt = (__popc(exec & ((1u << pass) - 1u)) & 1) != 0;
+  t->ksrc = from_alt ? k1 : k0;
+  t->kdst = from_alt ? k0 : k1;
+  t->vsrc = from_alt ? v1 : v0;
+  t->vdst = from_alt ? v0 : v1;
+  t->pass_offsets = pass_offsets;
+  t->status = lbw.status;
+  t->gagg = lbw.gagg;
+  t->sagg = lbw.sagg;
+  t->sinc = lbw.sinc;
+  t->lb_words = uint64_t(tiles) * RADIX;
+  t->g_words = uint64_t((tiles + kGroupTiles - 1) / kGroupTiles) * RADIX;
+  t->s_words = uint64_t((tiles + kSuperTiles - 1) / kSuperTiles) * RADIX;
+  t->xf = xf;
+  t->n = n;
+  t->shift = shift;
+  t->mask = mask;
+  t->tile0 = 0u;
+  t->tiles = tiles;
+  t->xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
+  t->xout = xf.on && pass == 31 - __clz(exec);
+  t->mirror = knobs.mirror != 0;
+  t->drop_tile = pass == knobs.drop_pass ? knobs.drop_tile : -1;
+  t->bad_tile = kDebugChecks && pass == 0 ? knobs.dbg_bad_tile : -1;
+  t->trace = pass == knobs.trace_pass ? knobs.trace : nullptr;
+  t->trace_tiles = knobs.trace_tiles;
 }
 
 // One digit pass, one tile per CTA.  The grid has one CTA per tile; tile ids
 // come from an atomic counter so that a tile's predecessors have always
 // started before it (forward progress of the look-back).
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB, int UNIT = 32,
-          bool INPLACE = false>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB, bool INDEX>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_onesweep(K* __restrict__ k0, K* __restrict__ k1, ValT<VB>* __restrict__ v0,
                ValT<VB>* __restrict__ v1, uint32_t n, int pass, uint32_t shift, uint32_t mask,
-               const uint32_t* __restrict__ pass_offsets, uint32_t* __restrict__ status,
-               uint32_t* __restrict__ gagg, uint32_t* __restrict__ ginc, uint32_t tiles,
+               const uint32_t* __restrict__ pass_offsets, LookBackWords lbw, uint32_t tiles,
                Ctrl* __restrict__ ctrl, Knobs knobs, KeyXf<K> xf, bool early_dependents) {
-  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, UNIT, INPLACE>;
+  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + S::MISC);
   pdl_wait();  // the kernel before (upsweep or previous pass) is complete
@@ -1119,42 +1318,17 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
   const uint32_t exec = ctrl->exec_mask;
   if (!((exec >> pass) & 1u)) return;  // every key has the same digit: nothing moves
-  const bool from_alt = (__popc(exec & ((1u << pass) - 1u)) & 1) != 0;
   if (threadIdx.x == 0) {
     s_misc[0] = atomicAdd(&ctrl->tile_counter[pass], 1u);
     s_misc[2] = ld_relaxed(&ctrl->error);  // an earlier pass of this call gave up
     if (s_misc[0] == 0u) ctrl->t_pass[pass][0] = stat_now(ctrl);
+    pass_args<K, VB, S::RADIX>(reinterpret_cast<TileArgs<K, VB>*>(smem + S::ARGS), k0, k1, v0, v1,
+                               n, pass, exec, shift, mask, pass_offsets, lbw, tiles, xf, knobs);
   }
   __syncthreads();
   if (s_misc[2] != 0u) return;  // CTA-uniform
-  TileArgs<K, VB> t;
-  t.ksrc = from_alt ? k1 : k0;
-  t.kdst = from_alt ? k0 : k1;
-  t.vsrc = from_alt ? v1 : v0;
-  t.vdst = from_alt ? v0 : v1;
-  t.n = n;
-  t.tile = s_misc[0];
-  t.shift = shift;
-  t.mask = mask;
-  t.pass_offsets = pass_offsets;
-  t.status = status;
-  t.tile0 = 0u;
-  t.gagg = gagg;
-  t.ginc = ginc;
-  t.tiles = tiles;
-  t.lb_words = uint64_t((tiles + 3u) / 4u * 4u) * S::RADIX;
-  t.g_words = uint64_t((tiles + kGroupTiles - 1) / kGroupTiles + 3u) / 4u * 4u * S::RADIX;
-  t.silent = (int(t.tile) == knobs.drop_tile) && (pass == knobs.drop_pass);
-  t.dbg_bad = kDebugChecks && int(t.tile) == knobs.dbg_bad_tile && pass == 0;
-  t.lb_small = knobs.lb_small != 0;
-  t.trace = (knobs.trace != nullptr && pass == knobs.trace_pass && t.tile < knobs.trace_tiles)
-                ? knobs.trace + size_t(t.tile) * 16
-                : nullptr;
-  t.xf = xf;
-  t.xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
-  t.xout = xf.on && pass == 31 - __clz(exec);
-  onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, false, false, UNIT, INPLACE>(
-      t, ctrl, knobs.timeout_ns, smem);
+  onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, false>(s_misc[0], ctrl, knobs.timeout_ns,
+                                                                smem);
   __syncthreads();
   if (threadIdx.x == 0) atomicMax(&ctrl->t_pass[pass][1], stat_now(ctrl));
 }
@@ -1164,16 +1338,14 @@ __global__ void __launch_bounds__(THREADS, MINB)
 // loading its next tile while it finishes the current one.  Tile ids are
 // still taken in order by running CTAs, so the look-back keeps making
 // progress: the lowest unfinished tile is always being worked on.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB, int UNIT = 32,
-          bool INPLACE = false>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB, bool INDEX>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_onesweep_persist(K* __restrict__ k0, K* __restrict__ k1, ValT<VB>* __restrict__ v0,
                        ValT<VB>* __restrict__ v1, uint32_t n, int pass, uint32_t shift,
                        uint32_t mask, const uint32_t* __restrict__ pass_offsets,
-                       uint32_t* __restrict__ status, uint32_t* __restrict__ gagg,
-                       uint32_t* __restrict__ ginc, uint32_t tiles, Ctrl* __restrict__ ctrl,
+                       LookBackWords lbw, uint32_t tiles, Ctrl* __restrict__ ctrl,
                        Knobs knobs, KeyXf<K> xf, bool early_dependents) {
-  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, UNIT, INPLACE>;
+  using S = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + S::MISC);
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + S::MBAR);
@@ -1182,7 +1354,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
   const uint32_t exec = ctrl->exec_mask;
   if (!((exec >> pass) & 1u)) return;  // every key has the same digit: nothing moves
-  const bool from_alt = (__popc(exec & ((1u << pass) - 1u)) & 1) != 0;
   Prefetch pf{&ctrl->tile_counter[pass], tiles};
   if (threadIdx.x == 0) {
     mbar_init(&s_bar[0]);
@@ -1190,60 +1361,19 @@ __global__ void __launch_bounds__(THREADS, MINB)
     s_misc[3] = atomicAdd(pf.counter, 1u);
     s_misc[2] = ld_relaxed(&ctrl->error);  // an earlier pass of this call gave up
     if (s_misc[3] == 0u) ctrl->t_pass[pass][0] = stat_now(ctrl);
+    pass_args<K, VB, S::RADIX>(reinterpret_cast<TileArgs<K, VB>*>(smem + S::ARGS), k0, k1, v0, v1,
+                               n, pass, exec, shift, mask, pass_offsets, lbw, tiles, xf, knobs);
   }
   __syncthreads();
-  TileArgs<K, VB> t;
-  t.ksrc = from_alt ? k1 : k0;
-  t.kdst = from_alt ? k0 : k1;
-  t.vsrc = from_alt ? v1 : v0;
-  t.vdst = from_alt ? v0 : v1;
-  t.n = n;
-  t.shift = shift;
-  t.mask = mask;
-  t.pass_offsets = pass_offsets;
-  t.status = status;
-  t.tile0 = 0u;
-  t.gagg = gagg;
-  t.ginc = ginc;
-  t.tiles = tiles;
-  t.lb_words = uint64_t((tiles + 3u) / 4u * 4u) * S::RADIX;
-  t.g_words = uint64_t((tiles + kGroupTiles - 1) / kGroupTiles + 3u) / 4u * 4u * S::RADIX;
-  t.lb_small = knobs.lb_small != 0;
-  t.xf = xf;
-  t.xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
-  t.xout = xf.on && pass == 31 - __clz(exec);
-  uint32_t tile = s_misc[3];
-  if (tile < tiles && s_misc[2] == 0u)
-    stage_keys<K, THREADS, S::TILE, false>(smem + S::KIN, t.ksrc, n, tile, &s_bar[0],
-                                           smem + S::WH, S::ZERO_BYTES);
-  else
-    tile = tiles;  // nothing to do
-  if (threadIdx.x == 0) s_misc[4] = 0u;
-  __syncthreads();
+  uint32_t tile = s_misc[2] == 0u ? s_misc[3] : tiles;
+  if (tile < tiles) stage_tile<S, K, VB, THREADS, false>(smem, tile);
   for (uint32_t it = 0; tile < tiles; ++it) {
-    t.tile = tile;
-    t.silent = (int(tile) == knobs.drop_tile) && (pass == knobs.drop_pass);
-    t.dbg_bad = kDebugChecks && int(tile) == knobs.dbg_bad_tile && pass == 0;
-    t.trace = (knobs.trace != nullptr && pass == knobs.trace_pass && tile < knobs.trace_tiles)
-                  ? knobs.trace + size_t(tile) * 16
-                  : nullptr;
-    const bool ok = onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, false, true, UNIT, INPLACE>(
-        t, ctrl, knobs.timeout_ns, smem, it & 1u, &pf);
-    __syncthreads();
-    const bool next = s_misc[4] != 0u;
-    const uint32_t next_tile = s_misc[3];
-    __syncthreads();  // every thread has read the next tile before it is cleared
-    if (threadIdx.x == 0) s_misc[4] = 0u;
-    if (!ok) {
-      // a bounded wait gave up: let the next tile's key copy land, then stop
-      if (next) {
-        bool done = mbar_wait_bounded(&s_bar[0], (it + 1u) & 1u, ctrl, knobs.timeout_ns, tile);
-        if (!done) mbar_wait_bounded(&s_bar[0], (it + 1u) & 1u, ctrl, knobs.timeout_ns, tile);
-        __syncthreads();
-      }
+    uint32_t next = tiles;
+    // a tile that gives up has taken no next one, or not started to load it
+    if (!onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, false, true>(
+            tile, ctrl, knobs.timeout_ns, smem, it & 1u, &pf, &next))
       break;
-    }
-    tile = next ? next_tile : tiles;
+    tile = next;
   }
   __syncthreads();
   if (threadIdx.x == 0) {

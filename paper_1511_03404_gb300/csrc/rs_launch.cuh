@@ -13,17 +13,32 @@
 
 namespace rs {
 
+// Whether a sort's tiles stage the keys themselves (whole keys, no values)
+// or their slots.
+template <class K, int VB>
+bool stages_keys(int begin_bit, int end_bit) {
+  return VB == 0 && begin_bit == 0 && end_bit == 8 * int(sizeof(K));
+}
+
 // PERSIST: the passes run as k_onesweep_persist on a grid of SMs x resident
-// CTAs instead of one CTA per tile.  UNIT: lanes per ranking unit (32: warps,
-// 16: half warps).  INPLACE: keys only, staged in the key buffer itself.
-template <class K, int VB, int R, int THREADS, int ITEMS, int MINB, bool PERSIST = false,
-          int UNIT = 32, bool INPLACE = false>
+// CTAs instead of one CTA per tile.
+template <class K, int VB, int R, int THREADS, int ITEMS, int MINB, bool PERSIST = false>
 struct OnesweepSort {
   static constexpr int RADIX = 1 << R;
   static constexpr int TILE = THREADS * ITEMS;
   static constexpr int UP_THREADS = 1024;
   static constexpr int MAXP = (8 * int(sizeof(K)) + R - 1) / R;
-  using S = OnesweepSmem<K, VB, R, THREADS, ITEMS, UNIT, INPLACE>;
+  template <bool INDEX>
+  using Smem = OnesweepSmem<K, VB, R, THREADS, ITEMS, INDEX>;
+
+  // the kernel this variant launches
+  template <bool INDEX>
+  static auto kernel() {
+    if constexpr (PERSIST)
+      return &k_onesweep_persist<K, VB, R, THREADS, ITEMS, MINB, INDEX>;
+    else
+      return &k_onesweep<K, VB, R, THREADS, ITEMS, MINB, INDEX>;
+  }
 
   static size_t tiles(uint32_t n) { return (size_t(n) + TILE - 1) / TILE; }
 
@@ -70,13 +85,15 @@ struct OnesweepSort {
     const size_t nt = tiles(a.n);
     const Layout L = onesweep_layout(passes, R, nt);
     using V = ValT<VB>;
-    auto kern = [] {  // instantiate only the kernel this variant launches
-      if constexpr (PERSIST)
-        return &k_onesweep_persist<K, VB, R, THREADS, ITEMS, MINB, UNIT, INPLACE>;
-      else
-        return &k_onesweep<K, VB, R, THREADS, ITEMS, MINB, UNIT, INPLACE>;
-    }();
-    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, S::BYTES);
+    auto kern = kernel<true>();
+    int smem = Smem<true>::BYTES;
+    if constexpr (VB == 0) {
+      if (stages_keys<K, VB>(a.begin_bit, a.end_bit)) {
+        kern = kernel<false>();
+        smem = Smem<false>::BYTES;
+      }
+    }
+    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, smem);
     if (occ <= 0) return cudaErrorInvalidConfiguration;
     // a pass grid that fills the GPU (resident CTAs, or more tiles than CTA
     // slots) is scheduled early, while the kernel before it runs; a one-wave
@@ -108,7 +125,7 @@ struct OnesweepSort {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(grid);
       cfg.blockDim = dim3(THREADS);
-      cfg.dynamicSmemBytes = S::BYTES;
+      cfg.dynamicSmemBytes = smem;
       cfg.stream = a.stream;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -121,9 +138,7 @@ struct OnesweepSort {
           static_cast<V*>(a.vals), static_cast<V*>(a.vals_alt), a.n, p, uint32_t(lo), mask,
           static_cast<const uint32_t*>(reinterpret_cast<const uint32_t*>(ws + L.offsets) +
                                        size_t(p) * RADIX),
-          reinterpret_cast<uint32_t*>(ws + L.status) + size_t(p) * L.tiles * RADIX,
-          reinterpret_cast<uint32_t*>(ws + L.gagg) + size_t(p) * L.groups * RADIX,
-          reinterpret_cast<uint32_t*>(ws + L.ginc) + size_t(p) * L.groups * RADIX, uint32_t(nt),
+          L.words(ws, p), uint32_t(nt),
           ctrl, a.knobs, xf, fills);
       if (e == cudaSuccess) e = cudaGetLastError();
       nvtx_pop();
@@ -160,7 +175,8 @@ struct OnesweepSort {
 template <class K, int VB, int R, int THREADS, int ITEMS, int MINB>
 struct FusedSort {
   using Base = OnesweepSort<K, VB, R, THREADS, ITEMS, MINB>;
-  using F = FusedSmem<K, VB, R, THREADS, ITEMS>;
+  template <bool INDEX>
+  using F = FusedSmem<K, VB, R, THREADS, ITEMS, INDEX>;
   static constexpr int RADIX = 1 << R;
 
   static cudaError_t run(const SortArgs& a, int* in_alt) {
@@ -173,8 +189,15 @@ struct FusedSort {
     cudaError_t e = cudaMemsetAsync(ws, 0, L.memset_bytes, a.stream);
     if (e != cudaSuccess) return e;
     using V = ValT<VB>;
-    auto kern = &k_fused<K, VB, R, THREADS, ITEMS, MINB>;
-    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, F::BYTES);
+    auto kern = &k_fused<K, VB, R, THREADS, ITEMS, MINB, true>;
+    int smem = F<true>::BYTES;
+    if constexpr (VB == 0) {
+      if (stages_keys<K, VB>(a.begin_bit, a.end_bit)) {
+        kern = &k_fused<K, VB, R, THREADS, ITEMS, MINB, false>;
+        smem = F<false>::BYTES;
+      }
+    }
+    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, smem);
     if (occ <= 0) return cudaErrorInvalidConfiguration;
     const unsigned grid =
         unsigned(std::max<size_t>(1, std::min<size_t>(nt, size_t(device_info().sms) * occ)));
@@ -185,22 +208,19 @@ struct FusedSort {
     uint32_t n = a.n;
     int begin = a.begin_bit, end = a.end_bit, np = passes;
     uint32_t* counts = reinterpret_cast<uint32_t*>(ws + L.counts);
-    uint32_t* status = reinterpret_cast<uint32_t*>(ws + L.status);
-    uint32_t* gagg = reinterpret_cast<uint32_t*>(ws + L.gagg);
-    uint32_t* ginc = reinterpret_cast<uint32_t*>(ws + L.ginc);
-    uint32_t tiles = uint32_t(nt), tiles_pad = uint32_t(L.tiles), groups_pad = uint32_t(L.groups);
+    Layout lay = L;
+    uint32_t tiles = uint32_t(nt);
     uint4* zero_base = reinterpret_cast<uint4*>(ws + L.status);
     uint64_t zero_vec4 = L.status_bytes / 16;
     Knobs knobs = a.knobs;
     KeyXf<K> xf = make_key_xf<K>(a.key_kind, a.descending);
     uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 | 2u << 24;
-    void* args[] = {&k0, &k1, &v0, &v1, &n, &begin, &end, &np, &counts, &status, &gagg, &ginc,
-                    &tiles, &tiles_pad, &groups_pad, &zero_base, &zero_vec4, &ctrl, &knobs, &xf,
-                    &shape};
+    void* args[] = {&k0, &k1, &v0, &v1, &n, &begin, &end, &np, &counts, &lay, &tiles, &zero_base,
+                    &zero_vec4, &ctrl, &knobs, &xf, &shape};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = F::BYTES;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;  // every CTA resident: the barriers need it

@@ -14,10 +14,9 @@ namespace {
 
 // MINB: resident CTAs per SM the short-segment kernel is compiled for (its
 // register budget); PASS_MINB: the same for the pass kernel.
-template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int UNIT,
-          int SMALL_ITEMS, int MINB = 4, int PASS_MINB = MINB>
+template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS, int MINB = 4, int PASS_MINB = MINB>
 struct SegSort {
-  using C = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, UNIT, SMALL_ITEMS>;
+  using C = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, SMALL_ITEMS>;
   static constexpr int PLAN_THREADS = 1024;
 
   static SegLayout layout(size_t n, size_t nseg, int passes) {
@@ -50,8 +49,15 @@ struct SegSort {
     const int occ_hist =
         prepare_kernel(reinterpret_cast<const void*>(hist), C::HIST_THREADS, C::HIST_BYTES);
     if (occ_hist <= 0) return cudaErrorInvalidConfiguration;
-    auto kern = &k_seg_persistent<K, VB, R, THREADS, ITEMS, CHUNK_TILES, UNIT, PASS_MINB>;
-    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, C::BYTES);
+    auto kern = &k_seg_persistent<K, VB, R, THREADS, ITEMS, CHUNK_TILES, PASS_MINB, true>;
+    int smem = C::BYTES;
+    if constexpr (VB == 0) {
+      if (begin_bit == 0 && end_bit == 8 * int(sizeof(K))) {  // whole keys: staged themselves
+        kern = &k_seg_persistent<K, VB, R, THREADS, ITEMS, CHUNK_TILES, PASS_MINB, false>;
+        smem = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, SMALL_ITEMS, false>::BYTES;
+      }
+    }
+    const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, smem);
     if (occ <= 0) return cudaErrorInvalidConfiguration;
     SegArgs a;
     a.off = d_off;
@@ -88,7 +94,7 @@ struct SegSort {
                                                  static_cast<V*>(vals_alt), a);
     hist<<<grid_hist, C::HIST_THREADS,
            passes * C::RADIX * C::HIST_SLOTS * 4, s>>>(static_cast<const K*>(keys), a);
-    kern<<<grid, THREADS, C::BYTES, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
+    kern<<<grid, THREADS, smem, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
                                          static_cast<K*>(keys_alt), static_cast<V*>(vals_alt), a);
     e = cudaGetLastError();
     prof_after(s, RS_KERNEL_SEGMENTED,
@@ -99,14 +105,14 @@ struct SegSort {
 
 // u32 pairs: pass tiles of 256 x 45 keys ranked in half-warp units, two CTAs
 // per SM; short segments up to 4096 elements sorted whole by one CTA
-using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 45, 12, 16, 16, 4, 2>;
+using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 41, 12, 16, 4, 2>;
 // u32 keys: 256 x 37 keys in half-warp units, two CTAs per SM; short
 // segments up to 4096
-using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 37, 16, 16, 16, 4, 2>;
+using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 45, 14, 16, 4, 2>;
 // 64-bit keys and pairs: 256 x 23 elements in half-warp units, two CTAs per
 // SM; short segments up to 2048 (pairs: that kernel at three CTAs per SM)
-using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 16, 8, 4, 2>;
-using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 16, 8, 3, 2>;
+using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 8, 4, 2>;
+using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 8, 3, 2>;
 
 bool seg_types(int kb, int vb) { return (kb == 4 || kb == 8) && (vb == 0 || vb == kb); }
 

@@ -206,11 +206,10 @@ struct SegSmallSmem {
   static constexpr int BYTES = VALS + (VB > 0 ? TILE * VB : 0);
 };
 
-// UNIT: lanes per ranking unit of the pass tiles (32 or 16, as for the
-// onesweep pass); SMALL_ITEMS: keys per thread of the short-segment sort,
-// whose tile bounds a short segment.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES, int UNIT = 32,
-          int SMALL_ITEMS = ITEMS>
+// SMALL_ITEMS: keys per thread of the short-segment sort, whose tile bounds a
+// short segment.
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES,
+          int SMALL_ITEMS = ITEMS, bool INDEX = true>
 struct SegKernelCfg {
   static constexpr int RADIX = 1 << RADIX_BITS;
   static constexpr int TILE = THREADS * ITEMS;
@@ -223,7 +222,7 @@ struct SegKernelCfg {
   static constexpr int HIST_BYTES = MAXP * RADIX * HIST_SLOTS * 4;
   // two CTAs per SM while their counters fit (32-bit keys), else one
   static constexpr int HIST_MINB = HIST_BYTES <= 100 * 1024 ? 2 : 1;
-  using OS = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, UNIT>;
+  using OS = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   using SS = SegSmallSmem<K, VB, RADIX_BITS, THREADS, SMALL_ITEMS>;
   static constexpr int MISC = (OS::BYTES + 15) / 16 * 16;  // u32 [8]
   static constexpr int BYTES = MISC + 32;
@@ -505,13 +504,13 @@ __global__ void __launch_bounds__(THREADS, MINB)
   }
 }
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES, int UNIT = 32,
-          int MINB = 4>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES,
+          int MINB, bool INDEX>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_seg_persistent(K* __restrict__ k0, ValT<VB>* __restrict__ v0, K* __restrict__ k1,
                      ValT<VB>* __restrict__ v1, SegArgs a) {
   using V = ValT<VB>;
-  using C = SegKernelCfg<K, VB, RADIX_BITS, THREADS, ITEMS, CHUNK_TILES, UNIT>;
+  using C = SegKernelCfg<K, VB, RADIX_BITS, THREADS, ITEMS, CHUNK_TILES, ITEMS, INDEX>;
   constexpr int RADIX = C::RADIX, TILE = C::TILE;
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + C::MISC);
@@ -556,39 +555,30 @@ __global__ void __launch_bounds__(THREADS, MINB)
       ok = s_misc[3] != 0u;
     }
     if (ok && ((exec >> p) & 1u)) {
-      const bool from_alt = (__popc(exec & ((1u << p) - 1u)) & 1) != 0;
-      TileArgs<K, VB> t;
-      t.ksrc = (from_alt ? k1 : k0) + d.off;
-      t.kdst = (from_alt ? k0 : k1) + d.off;
-      if constexpr (VB > 0) {
-        t.vsrc = (from_alt ? v1 : v0) + d.off;
-        t.vdst = (from_alt ? v0 : v1) + d.off;
-      } else {
-        t.vsrc = nullptr;
-        t.vdst = nullptr;
+      if (tid == 0) {
+        const int lo = a.begin_bit + p * RADIX_BITS;
+        auto* t = reinterpret_cast<TileArgs<K, VB>*>(smem + C::OS::ARGS);
+        K *ka = k0 + d.off, *kb = k1 + d.off;
+        V *va = nullptr, *vb = nullptr;
+        if constexpr (VB > 0) {
+          va = v0 + d.off;
+          vb = v1 + d.off;
+        }
+        // segments are short: a flat walk over tiles, no groups
+        pass_args<K, VB, RADIX>(t, ka, kb, va, vb, d.len, p, exec, uint32_t(lo),
+                                (1u << (min(lo + RADIX_BITS, a.end_bit) - lo)) - 1u,
+                                a.offsets + (size_t(li) * passes + p) * RADIX,
+                                LookBackWords{a.status + size_t(p) * a.tiles_max * RADIX, nullptr,
+                                              nullptr, nullptr},
+                                ntiles, KeyXf<K>{}, a.knobs);
+        t->tile0 = d.tile0;
+        t->lb_words = a.tiles_max * RADIX;
+        t->drop_tile = t->bad_tile = -1;
+        t->trace = nullptr;
       }
-      t.n = d.len;
-      t.tile = gt - d.tile0;
-      const int lo = a.begin_bit + p * RADIX_BITS;
-      t.shift = uint32_t(lo);
-      t.mask = (1u << (min(lo + RADIX_BITS, a.end_bit) - lo)) - 1u;
-      t.pass_offsets = a.offsets + (size_t(li) * passes + p) * RADIX;
-      t.status = a.status + size_t(p) * a.tiles_max * RADIX;
-      t.tile0 = d.tile0;
-      t.gagg = nullptr;  // segments are short: flat walk
-      t.ginc = nullptr;
-      t.tiles = ntiles;
-      t.lb_words = a.tiles_max * RADIX;
-      t.g_words = 0;
-      t.silent = false;
-      t.dbg_bad = false;
-      t.trace = nullptr;
-      t.lb_small = false;
-      t.xf = KeyXf<K>{};
-      t.xin = false;
-      t.xout = false;
-      onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, true, false, UNIT>(
-          t, ctrl, a.knobs.timeout_ns, smem);
+      __syncthreads();
+      onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, true, false, true>(gt - d.tile0, ctrl,
+                                                                    a.knobs.timeout_ns, smem);
     }
     __syncthreads();
     if (tid == 0) {

@@ -1,0 +1,78 @@
+"""The digit passes rank with atomics whose order among equal digits is the
+hardware's, check the order they got and repair it when it is not the input
+order.  Here every warp's lanes take their keys in reverse (a test-only
+knob), so that every repeated digit is out of turn and every tile needs the
+repair; the result must still be the oracle's, bit for bit.  Keys of few
+values make long runs of one digit, partial bit ranges take the slot-indexed
+stage for keys too, and the sizes lie around one tile and around the groups
+of 8 and 64 tiles of the look-back."""
+import numpy as np
+import pytest
+
+import inputs
+import oracle
+
+torch = pytest.importorskip("torch")
+from gpu_util import sort_via_abi  # noqa: E402
+
+from paper_1511_03404_gb300 import rs  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+TYPES = [(np.uint32, False), (np.uint32, True), (np.uint64, False), (np.uint64, True)]
+TYPE_IDS = ["k32", "kv32", "k64", "kv64"]
+
+
+def variants(kb, vb, kinds):
+    out = [rs.rs_variant_info(kb, vb, i) | {"index": i} for i in range(rs.rs_num_variants(kb, vb))]
+    return [v for v in out if v["kind"] in kinds]
+
+
+def check(k, v, what, **kw):
+    gk, gv, _ = sort_via_abi(torch, k, v, **kw)
+    ek, ev = oracle.lsd_sort(k, v, begin_bit=kw.get("begin_bit", 0), end_bit=kw.get("end_bit"))
+    assert np.array_equal(gk, ek), what
+    assert v is None or np.array_equal(gv, ev), what
+
+
+@pytest.fixture
+def mirrored():
+    rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 1))
+    yield
+    rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
+
+
+@pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
+def test_out_of_turn_ranks_are_repaired(dtype, pairs, mirrored):
+    kb = np.dtype(dtype).itemsize
+    for var in variants(kb, kb if pairs else 0, (0, 2, 3)):
+        tile = var["threads"] * var["items"]
+        for n in (tile - 1, tile, 3 * tile + 5):
+            v = inputs.values(dtype, n) if pairs else None
+            for name, k in (("uniform", inputs.keys(dtype, "uniform", n)),
+                            ("few", inputs.keys(dtype, "uniform", n) & dtype(0x0303)),
+                            ("sorted_desc", inputs.keys(dtype, "sorted_desc", n))):
+                check(k, v, (name, n, var), variant=var["index"])
+            check(inputs.keys(dtype, "uniform", n), v, ("bits", n, var), variant=var["index"],
+                  begin_bit=3, end_bit=17)
+
+
+@pytest.mark.parametrize("mirror", [0, 1])
+@pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
+def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
+    kb = np.dtype(dtype).itemsize
+    try:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, mirror))
+        for kind in (0, 2):
+            var = min(variants(kb, kb if pairs else 0, (kind,)),
+                      key=lambda x: x["threads"] * x["items"])
+            tile = var["threads"] * var["items"]
+            for tiles in (7, 8, 9, 63, 64, 65, 72, 129, 200):
+                n = tiles * tile - 3
+                v = inputs.values(dtype, n) if pairs else None
+                check(inputs.keys(dtype, "gaussian", n), v, (n, var), variant=var["index"])
+                if not pairs and not mirror:
+                    check(inputs.keys(dtype, "gaussian", n), v, (n, var, "bits"),
+                          variant=var["index"], begin_bit=0, end_bit=20)
+    finally:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
