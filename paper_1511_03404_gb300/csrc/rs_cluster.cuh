@@ -1,30 +1,29 @@
 // The whole sort inside one thread-block cluster, for arrays up to
-// CL x SLICE elements (SLICE = THREADS x ITEMS per CTA): every digit pass
-// (Sec. 2.6) runs on data held in the cluster's shared memory, with no trip
-// through global memory and no kernel boundary between passes.
+// CL x THREADS x ITEMS elements: every digit pass (Sec. 2.6) runs on data held
+// in the cluster's shared memory, with no trip through global memory and no
+// kernel boundary between passes.
 //
-// CTA c of the cluster owns positions [c * SLICE, (c + 1) * SLICE) of the
-// array.  One pass:
-//   1. each thread takes its ITEMS keys (warp-striped) from the CTA's source
-//      buffer and the warps rank them stably (shared peer masks, per-warp
-//      running counts); per-digit prefixes over the warps give every key's
-//      place among the CTA's keys of its digit, and the CTA's digit counts;
+// CTA c of the cluster owns positions [c * slice, (c + 1) * slice) of the
+// array; the slice follows the length, so that every CTA takes part.  One
+// pass:
+//   1. each warp draws its keys' ranks from its counters (draw_rank); per-digit
+//      prefixes over the warps give every key's place among the CTA's keys of
+//      its digit, and the CTA's digit counts;
 //   2. every CTA stores its digit counts into every CTA's count table
-//      (remote shared-memory stores); after a cluster barrier each CTA reads
-//      its own table: the start of digit d is the count of all smaller
-//      digits, plus the count of digit d in lower-ranked CTAs;
-//   3. the CTA first stages its keys (and values) in digit order in its own
-//      source buffer (its keys are in registers by then), then its threads
-//      take the staged keys in order and store each at its global position,
-//      in the destination buffer of the CTA that owns that position (a
-//      remote shared-memory store): consecutive threads store consecutive
-//      keys of a digit run to consecutive addresses of one CTA, instead of
-//      scattering single keys over the cluster;
+//      (remote shared-memory stores), and stages its keys (and their 16-bit
+//      input positions) in digit order in its own source buffer; after a
+//      cluster barrier each CTA reads its table: the start of digit d is the
+//      count of all smaller digits, plus the count of digit d in lower-ranked
+//      CTAs;
+//   3. the staged keys go, in order, each to its global position, in the
+//      destination buffer of the CTA that owns that position (a remote
+//      shared-memory store): consecutive threads store consecutive keys of a
+//      digit run to consecutive addresses of one CTA;
 //   4. cluster barrier; the destination buffer becomes the next source.
-// Past the end of the array the slices hold the largest key, which sorts
-// after every real key in every pass and is never written out.  The
-// cluster barriers are hardware barriers that every CTA passes the same
-// number of times; no CTA waits on a flag.
+// In the end the values are gathered by the positions that came with the
+// keys.  A result out of order (the draws' order is the hardware's) is sorted
+// again with careful ranks.  The cluster barriers are hardware barriers that
+// every CTA passes the same number of times; no CTA waits on a flag.
 #pragma once
 
 #include "rs_kernels.cuh"
@@ -59,44 +58,60 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, uint64_t v) {
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS>
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint16_t v) {
+  asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
+}
+
+template <class K, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 struct ClusterSmem {
   static constexpr int RADIX = 1 << RADIX_BITS;
   static constexpr int WARPS = THREADS / 32;
-  static constexpr int SLICE = THREADS * ITEMS;
+  static constexpr int SLICE = THREADS * ITEMS;  // the largest
   static constexpr int KB = int(sizeof(K));
-  static constexpr int WH = 0;                              // u32 [WARPS][RADIX] running counts
-  static constexpr int MM = WH + WARPS * RADIX * 4;         // u32 [WARPS][RADIX] peer masks
   static constexpr int MAX_CL = 8;
-  static constexpr int CNT = MM + WARPS * RADIX * 4;        // u32 [MAX_CL][RADIX] every CTA's counts
-  static constexpr int BASE = CNT + MAX_CL * RADIX * 4;     // u32 [RADIX] global digit bases
-  static constexpr int LST = BASE + RADIX * 4;              // u32 [RADIX] digit starts in the CTA
-  static constexpr int TOT = LST + RADIX * 4;               // u32 [32]
-  static constexpr int KEYS = (TOT + 32 * 4 + 15) / 16 * 16;  // K [2][SLICE]
-  static constexpr int VALS = KEYS + 2 * SLICE * KB;        // V [2][SLICE]
-  static constexpr int BYTES = VALS + (VB > 0 ? 2 * SLICE * VB : 0);
+  static constexpr int WH = 0;                             // u32 [2][WARPS][RADIX], by pass parity
+  static constexpr int CNT = WH + 2 * WARPS * RADIX * 4;   // u32 [MAX_CL][RADIX] every CTA's counts
+  static constexpr int BASE = CNT + MAX_CL * RADIX * 4;    // u32 [RADIX] global digit bases
+  static constexpr int TOT = BASE + RADIX * 4;             // u32 [32]
+  static constexpr int EDGE = TOT + 32 * 4;                // first key, its position; u32 [4]
+  static constexpr int FLAGS = EDGE + 16;                  // u32 [MAX_CL] out of order
+  static constexpr int KEYS = FLAGS + MAX_CL * 4;          // K [2][SLICE]
+  static constexpr int IDX = KEYS + 2 * SLICE * KB;        // u16 [2][SLICE]
+  static constexpr int BYTES = IDX + (INDEX ? 2 * SLICE * 2 : 0);
 };
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS>
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_cluster_sort(K* __restrict__ keys, ValT<VB>* __restrict__ vals, uint32_t n, int begin_bit,
-                   int end_bit, Ctrl* ctrl, KeyXf<K> xf) {
+    k_cluster_sort(K* __restrict__ keys, ValT<VB>* __restrict__ vals, uint32_t n, uint32_t slice,
+                   int begin_bit, int end_bit, Ctrl* ctrl, KeyXf<K> xf, bool mirror) {
   using V = ValT<VB>;
-  using S = ClusterSmem<K, VB, RADIX_BITS, THREADS, ITEMS>;
-  constexpr int RADIX = S::RADIX, WARPS = S::WARPS, SLICE = S::SLICE;
+  using S = ClusterSmem<K, RADIX_BITS, THREADS, ITEMS, INDEX>;
+  constexpr int RADIX = S::RADIX, WARPS = S::WARPS;
+  static_assert(INDEX || VB == 0, "values follow their keys' positions");
   extern __shared__ __align__(16) unsigned char smem[];
-  uint32_t* s_wh = reinterpret_cast<uint32_t*>(smem + S::WH);
-  uint32_t* s_mm = reinterpret_cast<uint32_t*>(smem + S::MM);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + S::CNT);
   uint32_t* s_base = reinterpret_cast<uint32_t*>(smem + S::BASE);
-  uint32_t* s_lst = reinterpret_cast<uint32_t*>(smem + S::LST);
   uint32_t* s_tot = reinterpret_cast<uint32_t*>(smem + S::TOT);
-  K* s_k = reinterpret_cast<K*>(smem + S::KEYS);
-  V* s_v = reinterpret_cast<V*>(smem + S::VALS);
+  uint32_t* s_edge = reinterpret_cast<uint32_t*>(smem + S::EDGE);
+  uint32_t* s_flags = reinterpret_cast<uint32_t*>(smem + S::FLAGS);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t rank = cluster_ctarank();
   const uint32_t ncta = gridDim.x;  // the grid is one cluster
   const int passes = (end_bit - begin_bit + RADIX_BITS - 1) / RADIX_BITS;
+  const int items = int(slice / THREADS);
+  const uint32_t base0 = rank * slice;
+  const uint32_t len = n > base0 ? min(slice, n - base0) : 0u;
+  const uint32_t magic = 0xffffffffu / slice + 1u;  // g / slice == mulhi(g, magic): g * slice < 2^32
+  constexpr int BATCH = ITEMS < 4 ? ITEMS : 4;
+  const K looked = (end_bit - begin_bit == 8 * int(sizeof(K)))
+                       ? ~K(0)
+                       : K(((K(1) << (end_bit - begin_bit)) - K(1)) << begin_bit);
   if (ctrl != nullptr && blockIdx.x == 0 && tid == 0) {
     ctrl->error = 0u;
     ctrl->error_info = 0u;
@@ -105,101 +120,192 @@ __global__ void __launch_bounds__(THREADS, 1)
     stat_begin(ctrl, n, uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 |
                             3u << 24);
   }
-
-  // load this CTA's slice (transformed keys; the largest key past the end)
-  const uint32_t base0 = rank * uint32_t(SLICE);
-  for (uint32_t i = tid; i < uint32_t(SLICE); i += THREADS) {
-    const uint32_t g = base0 + i;
-    K k = ~K(0);
-    if (g < n) k = xf.on ? xf_fwd(keys[g], xf) : keys[g];
-    s_k[i] = k;
-    if constexpr (VB > 0) s_v[i] = g < n ? vals[g] : V(0);
+  if constexpr (VB > 0) {  // needed in the end only: into the L2 meanwhile
+    for (uint32_t i = tid * (32 / VB); i < len; i += THREADS * (32 / VB))
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(vals + base0 + i));
   }
-  for (int i = tid; i < WARPS * RADIX; i += THREADS) s_mm[i] = 0u;
-  __syncthreads();
+  // exclusive prefix over the CTA of one value per digit (thread d < RADIX); a
+  // barrier, and the caller separates two calls by another
+  auto scan = [&](uint32_t x) {
+    const uint32_t inc = warp_inclusive_scan(x, lane);
+    if (lane == 31) s_tot[warp] = inc;
+    __syncthreads();
+    return __reduce_add_sync(kFull, lane < RADIX / 32 && lane < warp ? s_tot[lane] : 0u) + inc - x;
+  };
 
-  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + lane);
+  // the first remote store waits until every CTA of the cluster has started
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  bool started = false;
   int src = 0;
-  for (int lo = begin_bit; lo < end_bit; lo += RADIX_BITS) {
-    const uint32_t shift = uint32_t(lo);
-    const uint32_t mask = (1u << (min(lo + RADIX_BITS, end_bit) - lo)) - 1u;
-    K* ks = s_k + src * SLICE;
-    V* vs = s_v + src * SLICE;
-    // ---- 1. local rank
-    for (int i = tid; i < WARPS * RADIX; i += THREADS) s_wh[i] = 0u;
-    __syncthreads();
-    K key[ITEMS];
-    V val[ITEMS];
-    uint32_t dp[ITEMS];
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      key[j] = ks[slot0 + j * 32];
-      if constexpr (VB > 0) val[j] = vs[slot0 + j * 32];
-      dp[j] = digit_of(key[j], shift, mask);
-    }
-    warp_rank_packed<ITEMS>(dp, s_wh + warp * RADIX, s_mm + warp * RADIX, lane);
-    __syncthreads();
-    uint32_t run = 0u;
-    if (tid < RADIX) {
-#pragma unroll
-      for (int w = 0; w < WARPS; ++w) {
-        const uint32_t c = s_wh[w * RADIX + tid];
-        s_wh[w * RADIX + tid] = run;
-        run += c;
-      }
-      // ---- 2. this CTA's counts into every CTA's table
-      for (uint32_t c = 0; c < ncta; ++c)
-        st_cluster(map_shared(s_cnt + rank * RADIX + tid, c), run);
-    }
-    // ---- 3a. the CTA's keys in digit order, staged in its source buffer
-    const uint32_t lstart = block_exclusive_scan<THREADS>(run, s_tot);
-    if (tid < RADIX) s_lst[tid] = lstart;
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t d = dp[j] >> 16;
-      const uint32_t at = s_lst[d] + s_wh[warp * RADIX + d] + (dp[j] & 0xffffu);
-      ks[at] = key[j];
-      if constexpr (VB > 0) vs[at] = val[j];
-    }
-    // every CTA's counts have landed and the stage is complete
-    cluster_sync_all();
-    uint32_t total = 0u, below = 0u;
-    if (tid < RADIX) {
-      for (uint32_t c = 0; c < ncta; ++c) {
-        const uint32_t x = s_cnt[c * RADIX + tid];
-        total += x;
-        if (c < rank) below += x;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    const bool careful = attempt != 0;
+    const uint32_t slot0 = uint32_t(warp * items * 32 + (mirror && !careful ? 31 - lane : lane));
+    src = 0;
+    {
+      K* ks = reinterpret_cast<K*>(smem + S::KEYS);
+      uint16_t* is = reinterpret_cast<uint16_t*>(smem + S::IDX);
+      for (uint32_t i = tid; i < len; i += THREADS) {
+        const K k = keys[base0 + i];
+        ks[i] = xf.on ? xf_fwd(k, xf) : k;
+        if constexpr (INDEX) is[i] = uint16_t(base0 + i);
       }
     }
-    const uint32_t start = block_exclusive_scan<THREADS>(total, s_tot);
-    // staged key i of digit d goes to global position s_base[d] + i
-    if (tid < RADIX) s_base[tid] = start + below - s_lst[tid];
+    for (int i = tid; i < WARPS * RADIX / 4; i += THREADS)
+      reinterpret_cast<uint4*>(smem + S::WH)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    // ---- 3b. remote stores of the staged runs into the owners' destination buffers
-    K* kd = s_k + (src ^ 1) * SLICE;
-    V* vd = s_v + (src ^ 1) * SLICE;
+    int parity = 0;
+    for (int lo = begin_bit; lo < end_bit; lo += RADIX_BITS, parity ^= 1) {
+      const uint32_t shift = uint32_t(lo);
+      const uint32_t mask = (1u << (min(lo + RADIX_BITS, end_bit) - lo)) - 1u;
+      uint32_t* s_wh = reinterpret_cast<uint32_t*>(smem + S::WH) + parity * WARPS * RADIX;
+      uint32_t* wh = s_wh + warp * RADIX;
+      K* ks = reinterpret_cast<K*>(smem + S::KEYS) + src * S::SLICE;
+      uint16_t* is = reinterpret_cast<uint16_t*>(smem + S::IDX) + src * S::SLICE;
+      // ---- 1. draws
+      K key[ITEMS];
+      uint32_t meta[ITEMS];  // rank << 16 | input position
+#pragma unroll
+      for (int j0 = 0; j0 < ITEMS; j0 += BATCH) {
+        if (j0 >= items) break;
+#pragma unroll
+        for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+          const uint32_t at = slot0 + j * 32;
+          const bool in = j < items && at < len;
+          key[j] = in ? ks[at] : K(0);
+          meta[j] = 0u;
+          if constexpr (INDEX) meta[j] = in ? is[at] : 0u;
+        }
+#pragma unroll
+        for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+          const bool in = j < items && slot0 + j * 32 < len;
+          meta[j] |= draw_rank(wh, digit_of(key[j], shift, mask), in, careful, lane) << 16;
+        }
+      }
+      __syncthreads();
+      if (!started) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      started = true;
+      uint32_t c[WARPS], cnt = 0u;
+      if (tid < RADIX) {
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+          c[w] = s_wh[w * RADIX + tid];
+          cnt += c[w];
+        }
+        // ---- 2. this CTA's counts into every CTA's table
+        for (uint32_t q = 0; q < ncta; ++q)
+          st_cluster(map_shared(s_cnt + rank * RADIX + tid, q), cnt);
+      }
+      const uint32_t lstart = scan(cnt);
+      if (tid < RADIX) {
+        uint32_t run = lstart;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+          s_wh[w * RADIX + tid] = run;
+          run += c[w];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int j0 = 0; j0 < ITEMS; j0 += BATCH) {
+        if (j0 >= items) break;
+        uint32_t p[BATCH];
+#pragma unroll
+        for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j)
+          p[j - j0] = wh[digit_of(key[j], shift, mask)] + (meta[j] >> 16);
+#pragma unroll
+        for (int j = j0; j < ITEMS && j < j0 + BATCH; ++j) {
+          if (j < items && slot0 + j * 32 < len) {
+            ks[p[j - j0]] = key[j];
+            if constexpr (INDEX) is[p[j - j0]] = uint16_t(meta[j]);
+          }
+        }
+      }
+      uint4* zero = reinterpret_cast<uint4*>(smem + S::WH) + (parity ^ 1) * WARPS * RADIX / 4;
+      for (int i = tid; i < WARPS * RADIX / 4; i += THREADS) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+      // every CTA's counts have landed and the stage is complete
+      cluster_sync_all();
+      uint32_t total = 0u, below = 0u;
+      if (tid < RADIX) {
+#pragma unroll
+        for (uint32_t q = 0; q < S::MAX_CL; ++q) {
+          const uint32_t x = q < ncta ? s_cnt[q * RADIX + tid] : 0u;
+          total += x;
+          if (q < rank) below += x;
+        }
+      }
+      const uint32_t start = scan(total);
+      // staged key i of digit d goes to global position s_base[d] + i
+      if (tid < RADIX) s_base[tid] = start + below - lstart;
+      __syncthreads();
+      // ---- 3. remote stores of the staged runs into the owners' destination buffers
+      K* kd = reinterpret_cast<K*>(smem + S::KEYS) + (src ^ 1) * S::SLICE;
+      uint16_t* id = reinterpret_cast<uint16_t*>(smem + S::IDX) + (src ^ 1) * S::SLICE;
 #pragma unroll 4
-    for (int i = tid; i < SLICE; i += THREADS) {
-      const K k = ks[i];
-      const uint32_t g = s_base[digit_of(k, shift, mask)] + uint32_t(i);
-      const uint32_t owner = g / uint32_t(SLICE), at = g % uint32_t(SLICE);
-      st_cluster(map_shared(kd + at, owner), k);
-      if constexpr (VB > 0) st_cluster(map_shared(vd + at, owner), vs[i]);
+      for (uint32_t i = tid; i < len; i += THREADS) {
+        const K k = ks[i];
+        const uint32_t g = s_base[digit_of(k, shift, mask)] + i;
+        const uint32_t owner = __umulhi(g, magic), at = g - owner * slice;
+        st_cluster(map_shared(kd + at, owner), k);
+        if constexpr (INDEX) st_cluster(map_shared(id + at, owner), is[i]);
+      }
+      // ---- 4. the destination buffers are complete
+      cluster_sync_all();
+      src ^= 1;
     }
-    // ---- 4. the destination buffers are complete
+
+    // in order?  Each CTA checks its slice and, against the next one's first
+    // key, its end; every CTA learns every CTA's finding
+    const K* ks = reinterpret_cast<const K*>(smem + S::KEYS) + src * S::SLICE;
+    const uint16_t* is = reinterpret_cast<const uint16_t*>(smem + S::IDX) + src * S::SLICE;
+    if (tid == 0) {
+      const uint64_t first = len ? uint64_t(ks[0] & looked) : ~uint64_t(0);
+      s_edge[0] = uint32_t(first);
+      s_edge[1] = uint32_t(first >> 32);
+      s_edge[2] = INDEX && len ? is[0] : 0xffffu;
+    }
+    bool bad = false;
+    for (uint32_t i = tid; i + 1u < len; i += THREADS) {
+      const K a = ks[i] & looked, b = ks[i + 1] & looked;
+      if constexpr (INDEX) bad = bad || a > b || (a == b && is[i] > is[i + 1]);
+      else bad = bad || a > b;
+    }
     cluster_sync_all();
-    src ^= 1;
+    if (tid == 0 && len && rank + 1u < ncta) {
+      const uint64_t last = uint64_t(ks[len - 1u] & looked);
+      const uint64_t next = uint64_t(ld_cluster_u32(map_shared(s_edge, rank + 1u))) |
+                            uint64_t(ld_cluster_u32(map_shared(s_edge + 1, rank + 1u))) << 32;
+      const uint32_t next_i = ld_cluster_u32(map_shared(s_edge + 2, rank + 1u));
+      bad = bad || last > next || (INDEX && last == next && is[len - 1u] > next_i);
+    }
+    const int any = __syncthreads_or(bad);
+    if (uint32_t(tid) < ncta)
+      st_cluster(map_shared(s_flags + rank, uint32_t(tid)), uint32_t(any != 0));
+    cluster_sync_all();
+    uint32_t found = 0u;
+    for (uint32_t q = 0; q < ncta; ++q) found |= s_flags[q];
+    if (!found) break;  // the same in every CTA
   }
 
-  // write this CTA's slice out (untransformed)
-  const K* ks = s_k + src * SLICE;
-  const V* vs = s_v + src * SLICE;
-  for (uint32_t i = tid; i < uint32_t(SLICE); i += THREADS) {
-    const uint32_t g = base0 + i;
-    if (g < n && dbg_ok(g, n, kSiteClusterOut)) {
-      keys[g] = xf.on ? xf_inv(ks[i], xf) : ks[i];
-      if constexpr (VB > 0) vals[g] = vs[i];
+  // write this CTA's slice out (untransformed): everything is read before the
+  // first write
+  const K* ks = reinterpret_cast<const K*>(smem + S::KEYS) + src * S::SLICE;
+  [[maybe_unused]] const uint16_t* is =
+      reinterpret_cast<const uint16_t*>(smem + S::IDX) + src * S::SLICE;
+  V v[VB > 0 ? ITEMS : 1];
+  if constexpr (VB > 0) {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const uint32_t i = uint32_t(j * THREADS + tid);
+      if (i < len) v[j] = vals[is[i]];
+    }
+    cluster_sync_all();
+  }
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t i = uint32_t(j * THREADS + tid);
+    if (i < len && dbg_ok(base0 + i, n, kSiteClusterOut)) {
+      keys[base0 + i] = xf.on ? xf_inv(ks[i], xf) : ks[i];
+      if constexpr (VB > 0) vals[base0 + i] = v[j];
     }
   }
   if (ctrl != nullptr) {

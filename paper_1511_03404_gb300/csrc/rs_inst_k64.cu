@@ -10,7 +10,7 @@ const Variant* variants_k64(int* count) {
       SmallSort<uint64_t, 0, 8, 512, 16>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 16, 3>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 8, 4>::describe(),
-      SmallSort<uint64_t, 0, 8, 256, 16>::describe(),
+      SmallSort<uint64_t, 0, 8, 1024, 8>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 12, 3, true>::describe(),
       FusedSort<uint64_t, 0, 8, 256, 12, 3>::describe(),
       ClusterSort<uint64_t, 0, 8, 512, 16, 8>::describe(),

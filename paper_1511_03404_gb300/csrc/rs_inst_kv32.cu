@@ -12,7 +12,7 @@ const Variant* variants_kv32(int* count) {
       OnesweepSort<uint32_t, 4, 8, 256, 12, 4>::describe(),
       OnesweepSort<uint32_t, 4, 8, 256, 20, 3>::describe(),
       OnesweepSort<uint32_t, 4, 7, 256, 16, 4>::describe(),
-      SmallSort<uint32_t, 4, 8, 256, 16>::describe(),
+      SmallSort<uint32_t, 4, 8, 1024, 8>::describe(),
       OnesweepSort<uint32_t, 4, 8, 256, 16, 4, true>::describe(),
       FusedSort<uint32_t, 4, 8, 256, 16, 4>::describe(),
       FusedSort<uint32_t, 4, 8, 256, 8, 4>::describe(),

@@ -10,10 +10,10 @@ const Variant* variants_kv64(int* count) {
       SmallSort<uint64_t, 8, 8, 512, 16>::describe(),
       OnesweepSort<uint64_t, 8, 8, 256, 8, 3>::describe(),
       OnesweepSort<uint64_t, 8, 8, 256, 16, 2>::describe(),
-      SmallSort<uint64_t, 8, 8, 256, 16>::describe(),
+      SmallSort<uint64_t, 8, 8, 1024, 8>::describe(),
       OnesweepSort<uint64_t, 8, 8, 256, 12, 2, true>::describe(),
       FusedSort<uint64_t, 8, 8, 256, 12, 2>::describe(),
-      ClusterSort<uint64_t, 8, 8, 512, 8, 8>::describe(),
+      ClusterSort<uint64_t, 8, 8, 512, 16, 8>::describe(),
       OnesweepSort<uint64_t, 8, 8, 256, 14, 3, true>::describe(),
       OnesweepSort<uint64_t, 8, 8, 256, 23, 2, true>::describe(),
       OnesweepSort<uint64_t, 8, 8, 384, 14, 2, true>::describe(),

@@ -247,19 +247,24 @@ struct FusedSort {
 // the cluster's shared memory for every pass.
 template <class K, int VB, int R, int THREADS, int ITEMS, int CL>
 struct ClusterSort {
-  using S = ClusterSmem<K, VB, R, THREADS, ITEMS>;
-  static_assert(CL >= 1 && CL <= S::MAX_CL, "portable cluster sizes");
+  static constexpr int SLICE = THREADS * ITEMS;
+  static_assert(CL >= 1 && CL <= ClusterSmem<K, R, THREADS, ITEMS, true>::MAX_CL,
+                "portable cluster sizes");
+  static_assert(CL * SLICE <= 65536, "positions fit 16 bits");
 
   static size_t workspace(uint32_t, int) { return 0; }
 
-  static cudaError_t run(const SortArgs& a, int* in_alt) {
+  template <bool INDEX>
+  static cudaError_t launch(const SortArgs& a) {
     using V = ValT<VB>;
-    *in_alt = 0;  // sorted in place
-    auto kern = &k_cluster_sort<K, VB, R, THREADS, ITEMS>;
+    using S = ClusterSmem<K, R, THREADS, ITEMS, INDEX>;
+    auto kern = &k_cluster_sort<K, VB, R, THREADS, ITEMS, INDEX>;
     if (prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, S::BYTES) <= 0)
       return cudaErrorInvalidConfiguration;
-    const unsigned ncta = unsigned((size_t(a.n) + S::SLICE - 1) / S::SLICE);
-    if (ncta < 1 || ncta > unsigned(CL)) return cudaErrorInvalidValue;
+    if (a.n < 1 || a.n > uint32_t(CL) * SLICE) return cudaErrorInvalidValue;
+    // every CTA of the cluster takes part, whatever the length
+    uint32_t slice = (a.n + CL * THREADS - 1) / (CL * THREADS) * THREADS;
+    const unsigned ncta = (a.n + slice - 1) / slice;
     Ctrl* ctrl = (a.ws != nullptr && a.ws_bytes >= sizeof(Ctrl)) ? static_cast<Ctrl*>(a.ws)
                                                                   : nullptr;
     K* keys = static_cast<K*>(a.keys);
@@ -267,7 +272,8 @@ struct ClusterSort {
     uint32_t n = a.n;
     int begin = a.begin_bit, end = a.end_bit;
     KeyXf<K> xf = make_key_xf<K>(a.key_kind, a.descending);
-    void* args[] = {&keys, &vals, &n, &begin, &end, &ctrl, &xf};
+    bool mirror = a.knobs.mirror != 0;
+    void* args[] = {&keys, &vals, &n, &slice, &begin, &end, &ctrl, &xf, &mirror};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncta);
     cfg.blockDim = dim3(THREADS);
@@ -286,6 +292,14 @@ struct ClusterSort {
     return e;
   }
 
+  static cudaError_t run(const SortArgs& a, int* in_alt) {
+    *in_alt = 0;  // sorted in place
+    if constexpr (VB == 0) {
+      if (stages_keys<K, VB>(a.begin_bit, a.end_bit)) return launch<false>(a);
+    }
+    return launch<true>(a);
+  }
+
   static Variant describe() {
     Variant v{};
     v.key_bytes = int(sizeof(K));
@@ -294,7 +308,7 @@ struct ClusterSort {
     v.radix_bits = R;
     v.threads = THREADS;
     v.items = ITEMS;
-    v.max_n = uint32_t(CL) * uint32_t(S::SLICE);
+    v.max_n = uint32_t(CL) * uint32_t(SLICE);
     v.workspace = &workspace;
     v.run = &run;
     v.count = nullptr;
@@ -305,14 +319,14 @@ struct ClusterSort {
 template <class K, int VB, int R, int THREADS, int ITEMS>
 struct SmallSort {
   static constexpr int TILE = THREADS * ITEMS;
-  using S = SmallSmem<K, VB, R, THREADS, ITEMS>;
 
   static size_t workspace(uint32_t, int) { return 0; }
 
-  static cudaError_t run(const SortArgs& a, int* in_alt) {
+  template <bool INDEX>
+  static cudaError_t launch(const SortArgs& a) {
     using V = ValT<VB>;
-    *in_alt = 0;  // sorted in place
-    auto kern = &k_small_sort<K, VB, R, THREADS, ITEMS>;
+    using S = SmallSmem<K, VB, R, THREADS, ITEMS, INDEX>;
+    auto kern = &k_small_sort<K, VB, R, THREADS, ITEMS, INDEX>;
     if (prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, S::BYTES) <= 0)
       return cudaErrorInvalidConfiguration;
     prof_before(a.stream);
@@ -320,10 +334,19 @@ struct SmallSort {
                                                                   : nullptr;
     kern<<<1, THREADS, S::BYTES, a.stream>>>(static_cast<K*>(a.keys), static_cast<V*>(a.vals),
                                              a.n, a.begin_bit, a.end_bit, ctrl,
-                                             make_key_xf<K>(a.key_kind, a.descending));
+                                             make_key_xf<K>(a.key_kind, a.descending),
+                                             a.knobs.mirror != 0);
     const cudaError_t e = cudaGetLastError();
     prof_after(a.stream, 2, 2.0 * double(a.n) * double(sizeof(K) + VB));
     return e;
+  }
+
+  static cudaError_t run(const SortArgs& a, int* in_alt) {
+    *in_alt = 0;  // sorted in place
+    if constexpr (VB == 0) {
+      if (stages_keys<K, VB>(a.begin_bit, a.end_bit)) return launch<false>(a);
+    }
+    return launch<true>(a);
   }
 
   static Variant describe() {

@@ -17,7 +17,7 @@ namespace {
 template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS, int MINB = 4, int PASS_MINB = MINB>
 struct SegSort {
   using C = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, SMALL_ITEMS>;
-  static constexpr int PLAN_THREADS = 1024;
+  static constexpr int PLAN_THREADS = 256;
 
   static SegLayout layout(size_t n, size_t nseg, int passes) {
     return seg_layout(n, nseg, passes, R, C::TILE, C::CHUNK);
@@ -30,19 +30,18 @@ struct SegSort {
     const SegLayout L = layout(n, nseg, passes);
     char* w = static_cast<char*>(ws);
     Ctrl* ctrl = reinterpret_cast<Ctrl*>(w);
-    cudaError_t e = cudaMemsetAsync(w, 0, L.memset_bytes, s);
-    if (e != cudaSuccess) return e;
-    k_seg_plan<PLAN_THREADS><<<1, PLAN_THREADS, 0, s>>>(
-        d_off, nseg, n, uint32_t(C::SMALL_TILE), uint32_t(C::TILE), uint32_t(C::CHUNK), ctrl,
-        reinterpret_cast<uint32_t*>(w + L.small_ids), reinterpret_cast<SegDesc*>(w + L.descs),
-        reinterpret_cast<uint32_t*>(w + L.chunk_seg),
-        L.tiles_max, L.chunks_max);
-    e = cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(w, 0, sizeof(Ctrl), s);
     if (e != cudaSuccess) return e;
     // short segments: one CTA each, before the persistent kernel
-    auto small = &k_seg_small<K, VB, R, THREADS, SMALL_ITEMS, MINB>;
-    using SS = typename C::SS;
-    const int occ_small = prepare_kernel(reinterpret_cast<const void*>(small), THREADS, SS::BYTES);
+    auto small = &k_seg_small<K, VB, R, THREADS, SMALL_ITEMS, true, MINB>;
+    int smem_small = SmallSmem<K, VB, R, THREADS, SMALL_ITEMS, true>::BYTES;
+    if constexpr (VB == 0) {
+      if (begin_bit == 0 && end_bit == 8 * int(sizeof(K))) {  // whole keys need no positions
+        small = &k_seg_small<K, VB, R, THREADS, SMALL_ITEMS, false, MINB>;
+        smem_small = SmallSmem<K, VB, R, THREADS, SMALL_ITEMS, false>::BYTES;
+      }
+    }
+    const int occ_small = prepare_kernel(reinterpret_cast<const void*>(small), THREADS, smem_small);
     if (occ_small <= 0) return cudaErrorInvalidConfiguration;
     auto hist = &k_seg_hist<K, R, C::HIST_THREADS, C::MAXP, C::HIST_SLOTS, C::CHUNK, C::TILE,
                             CHUNK_TILES, C::HIST_MINB>;
@@ -77,6 +76,13 @@ struct SegSort {
     a.nseg = nseg;
     a.knobs = knobs;
     using V = ValT<VB>;
+    k_seg_plan<PLAN_THREADS, C::RADIX>
+        <<<unsigned((nseg + PLAN_THREADS - 1) / PLAN_THREADS), PLAN_THREADS, 0, s>>>(
+            n, uint32_t(C::SMALL_TILE), uint32_t(C::TILE), uint32_t(C::CHUNK), L.chunks_max,
+            reinterpret_cast<uint32_t*>(w + L.small_ids), reinterpret_cast<SegDesc*>(w + L.descs),
+            reinterpret_cast<uint32_t*>(w + L.chunk_seg), a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     // grids no larger than the work can be: at most tiles_max pass tiles per
     // pass and chunks_max histogram chunks (bounds the host knows without
     // the plan), so that a small batch does not spread idle CTAs over every
@@ -89,7 +95,7 @@ struct SegSort {
     const unsigned grid_small =
         unsigned(std::max<size_t>(1, std::min<size_t>(nseg, sms * occ_small)));
     prof_before(s);
-    small<<<grid_small, THREADS, SS::BYTES, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
+    small<<<grid_small, THREADS, smem_small, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
                                                  static_cast<K*>(keys_alt),
                                                  static_cast<V*>(vals_alt), a);
     hist<<<grid_hist, C::HIST_THREADS,

@@ -2,11 +2,11 @@
 // independently to every segment [off[s], off[s+1]) of one array, for all
 // segments in one persistent launch.
 //
-//   k_seg_plan        one CTA: classifies segments (short ones fit one CTA,
-//                     long ones are tiled), numbers the work items and maps
-//                     every histogram chunk to its segment.
+//   k_seg_plan        classifies segments (tiny ones fit one warp, short ones
+//                     one CTA, long ones are tiled), numbers the work items
+//                     and maps every histogram chunk to its segment.
 //   k_seg_small       short segments, each sorted whole in one CTA's shared
-//                     memory (every pass), grid-stride over the short list;
+//                     memory (every pass) or by one warp;
 //   k_seg_hist        the digit histograms of the long segments, chunk by
 //                     chunk; each segment's last chunk scans them and writes
 //                     the descriptors of the segment's pass tiles;
@@ -53,11 +53,9 @@ struct TileDesc {
 };
 static_assert(sizeof(TileDesc) == 32, "TileDesc is 32 bytes");
 
-// Per long segment: histogram ticket, ready word (bit 0: the histograms are
-// scanned; bits 1..: the mask of passes that move data; kept for inspection,
-// the pass kernel takes the mask from its tile descriptor), done counters.
+// Per long segment: histogram ticket, done counters.
 constexpr int kSegStateWords = 16;
-enum SegStateField { kSegTicket = 0, kSegReady = 1, kSegDone0 = 3 };
+enum SegStateField { kSegTicket = 0, kSegDone0 = 3 };
 
 // Plan results in Ctrl::tile_counter[]
 enum SegCtrlField {
@@ -66,12 +64,13 @@ enum SegCtrlField {
   kNLarge = 2,
   kNTiles = 3,   // pass tiles of all long segments (one pass)
   kNChunks = 4,  // histogram chunks of all long segments
-  kPlanned = 5   // 1 once the plan is complete
+  kNTiny = 6,    // segments of 1 to 32 elements
+  kSmallQueue = 7  // work-queue ticket of the short segments
 };
+constexpr uint32_t kTinyMax = 32;
 
 struct SegLayout {
   size_t small_ids, descs, tdesc, chunk_seg, state, counts, offsets, status, total;
-  size_t memset_bytes;  // Ctrl + state + counts
   size_t tiles_max, chunks_max;
 };
 
@@ -83,8 +82,7 @@ inline SegLayout seg_layout(size_t n, size_t nseg, int passes, int radix_bits, i
   L.chunks_max = (n + chunk - 1) / chunk + nseg;
   L.state = 256;
   L.counts = align_up(L.state + nseg * kSegStateWords * 4, 256);
-  L.memset_bytes = align_up(L.counts + nseg * passes * radix * 4, 256);
-  L.offsets = L.memset_bytes;
+  L.offsets = align_up(L.counts + nseg * passes * radix * 4, 256);
   L.small_ids = align_up(L.offsets + nseg * passes * radix * 4, 256);
   L.descs = align_up(L.small_ids + nseg * 4, 256);
   L.tdesc = align_up(L.descs + nseg * sizeof(SegDesc), 256);
@@ -93,140 +91,6 @@ inline SegLayout seg_layout(size_t n, size_t nseg, int passes, int radix_bits, i
   L.total = align_up(L.status + size_t(passes) * L.tiles_max * radix * 4, 256);
   return L;
 }
-
-// One CTA numbers the work.  Segments longer than small_max are "long".
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1)
-    k_seg_plan(const uint64_t* __restrict__ off, uint64_t nseg, uint64_t n, uint32_t small_max,
-               uint32_t tile, uint32_t chunk, Ctrl* __restrict__ ctrl,
-               uint32_t* __restrict__ small_ids, SegDesc* __restrict__ descs,
-               uint32_t* __restrict__ chunk_seg,
-               uint64_t tiles_max, uint64_t chunks_max) {
-  __shared__ uint32_t s_tot[32];
-  __shared__ uint32_t s_run[4];
-  __shared__ int s_bad;
-  const int tid = threadIdx.x;
-  if (tid < 4) s_run[tid] = 0u;
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  if (off[0] != 0ull || off[nseg] != n) s_bad = 1;  // benign race: same value
-  for (uint64_t base = 0; base < nseg; base += THREADS) {
-    const uint64_t s = base + tid;
-    uint64_t len = 0;
-    bool valid = s < nseg;
-    if (valid) {
-      const uint64_t a = off[s], b = off[s + 1];
-      if (b < a || b > n || b - a > uint64_t((1u << 30) - 1u)) {
-        s_bad = 1;
-        valid = false;
-      } else {
-        len = b - a;
-      }
-    }
-    const bool is_long = valid && len > small_max;
-    const uint32_t small = (valid && !is_long) ? 1u : 0u;
-    const uint32_t lng = is_long ? 1u : 0u;
-    const uint32_t nt = is_long ? uint32_t((len + tile - 1) / tile) : 0u;
-    const uint32_t nc = is_long ? uint32_t((len + chunk - 1) / chunk) : 0u;
-    const uint32_t e_small = block_exclusive_scan<THREADS>(small, s_tot);
-    __syncthreads();
-    const uint32_t e_long = block_exclusive_scan<THREADS>(lng, s_tot);
-    __syncthreads();
-    const uint32_t e_tile = block_exclusive_scan<THREADS>(nt, s_tot);
-    __syncthreads();
-    const uint32_t e_chunk = block_exclusive_scan<THREADS>(nc, s_tot);
-    const uint32_t r_small = s_run[0], r_long = s_run[1], r_tile = s_run[2],
-                   r_chunk = s_run[3];
-    if (small && dbg_ok(r_small + e_small, nseg, kSiteSegPlan))
-      small_ids[r_small + e_small] = uint32_t(s);
-    const uint32_t li = r_long + e_long;
-    bool map_ok = false;
-    if (is_long) {
-      SegDesc d;
-      d.off = off[s];
-      d.len = uint32_t(len);
-      d.tile0 = r_tile + e_tile;
-      d.chunk0 = r_chunk + e_chunk;
-      d.seg = uint32_t(s);
-      d.pad[0] = d.pad[1] = 0u;
-      if (dbg_ok(li, nseg, kSiteSegPlan)) descs[li] = d;
-      map_ok = uint64_t(d.tile0) + nt <= tiles_max && uint64_t(d.chunk0) + nc <= chunks_max;
-      if (!map_ok) s_bad = 1;
-    }
-    // the chunk map of these long segments: each warp writes its lanes'
-    // segments one after another, 32 consecutive entries per store (one
-    // thread writing its own segment's entries issued one store each)
-    {
-      const int lane = tid & 31;
-      const uint32_t c0 = r_chunk + e_chunk;
-      for (uint32_t m = __ballot_sync(kFull, map_ok); m != 0u; m &= m - 1u) {
-        const int src = __ffs(int(m)) - 1;
-        const uint32_t sli = __shfl_sync(kFull, li, src), sc0 = __shfl_sync(kFull, c0, src);
-        const uint32_t snc = __shfl_sync(kFull, nc, src);
-        for (uint32_t i = uint32_t(lane); i < snc; i += 32)
-          if (dbg_ok(uint64_t(sc0) + i, chunks_max, kSiteSegPlan)) chunk_seg[sc0 + i] = sli;
-      }
-    }
-    __syncthreads();
-    if (tid == THREADS - 1) {  // the last thread's inclusive sums are the block totals
-      s_run[0] = r_small + e_small + small;
-      s_run[1] = r_long + e_long + lng;
-      s_run[2] = r_tile + e_tile + nt;
-      s_run[3] = r_chunk + e_chunk + nc;
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    if (s_bad) {
-      report_error(ctrl, kDevInvalid, 0u);
-      ctrl->tile_counter[kNSmall] = ctrl->tile_counter[kNLarge] = 0u;
-      ctrl->tile_counter[kNTiles] = ctrl->tile_counter[kNChunks] = 0u;
-    } else {
-      ctrl->tile_counter[kNSmall] = s_run[0];
-      ctrl->tile_counter[kNLarge] = s_run[1];
-      ctrl->tile_counter[kNTiles] = s_run[2];
-      ctrl->tile_counter[kNChunks] = s_run[3];
-    }
-    ctrl->tile_counter[kPlanned] = 1u;
-  }
-}
-
-// Shared memory of one short-segment sort: the warps' counters and peer
-// masks, and the segment's keys and values, each in a buffer of its own.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS>
-struct SegSmallSmem {
-  static constexpr int RADIX = 1 << RADIX_BITS;
-  static constexpr int WARPS = THREADS / 32;
-  static constexpr int TILE = THREADS * ITEMS;
-  static constexpr int WH = 0;                        // u32 [WARPS][RADIX] warp counters
-  static constexpr int MM = WH + WARPS * RADIX * 4;   // u32 [WARPS][RADIX] peer masks
-  static constexpr int TOT = MM + WARPS * RADIX * 4;  // u32 [32]
-  static constexpr int KEYS = (TOT + 32 * 4 + 15) / 16 * 16;  // K [TILE]
-  static constexpr int VALS = KEYS + TILE * int(sizeof(K));   // V [TILE]
-  static constexpr int BYTES = VALS + (VB > 0 ? TILE * VB : 0);
-};
-
-// SMALL_ITEMS: keys per thread of the short-segment sort, whose tile bounds a
-// short segment.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES,
-          int SMALL_ITEMS = ITEMS, bool INDEX = true>
-struct SegKernelCfg {
-  static constexpr int RADIX = 1 << RADIX_BITS;
-  static constexpr int TILE = THREADS * ITEMS;
-  static constexpr int SMALL_TILE = THREADS * SMALL_ITEMS;
-  static constexpr int CHUNK = TILE * CHUNK_TILES;
-  static constexpr int MAXP = (8 * int(sizeof(K)) + RADIX_BITS - 1) / RADIX_BITS;
-  // histogram kernel: [pass][digit][16 lane slots] u32 counters, 1024 threads
-  static constexpr int HIST_THREADS = 1024;
-  static constexpr int HIST_SLOTS = 16;
-  static constexpr int HIST_BYTES = MAXP * RADIX * HIST_SLOTS * 4;
-  // two CTAs per SM while their counters fit (32-bit keys), else one
-  static constexpr int HIST_MINB = HIST_BYTES <= 100 * 1024 ? 2 : 1;
-  using OS = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
-  using SS = SegSmallSmem<K, VB, RADIX_BITS, THREADS, SMALL_ITEMS>;
-  static constexpr int MISC = (OS::BYTES + 15) / 16 * 16;  // u32 [8]
-  static constexpr int BYTES = MISC + 32;
-};
 
 struct SegArgs {
   const uint64_t* off;
@@ -245,102 +109,179 @@ struct SegArgs {
   Knobs knobs;
 };
 
-// Every digit pass (Sec. 2.6) of one segment of len <= TILE elements inside
-// one CTA.  The segment lives in shared memory from the first load to the
-// last store; a pass reads each thread's items from it, ranks them, and
-// writes them back at their stable positions (a barrier separates the reads
-// from the writes), keys first, then values.  So no more than one item array
-// and the positions are live in registers at a time, and four CTAs fit on an
-// SM.  Past the end the keys are the largest key: they rank after every real
-// key in every pass and are never written out.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS>
-__device__ __forceinline__ void seg_cta_sort(const K* kin, const ValT<VB>* vin, K* kout,
-                                             ValT<VB>* vout, uint32_t len, int begin_bit,
-                                             int end_bit, unsigned char* smem) {
-  using V = ValT<VB>;
-  using S = SegSmallSmem<K, VB, RADIX_BITS, THREADS, ITEMS>;
-  constexpr int RADIX = S::RADIX, WARPS = S::WARPS, TILE = S::TILE;
-  uint32_t* s_wh = reinterpret_cast<uint32_t*>(smem + S::WH);
-  uint32_t* s_mm = reinterpret_cast<uint32_t*>(smem + S::MM);
-  uint32_t* s_tot = reinterpret_cast<uint32_t*>(smem + S::TOT);
-  K* s_k = reinterpret_cast<K*>(smem + S::KEYS);
-  V* s_v = reinterpret_cast<V*>(smem + S::VALS);
+// Numbers the work, one segment a thread.  Segments longer than small_max are
+// "long"; of the others, those of 1 to 32 elements are "tiny" (listed from the
+// end of small_ids), the rest "small"; empty ones are left out.  The order
+// inside the lists is of no consequence, so each CTA takes its places from
+// global counters: with one CTA scanning all segments in order, 20,000 of them
+// took 87 us.  The state of long segments, and the digit counts of those of
+// several chunks, are cleared here: clearing every segment's took 80 MB of
+// stores for 20,000.  Bad offsets are reported; the kernels that follow then
+// do nothing.
+template <int THREADS, int RADIX>
+__global__ void __launch_bounds__(THREADS)
+    k_seg_plan(uint64_t n, uint32_t small_max, uint32_t tile, uint32_t chunk, uint64_t chunks_max,
+               uint32_t* __restrict__ small_ids, SegDesc* __restrict__ descs,
+               uint32_t* __restrict__ chunk_seg, SegArgs a) {
+  constexpr int COUNTS = 5, WARPS = THREADS / 32;
+  const int field[COUNTS] = {kNTiny, kNSmall, kNLarge, kNTiles, kNChunks};
+  __shared__ uint32_t s_tot[COUNTS][WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + lane);
-
-  for (uint32_t i = tid; i < uint32_t(TILE); i += THREADS) {
-    s_k[i] = i < len ? kin[i] : ~K(0);
-    if constexpr (VB > 0) s_v[i] = i < len ? vin[i] : V(0);
+  const uint64_t s = uint64_t(blockIdx.x) * THREADS + tid;
+  uint64_t from = 0;
+  uint32_t len = 0u;
+  bool bad = s == 0 && (a.off[0] != 0ull || a.off[a.nseg] != n);
+  if (s < a.nseg) {
+    from = a.off[s];
+    const uint64_t to = a.off[s + 1];
+    if (to < from || to > n || to - from > uint64_t((1u << 30) - 1u)) bad = true;
+    else len = uint32_t(to - from);
   }
-  for (int lo = begin_bit; lo < end_bit; lo += RADIX_BITS) {
-    const uint32_t shift = uint32_t(lo);
-    const uint32_t mask = (1u << (min(lo + RADIX_BITS, end_bit) - lo)) - 1u;
-    for (int i = tid; i < 2 * WARPS * RADIX; i += THREADS) s_wh[i] = 0u;  // counters + masks
-    __syncthreads();
-    K key[ITEMS];
-    uint32_t dp[ITEMS];  // digit << 16 | rank in the warp, then the item's position
+  const bool tiny = len >= 1u && len <= kTinyMax, lng = len > small_max;
+  const bool small = len > kTinyMax && !lng;
+  const uint32_t nt = lng ? (len + tile - 1u) / tile : 0u, nc = lng ? (len + chunk - 1u) / chunk : 0u;
+  const uint32_t mine[COUNTS] = {tiny, small, lng, nt, nc};
+  uint32_t at[COUNTS];
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      key[j] = s_k[slot0 + j * 32];
-      dp[j] = digit_of(key[j], shift, mask);
-    }
-    warp_rank_packed<ITEMS>(dp, s_wh + warp * RADIX, s_mm + warp * RADIX, lane);
-    __syncthreads();
-    // per digit: exclusive prefix over the warps, from the digit's start
-    uint32_t cnt = 0u;
-    if (tid < RADIX) {
-#pragma unroll
-      for (int w = 0; w < WARPS; ++w) cnt += s_wh[w * RADIX + tid];
-    }
-    const uint32_t start = block_exclusive_scan<THREADS>(cnt, s_tot);
-    if (tid < RADIX) {
-      uint32_t run = start;
-#pragma unroll
-      for (int w = 0; w < WARPS; ++w) {
-        const uint32_t c = s_wh[w * RADIX + tid];
-        s_wh[w * RADIX + tid] = run;
-        run += c;
-      }
-    }
-    __syncthreads();  // every key of the pass was read above
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      dp[j] = (dp[j] & 0xffffu) + s_wh[warp * RADIX + (dp[j] >> 16)];
-      s_k[dp[j]] = key[j];
-    }
-    if constexpr (VB > 0) {
-      V val[ITEMS];
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) val[j] = s_v[slot0 + j * 32];
-      __syncthreads();  // every value was read
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) s_v[dp[j]] = val[j];
-    }
-    __syncthreads();
+  for (int q = 0; q < COUNTS; ++q) {
+    const uint32_t inc = warp_inclusive_scan(mine[q], lane);
+    if (lane == 31) s_tot[q][warp] = inc;
+    at[q] = inc - mine[q];
   }
-  for (uint32_t i = tid; i < len; i += THREADS) {
-    if (!dbg_ok(i, len, kSiteSegSmallOut)) continue;
-    kout[i] = s_k[i];
-    if constexpr (VB > 0) vout[i] = s_v[i];
+  __syncthreads();
+  if (tid < COUNTS) {  // thread q: the warps' places among count q
+    uint32_t sum = 0u;
+    for (int w = 0; w < WARPS; ++w) sum += s_tot[tid][w];
+    uint32_t run = sum ? atomicAdd(&a.ctrl->tile_counter[field[tid]], sum) : 0u;
+    for (int w = 0; w < WARPS; ++w) {
+      const uint32_t x = s_tot[tid][w];
+      s_tot[tid][w] = run;
+      run += x;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < COUNTS; ++q) at[q] += s_tot[q][warp];
+  const uint64_t slot = tiny ? a.nseg - 1u - at[0] : at[1];
+  if ((tiny || small) && dbg_ok(slot, a.nseg, kSiteSegPlan)) small_ids[slot] = uint32_t(s);
+  const uint32_t li = at[2], c0 = at[4];
+  bool map_ok = false;
+  if (lng) {
+    SegDesc d;
+    d.off = from;
+    d.len = len;
+    d.tile0 = at[3];
+    d.chunk0 = c0;
+    d.seg = uint32_t(s);
+    d.pad[0] = d.pad[1] = 0u;
+    if (dbg_ok(li, a.nseg, kSiteSegPlan)) descs[li] = d;
+    map_ok = uint64_t(d.tile0) + nt <= a.tiles_max && uint64_t(c0) + nc <= chunks_max;
+    if (!map_ok) bad = true;
+  }
+  if (bad) report_error(a.ctrl, kDevInvalid, 0u);
+  // each warp writes its lanes' long segments one after another, consecutive
+  // entries per store: the chunk map, the state, the counts
+  for (uint32_t m = __ballot_sync(kFull, map_ok); m != 0u; m &= m - 1u) {
+    const int src = __ffs(int(m)) - 1;
+    const uint32_t sli = __shfl_sync(kFull, li, src), sc0 = __shfl_sync(kFull, c0, src);
+    const uint32_t snc = __shfl_sync(kFull, nc, src);
+    for (uint32_t i = uint32_t(lane); i < snc; i += 32)
+      if (dbg_ok(uint64_t(sc0) + i, chunks_max, kSiteSegPlan)) chunk_seg[sc0 + i] = sli;
+    if (!dbg_ok(sli, a.nseg, kSiteSegState)) continue;
+    if (lane < kSegStateWords) a.state[size_t(sli) * kSegStateWords + lane] = 0u;
+    if (snc > 1u) {
+      uint32_t* cnt = a.counts + size_t(sli) * a.passes * RADIX;
+      for (int i = lane; i < a.passes * RADIX; i += 32) cnt[i] = 0u;
+    }
   }
 }
 
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int MINB = 4>
+// SMALL_ITEMS: keys per thread of the short-segment sort, whose tile bounds a
+// short segment.
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, int CHUNK_TILES,
+          int SMALL_ITEMS = ITEMS, bool INDEX = true>
+struct SegKernelCfg {
+  static constexpr int RADIX = 1 << RADIX_BITS;
+  static constexpr int TILE = THREADS * ITEMS;
+  static constexpr int SMALL_TILE = THREADS * SMALL_ITEMS;
+  static constexpr int CHUNK = TILE * CHUNK_TILES;
+  static constexpr int MAXP = (8 * int(sizeof(K)) + RADIX_BITS - 1) / RADIX_BITS;
+  // histogram kernel: [pass][digit][16 lane slots] u32 counters, 1024 threads
+  static constexpr int HIST_THREADS = 1024;
+  static constexpr int HIST_SLOTS = 16;
+  static constexpr int HIST_BYTES = MAXP * RADIX * HIST_SLOTS * 4;
+  // two CTAs per SM while their counters fit (32-bit keys), else one
+  static constexpr int HIST_MINB = HIST_BYTES <= 100 * 1024 ? 2 : 1;
+  using OS = OnesweepSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
+  static constexpr int MISC = (OS::BYTES + 15) / 16 * 16;  // u32 [8]
+  static constexpr int BYTES = MISC + 32;
+};
+
+// One segment of at most 32 elements, sorted by one warp: an element's place
+// is the number of elements that are smaller, or equal and earlier.
+template <class K, int VB>
+__device__ __forceinline__ void seg_warp_sort(const K* kin, const ValT<VB>* vin, K* kout,
+                                              ValT<VB>* vout, uint32_t len, K looked) {
+  const uint32_t lane = threadIdx.x & 31u;
+  K k = K(0);
+  ValT<VB> v = 0;
+  if (lane < len) {
+    k = kin[lane];
+    if constexpr (VB > 0) v = vin[lane];
+  }
+  const K mine = k & looked;
+  uint32_t place = 0u;
+  for (uint32_t j = 0; j < len; ++j) {
+    const K other = __shfl_sync(kFull, mine, int(j));
+    place += (other < mine || (other == mine && j < lane)) ? 1u : 0u;
+  }
+  // (every load of the warp has completed: its key was shuffled, its value
+  // is ordered by the warp barrier)
+  __syncwarp();
+  if (lane < len && dbg_ok(place, len, kSiteSegSmallOut)) {
+    kout[place] = k;
+    if constexpr (VB > 0) vout[place] = v;
+  }
+}
+
+// The short segments: those of up to 32 elements one warp each, the others
+// one CTA each, taken from a queue (the next one is asked for while the
+// current one is sorted), so that long and short ones even out.
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_seg_small(K* __restrict__ k0, ValT<VB>* __restrict__ v0, K* __restrict__ k1,
                 ValT<VB>* __restrict__ v1, SegArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t s_next[2];
   const int passes = a.passes;
   K* kout = (passes & 1) ? k1 : k0;  // where the pass count parity puts the result
   ValT<VB>* vout = (passes & 1) ? v1 : v0;
+  if (a.ctrl->error != 0u) return;  // bad offsets: nothing is written
   const uint32_t n_small = a.ctrl->tile_counter[kNSmall];
-  for (uint32_t i = blockIdx.x; i < n_small; i += gridDim.x) {
+  const uint32_t n_tiny = a.ctrl->tile_counter[kNTiny];
+  const K looked = (a.end_bit - a.begin_bit == 8 * int(sizeof(K)))
+                       ? ~K(0)
+                       : K(((K(1) << (a.end_bit - a.begin_bit)) - K(1)) << a.begin_bit);
+  if (threadIdx.x == 0) s_next[0] = atomicAdd(&a.ctrl->tile_counter[kSmallQueue], 1u);
+  __syncthreads();
+  for (uint32_t it = 0;; ++it) {
+    const uint32_t i = s_next[it & 1u];
+    if (i >= n_small) break;
+    if (threadIdx.x == 0) s_next[(it + 1u) & 1u] = atomicAdd(&a.ctrl->tile_counter[kSmallQueue], 1u);
     const uint32_t s = a.small_ids[i];
     const uint64_t b = a.off[s];
     const uint32_t len = uint32_t(a.off[s + 1] - b);
-    seg_cta_sort<K, VB, RADIX_BITS, THREADS, ITEMS>(k0 + b, v0 + b, kout + b, vout + b, len,
-                                                    a.begin_bit, a.end_bit, smem);
+    cta_sort<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>(k0 + b, v0 + b, kout + b, vout + b, len,
+                                                       a.begin_bit, a.end_bit, smem,
+                                                       KeyXf<K>{}, a.knobs.mirror != 0);
     __syncthreads();
+  }
+  const uint32_t warps = gridDim.x * (THREADS / 32);
+  for (uint32_t i = (blockIdx.x * THREADS + threadIdx.x) / 32u; i < n_tiny; i += warps) {
+    const uint32_t s = a.small_ids[a.nseg - 1u - i];  // listed from the end
+    const uint64_t b = a.off[s];
+    const uint32_t len = uint32_t(a.off[s + 1] - b);
+    seg_warp_sort<K, VB>(k0 + b, v0 + b, kout + b, vout + b, len, looked);
   }
 }
 
@@ -349,18 +290,24 @@ __global__ void __launch_bounds__(THREADS, MINB)
 // the whole-array upsweep: 16-byte loads, every pass's digit counted into
 // per-lane-slot shared counters, then the chunk's counts added to its
 // segment's.  The chunk also clears the look-back words of its tiles.  The
-// last chunk of a segment (ticket) scans the segment's histograms, chooses the
-// passes that move data and marks the segment ready for its pass tiles.
+// last chunk of a segment (ticket; most segments are one chunk, and need no
+// counts in memory) scans the segment's histograms, chooses the passes that
+// move data and writes the descriptors of the segment's pass tiles.
+//
+// Bound by latency for segments of a tile or two: counting each in its own
+// chunk, adding it up in memory and scanning one pass after another took 218
+// us for the 3,500 long ones of 2^26 pairs in 20,000 segments.
 template <class K, int RADIX_BITS, int THREADS, int MAXP, int SLOTS, int CHUNK, int TILE,
           int CHUNK_TILES, int MINB = 2>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_seg_hist(const K* __restrict__ k0, SegArgs a) {
   constexpr int RADIX = 1 << RADIX_BITS;
   constexpr int VEC = 16 / int(sizeof(K));
-  static_assert(RADIX <= THREADS, "one thread per digit in the scan");
+  static_assert(THREADS == 1024 && RADIX % 32 == 0, "32 warps' sums, whole warps per pass");
   extern __shared__ uint32_t sh[];  // [passes][RADIX][SLOTS]
   __shared__ uint32_t s_tot[32];
   __shared__ int s_last;
+  __shared__ uint32_t s_one;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t slot = uint32_t(lane & (SLOTS - 1));
   const int passes = a.passes;
@@ -379,6 +326,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
         atomicAdd(&sh[(p * RADIX + int(digit_of(k, shiftp[p], maskp[p]))) * SLOTS + int(slot)],
                   1u);
   };
+  if (a.ctrl->error != 0u) return;  // bad offsets
   const uint32_t n_chunks = a.ctrl->tile_counter[kNChunks];
   const int words = passes * RADIX * SLOTS;
   for (uint32_t item = blockIdx.x; item < n_chunks; item += gridDim.x) {
@@ -419,15 +367,27 @@ __global__ void __launch_bounds__(THREADS, MINB)
       }
     }
     __syncthreads();
-    // the chunk's counts into the segment's: one (pass, digit) per thread
+    // the chunk's counts, one (pass, digit) per thread; a segment of several
+    // chunks adds them up in memory
+    constexpr int PER = THREADS / RADIX;  // passes at a time
+    const int pq = tid / RADIX, dq = tid % RADIX;
+    const uint32_t chunks = (d.len + CHUNK - 1) / CHUNK;
     uint32_t* cnt = a.counts + size_t(li) * passes * RADIX;
-    for (int w = tid; w < passes * RADIX; w += THREADS) {
-      const uint32_t* row = sh + w * SLOTS;
-      uint32_t c = 0u;
+    uint32_t mine[(MAXP + PER - 1) / PER];
 #pragma unroll
-      for (int l = 0; l < SLOTS; ++l) c += row[(l + lane) & (SLOTS - 1)];  // rotated: no conflicts
-      if (c && dbg_ok(uint64_t(li) * passes * RADIX + w, a.nseg * passes * RADIX, kSiteSegCounts))
-        atomicAdd(&cnt[w], c);
+    for (int q = 0; q < (MAXP + PER - 1) / PER; ++q) {
+      const int p = q * PER + pq;
+      uint32_t c = 0u;
+      if (p < passes) {
+        const uint32_t* row = sh + (p * RADIX + dq) * SLOTS;
+#pragma unroll
+        for (int l = 0; l < SLOTS; ++l) c += row[(l + lane) & (SLOTS - 1)];  // rotated: no conflicts
+        if (chunks > 1u && c != 0u &&
+            dbg_ok((uint64_t(li) * passes + p) * RADIX + dq, a.nseg * passes * RADIX,
+                   kSiteSegCounts))
+          atomicAdd(&cnt[p * RADIX + dq], c);
+      }
+      mine[q] = c;
     }
     // clear the look-back words of this chunk's tiles [ta, tb), every pass.
     // In the [tile/4][digit][tile%4] layout one digit's words of four
@@ -453,30 +413,48 @@ __global__ void __launch_bounds__(THREADS, MINB)
         }
       }
     }
-    __syncthreads();
-    uint32_t* state = a.state + size_t(li) * kSegStateWords;
-    if (tid == 0) {
-      // the CTA's counts and cleared words (ordered before by the barrier)
-      // become visible before the ticket
-      __threadfence();
-      const uint32_t chunks = (d.len + CHUNK - 1) / CHUNK;
-      s_last = dbg_ok(li, a.nseg, kSiteSegState) &&
-               atomicAdd(&state[kSegTicket], 1u) == chunks - 1u;
-    }
-    __syncthreads();
-    if (s_last) {
-      // last chunk of the segment: scan each pass's histogram
-      __threadfence();
-      uint32_t* offs = a.offsets + size_t(li) * passes * RADIX;
-      uint32_t exec = 0u;
-      for (int p = 0; p < passes; ++p) {
-        const uint32_t c = tid < RADIX ? ld_relaxed(&cnt[p * RADIX + tid]) : 0u;
-        const uint32_t e = block_exclusive_scan<THREADS>(c, s_tot);
-        if (tid < RADIX && dbg_ok(uint64_t(li) * passes * RADIX + p * RADIX + tid,
-                                  a.nseg * passes * RADIX, kSiteSegCounts))
-          offs[p * RADIX + tid] = e;
-        if (!__syncthreads_or(tid < RADIX && c == d.len)) exec |= 1u << p;
+    bool last = true;
+    if (chunks > 1u) {
+      __syncthreads();
+      if (tid == 0) {
+        // the CTA's counts and cleared words (ordered before by the barrier)
+        // become visible before the ticket
+        __threadfence();
+        uint32_t* state = a.state + size_t(li) * kSegStateWords;
+        s_last = dbg_ok(li, a.nseg, kSiteSegState) &&
+                 atomicAdd(&state[kSegTicket], 1u) == chunks - 1u;
       }
+      __syncthreads();
+      last = s_last != 0;
+      if (last) {
+        __threadfence();
+#pragma unroll
+        for (int q = 0; q < (MAXP + PER - 1) / PER; ++q)
+          mine[q] = q * PER + pq < passes ? ld_relaxed(&cnt[(q * PER + pq) * RADIX + dq]) : 0u;
+      }
+    }
+    if (last) {
+      // the segment's counts are complete: scan every pass's at once, and
+      // find the passes that move data
+      uint32_t* offs = a.offsets + size_t(li) * passes * RADIX;
+      if (tid == 0) s_one = 0u;
+#pragma unroll
+      for (int q = 0; q < (MAXP + PER - 1) / PER; ++q) {
+        const int p = q * PER + pq;
+        const uint32_t inc = warp_inclusive_scan(mine[q], lane);
+        const int warp = tid >> 5;
+        __syncthreads();  // s_one is clear; the round before has read s_tot
+        if (lane == 31) s_tot[warp] = inc;
+        if (mine[q] == d.len) atomicOr(&s_one, 1u << p);  // one digit value holds every key
+        __syncthreads();
+        const int w0 = warp / (RADIX / 32) * (RADIX / 32);  // my pass's first warp
+        const uint32_t start =
+            __reduce_add_sync(kFull, lane >= w0 && lane < warp ? s_tot[lane] : 0u) + inc - mine[q];
+        if (p < passes && dbg_ok((uint64_t(li) * passes + p) * RADIX + dq,
+                                 a.nseg * passes * RADIX, kSiteSegCounts))
+          offs[p * RADIX + dq] = start;
+      }
+      uint32_t exec = ~s_one & ((1u << passes) - 1u);
       if ((__popc(exec) & 1) != (passes & 1)) {  // every thread: the same exec
         const uint32_t skipped = ~exec & ((1u << passes) - 1u);
         exec |= skipped & (0u - skipped);
@@ -494,10 +472,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
         td.exec = exec;
         td.pad[0] = td.pad[1] = 0u;
         a.tdesc[d.tile0 + t] = td;
-      }
-      if (tid == 0) {
-        __threadfence();
-        st_release(&state[kSegReady], 1u | (exec << 1));
       }
     }
     __syncthreads();

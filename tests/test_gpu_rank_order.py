@@ -13,7 +13,7 @@ import inputs
 import oracle
 
 torch = pytest.importorskip("torch")
-from gpu_util import sort_via_abi  # noqa: E402
+from gpu_util import from_dev, sort_via_abi, to_dev  # noqa: E402
 
 from paper_1511_03404_gb300 import rs  # noqa: E402
 
@@ -45,9 +45,13 @@ def mirrored():
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
 def test_out_of_turn_ranks_are_repaired(dtype, pairs, mirrored):
     kb = np.dtype(dtype).itemsize
-    for var in variants(kb, kb if pairs else 0, (0, 2, 3)):
+    for var in variants(kb, kb if pairs else 0, (0, 1, 2, 3, 4)):
         tile = var["threads"] * var["items"]
-        for n in (tile - 1, tile, 3 * tile + 5):
+        sizes = [tile - 1, tile, 3 * tile + 5]
+        if var["max_n"] < 1 << 17:  # one CTA, one cluster: the work follows the length
+            sizes += [2, 33, var["threads"] + 1, 5 * var["threads"] - 1,
+                      8 * var["threads"] + 1, var["max_n"]]
+        for n in sorted(s for s in sizes if s <= var["max_n"]):
             v = inputs.values(dtype, n) if pairs else None
             for name, k in (("uniform", inputs.keys(dtype, "uniform", n)),
                             ("few", inputs.keys(dtype, "uniform", n) & dtype(0x0303)),
@@ -74,5 +78,32 @@ def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
                 if not pairs and not mirror:
                     check(inputs.keys(dtype, "gaussian", n), v, (n, var, "bits"),
                           variant=var["index"], begin_bit=0, end_bit=20)
+    finally:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
+
+
+@pytest.mark.parametrize("mirror", [0, 1])
+@pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
+def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
+    """Empty, one-warp (up to 32), one-CTA (every number of items a thread)
+    and tiled segments, more of them than one round of the planner takes."""
+    rng = np.random.default_rng(7)
+    lengths = [0, 1, 2, 31, 32, 33, 255, 256, 257, 1023, 1025, 2047, 2048, 2049, 3841, 4096, 4097,
+               12000, 0, 30011]
+    lengths += list(rng.integers(0, 70, 9000)) + [5, 0, 4096, 0]
+    off = inputs.offsets_from_lengths(np.asarray(lengths, dtype=np.uint64))
+    n = int(off[-1])
+    kb = np.dtype(dtype).itemsize
+    v = inputs.values(dtype, n) if pairs else None
+    try:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, mirror))
+        for k in (inputs.keys(dtype, "uniform", n), inputs.keys(dtype, "uniform", n) & dtype(0x303)):
+            for begin, end in ((0, 8 * kb), (3, 20)):
+                dk = to_dev(k, torch)
+                dv = to_dev(v, torch) if pairs else None
+                rs.segmented_sort(dk, to_dev(off, torch), dv, begin, end)
+                ek, ev = oracle.segmented_sort(k, v, off, begin_bit=begin, end_bit=end)
+                assert np.array_equal(from_dev(dk, dtype), ek), (begin, end)
+                assert not pairs or np.array_equal(from_dev(dv, dtype), ev), (begin, end)
     finally:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
