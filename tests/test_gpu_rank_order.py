@@ -35,6 +35,23 @@ def check(k, v, what, **kw):
     assert v is None or np.array_equal(gv, ev), what
 
 
+def merge_via_abi(k, v, kb, vb):
+    n = k.shape[0]
+    dk = to_dev(k, torch)
+    ka = torch.empty_like(dk)
+    dv = to_dev(v, torch) if vb else None
+    va = torch.empty_like(dv) if vb else None
+    st, need = rs.rs_merge_workspace_bytes(kb, vb, n)
+    rs.check(st)
+    ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
+    st, alt = rs.rs_merge_sort(kb, vb, dk.data_ptr(), dv.data_ptr() if vb else None,
+                               ka.data_ptr(), va.data_ptr() if vb else None, n, ws.data_ptr(),
+                               ws.numel(), torch.cuda.current_stream().cuda_stream)
+    rs.check(st)
+    return (from_dev(ka if alt else dk, k.dtype).reshape(k.shape),
+            from_dev(va if alt else dv, v.dtype) if vb else None)
+
+
 @pytest.fixture
 def mirrored():
     rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 1))
@@ -105,5 +122,31 @@ def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
                 ek, ev = oracle.segmented_sort(k, v, off, begin_bit=begin, end_bit=end)
                 assert np.array_equal(from_dev(dk, dtype), ek), (begin, end)
                 assert not pairs or np.array_equal(from_dev(dv, dtype), ev), (begin, end)
+    finally:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
+
+
+@pytest.mark.parametrize("mirror", [0, 1])
+@pytest.mark.parametrize("kb,vb", [(4, 0), (4, 4), (8, 0), (8, 8), (16, 0), (16, 8)])
+def test_merge_tiles_by_bytes(kb, vb, mirror):
+    """The merge sort's tiles: bytes that are the same in a whole tile are
+    left out, few-valued ones repeat in every warp."""
+    rng = np.random.default_rng(3)
+    words = max(1, kb // 8)
+    dt = np.uint32 if kb == 4 else np.uint64
+    try:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, mirror))
+        for n in (2, 33, 4095, 4096, 4097, 3 * 4096 + 77):
+            for mask in (0, 0x30000, 0xff00ff00, None):
+                k = rng.integers(0, np.iinfo(dt).max, (n, words), dtype=dt, endpoint=True)
+                if mask is not None:
+                    k &= dt(mask)
+                k = k if words > 1 else k[:, 0]
+                vdt = np.uint32 if vb == 4 else np.uint64
+                v = np.arange(n, dtype=vdt) if vb else None
+                gk, gv = merge_via_abi(k, v, kb, vb)
+                ek, ev = oracle.sort_wide(k, v) if kb == 16 else oracle.lsd_sort(k, v)
+                assert np.array_equal(gk, ek), (n, mask)
+                assert not vb or np.array_equal(gv, ev), (n, mask)
     finally:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
