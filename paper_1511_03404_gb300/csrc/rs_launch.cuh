@@ -63,7 +63,7 @@ struct OnesweepSort {
     const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), UP_THREADS, max_smem);
     if (occ <= 0) return cudaErrorInvalidConfiguration;
     const int smem = passes * RADIX * SLOTS * 4;
-    constexpr uint32_t per_cta = UP_THREADS * (16 / sizeof(K)) * 4;
+    constexpr uint32_t per_cta = UP_THREADS * (16 / sizeof(K));  // a vector a thread, until the GPU is full
     const uint32_t want = (a.n + per_cta - 1) / per_cta;
     const uint32_t grid =
         std::max(1u, std::min(uint32_t(device_info().sms * occ), want));
