@@ -73,6 +73,38 @@ int prepare_kernel(const void* func, int threads, int smem_bytes) {
   return blocks;
 }
 
+int prepare_cluster(const void* func, int threads, int smem_bytes, int want) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, int> cache;  // (func, device) -> CTAs
+  if (want <= 8) return want;
+  const DeviceInfo& di = device_info();
+  std::lock_guard<std::mutex> g(mu);
+  auto key = std::make_pair(func, di.device);
+  auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  int got = 8;
+  if (cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+      cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(want));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = size_t(smem_bytes);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(want);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, func, &cfg) == cudaSuccess && clusters > 0)
+      got = want;
+  }
+  cudaGetLastError();
+  cache[key] = got;
+  return got;
+}
+
 // ------------------------------------------------- debug bounds checks
 
 namespace {

@@ -74,7 +74,7 @@ struct ClusterSmem {
   static constexpr int WARPS = THREADS / 32;
   static constexpr int SLICE = THREADS * ITEMS;  // the largest
   static constexpr int KB = int(sizeof(K));
-  static constexpr int MAX_CL = 8;
+  static constexpr int MAX_CL = 16;
   static constexpr int WH = 0;                             // u32 [2][WARPS][RADIX], by pass parity
   static constexpr int CNT = WH + 2 * WARPS * RADIX * 4;   // u32 [MAX_CL][RADIX] every CTA's counts
   static constexpr int BASE = CNT + MAX_CL * RADIX * 4;    // u32 [RADIX] global digit bases

@@ -58,6 +58,10 @@ const DeviceInfo& device_info();
 // (once per device) and return its resident CTAs per SM at `threads`.
 int prepare_kernel(const void* func, int threads, int smem_bytes);
 
+// The largest cluster of `want` or 8 (the portable size) CTAs of a prepared
+// kernel that the current device can hold (once per device).
+int prepare_cluster(const void* func, int threads, int smem_bytes, int want);
+
 // Whether digit passes use programmatic dependent launch (on unless the
 // environment sets RS_NO_PDL, read once; a diagnostic switch).
 bool pdl_enabled();

@@ -22,6 +22,7 @@ const Variant* variants_kv32(int* count) {
       OnesweepSort<uint32_t, 4, 8, 256, 26, 3, true>::describe(),
       OnesweepSort<uint32_t, 4, 8, 384, 26, 2, true>::describe(),
       OnesweepSort<uint32_t, 4, 8, 512, 19, 2, true>::describe(),
+      ClusterSort<uint32_t, 4, 8, 512, 16, 16>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

@@ -243,14 +243,16 @@ struct FusedSort {
 };
 
 // The whole sort in one thread-block cluster of up to CL CTAs
-// (k_cluster_sort): arrays of up to CL x THREADS x ITEMS elements stay in
-// the cluster's shared memory for every pass.
+// (k_cluster_sort): arrays of up to 8 x THREADS x ITEMS elements stay in the
+// cluster's shared memory for every pass.
+// CL above 8 is not portable: where the device cannot hold such a cluster, 8
+// CTAs take the same arrays with twice the items each.
 template <class K, int VB, int R, int THREADS, int ITEMS, int CL>
 struct ClusterSort {
   static constexpr int SLICE = THREADS * ITEMS;
-  static_assert(CL >= 1 && CL <= ClusterSmem<K, R, THREADS, ITEMS, true>::MAX_CL,
-                "portable cluster sizes");
-  static_assert(CL * SLICE <= 65536, "positions fit 16 bits");
+  static constexpr int MAX_N = 8 * SLICE;
+  static_assert(CL >= 1 && CL <= ClusterSmem<K, R, THREADS, ITEMS, true>::MAX_CL, "cluster sizes");
+  static_assert(MAX_N <= 65536, "positions fit 16 bits");
 
   static size_t workspace(uint32_t, int) { return 0; }
 
@@ -261,9 +263,11 @@ struct ClusterSort {
     auto kern = &k_cluster_sort<K, VB, R, THREADS, ITEMS, INDEX>;
     if (prepare_kernel(reinterpret_cast<const void*>(kern), THREADS, S::BYTES) <= 0)
       return cudaErrorInvalidConfiguration;
-    if (a.n < 1 || a.n > uint32_t(CL) * SLICE) return cudaErrorInvalidValue;
+    if (a.n < 1 || a.n > uint32_t(MAX_N)) return cudaErrorInvalidValue;
     // every CTA of the cluster takes part, whatever the length
-    uint32_t slice = (a.n + CL * THREADS - 1) / (CL * THREADS) * THREADS;
+    const uint32_t cl =
+        uint32_t(prepare_cluster(reinterpret_cast<const void*>(kern), THREADS, S::BYTES, CL));
+    uint32_t slice = (a.n + cl * THREADS - 1) / (cl * THREADS) * THREADS;
     const unsigned ncta = (a.n + slice - 1) / slice;
     Ctrl* ctrl = (a.ws != nullptr && a.ws_bytes >= sizeof(Ctrl)) ? static_cast<Ctrl*>(a.ws)
                                                                   : nullptr;
@@ -308,7 +312,7 @@ struct ClusterSort {
     v.radix_bits = R;
     v.threads = THREADS;
     v.items = ITEMS;
-    v.max_n = uint32_t(CL) * uint32_t(SLICE);
+    v.max_n = uint32_t(MAX_N);
     v.workspace = &workspace;
     v.run = &run;
     v.count = nullptr;
