@@ -22,7 +22,7 @@ const Variant* variants_k32(int* count) {
       OnesweepSort<uint32_t, 0, 8, 256, 45, 2, true>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 31, 3, true>::describe(),
       OnesweepSort<uint32_t, 0, 8, 384, 31, 2, true>::describe(),
-      OnesweepSort<uint32_t, 0, 8, 512, 23, 2, true>::describe(),
+      OnesweepSort<uint32_t, 0, 8, 256, 51, 2, true>::describe(),
       ClusterSort<uint32_t, 0, 8, 512, 16, 16>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));

@@ -909,8 +909,14 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   K key[INDEX ? 1 : ITEMS];
   uint32_t dig[INDEX ? (ITEMS + 3) / 4 : 1];
   // in batches, so that a batch's loads, atomics and stores each go back to
-  // back: one after another per item they would wait on one another
-  constexpr int BATCH = ITEMS < 9 ? ITEMS : 9;
+  // back: one after another per item they would wait on one another.  Three
+  // at a time where many tiles compete for the pipe (nine: u32 pairs at 2^26
+  // 1.088 ms instead of 1.010, u64 pairs 3.68 instead of 3.46; one: 1.110 and
+  // 3.45), nine to count and stage where a tile is alone on its SM (2^18 u32
+  // keys 41.4 -> 39.6 us).
+  constexpr int MOST = PERSIST ? 3 : 9;
+  constexpr int BATCH = ITEMS < MOST ? ITEMS : MOST;
+  constexpr int OUT_BATCH = ITEMS < 3 ? ITEMS : 3;
   auto count = [&](auto FULL) __attribute__((always_inline)) {
     const uint32_t shift = t.shift, mask = t.mask;
     const bool xin = t.xin;
@@ -1086,6 +1092,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   // registers across the branch and spilled
   uint32_t bad = 0u;
   uint32_t dst[VB > 0 ? ITEMS : 1];  // the values' destinations
+  uint32_t places[VB > 0 ? (ITEMS + 1) / 2 : 1];  // and places in the tile, two a word
   {
     const uint32_t shift = t.shift, mask = t.mask;
     const bool xout = t.xout;
@@ -1096,23 +1103,25 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
     // so that the bounds checks must drop the stores (0 otherwise)
     const uint32_t dbg_push = (kDebugChecks && int(tile) == t.bad_tile) ? n : 0u;
 #pragma unroll
-    for (int s0 = 0; s0 < ITEMS; s0 += BATCH) {
-      K k[BATCH];
-      uint32_t g[BATCH];
-      [[maybe_unused]] uint32_t at[BATCH];
+    for (int s0 = 0; s0 < ITEMS; s0 += OUT_BATCH) {
+      K k[OUT_BATCH];
+      uint32_t g[OUT_BATCH];
+      [[maybe_unused]] uint32_t at[OUT_BATCH];
 #pragma unroll
-      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+      for (int s = s0; s < ITEMS && s < s0 + OUT_BATCH; ++s) {
         const uint32_t i = uint32_t(s * THREADS + tid);
         if constexpr (INDEX) {
           at[s - s0] = s_idx[i];
           bad += at[s - s0] > uint32_t(s_idx[i + 1]) ? 1u : 0u;
+          if constexpr (VB > 0)
+            places[s / 2] = s & 1 ? places[s / 2] | at[s - s0] << 16 : at[s - s0];
         } else {
           k[s - s0] = s_out[i];
           bad |= (k[s - s0] & upto) > (s_out[i + 1] & upto) ? 1u : 0u;
         }
       }
 #pragma unroll
-      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+      for (int s = s0; s < ITEMS && s < s0 + OUT_BATCH; ++s) {
         if constexpr (INDEX) k[s - s0] = s_kin[at[s - s0]];
         g[s - s0] = s_gbase[digit_of(k[s - s0], shift, mask)] + uint32_t(s * THREADS + tid) +
                     dbg_push;
@@ -1120,10 +1129,10 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
       if (xout) {  // the last pass that moves data writes the keys back untransformed
         const KeyXf<K> xf = t.xf;
 #pragma unroll
-        for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) k[s - s0] = xf_inv(k[s - s0], xf);
+        for (int s = s0; s < ITEMS && s < s0 + OUT_BATCH; ++s) k[s - s0] = xf_inv(k[s - s0], xf);
       }
 #pragma unroll
-      for (int s = s0; s < ITEMS && s < s0 + BATCH; ++s) {
+      for (int s = s0; s < ITEMS && s < s0 + OUT_BATCH; ++s) {
         const bool in = uint32_t(s * THREADS + tid) < tile_len;
         if (in && dbg_ok(g[s - s0], n, kSiteKeyScatter)) kdst[g[s - s0]] = k[s - s0];
         if constexpr (VB > 0) dst[s] = g[s - s0];
@@ -1205,7 +1214,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
 #pragma unroll
       for (int s = 0; s < ITEMS; ++s) {
         const uint32_t i = uint32_t(s * THREADS + tid);
-        const V v = s_vin[s_idx[i]];
+        const V v = s_vin[s & 1 ? places[s / 2] >> 16 : places[s / 2] & 0xffffu];
         if (i < tile_len && dbg_ok(dst[s], n, kSiteValScatter)) vdst[dst[s]] = v;
       }
     }
