@@ -6,14 +6,21 @@
 //      keys (shared counters, then one global add per digit), and clears
 //      the look-back words;
 //   -- grid barrier --
-//   2. in every CTA, the exclusive scans and the set of passes that move
-//      data (the same rule as the upsweep's last CTA), kept in shared memory;
-//   3. each moving pass: tiles taken from the pass's counter and sorted by
-//      the onesweep tile (rank, decoupled look-back, stable scatter), with
-//      L2-coherent loads of the previous pass's output;
+//   2. in every CTA, the exclusive scans (all passes at once) and the set of
+//      passes that move data (the same rule as the upsweep's last CTA), kept
+//      in shared memory;
+//   3. each moving pass: the onesweep tile (rank, look-back, stable scatter)
+//      on L2-coherent loads of the previous pass's output.  An array of no
+//      more tiles than CTAs gives CTA b tile b (all are resident, so that the
+//      look-back makes progress); a larger one takes tiles from the pass's
+//      counter;
 //   -- grid barrier after each pass --
 // Every barrier wait is bounded; a CTA that gives up records
 // RS_ERR_TIMEOUT and returns, and the others' bounded waits end as well.
+//
+// Bound by latency.  A barrier costs about 1.5 us against 2.5 to 3 from one
+// kernel to the next, but scans one pass after another (1.2 us each) and two
+// tile tickets a pass (0.7 us each) had taken more than that back.
 #pragma once
 
 #include <type_traits>
@@ -40,10 +47,11 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* ctrl, uint32_t gen, uint64_t 
                                              uint32_t* s_flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&ctrl->grid_bar, 1u);
+    // release and acquire order the CTA's stores (before the barrier above)
+    // and its later loads; sequentially consistent fences took twice as long
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&ctrl->grid_bar), "r"(1u)
+                 : "memory");
     const bool ok = wait_geq(&ctrl->grid_bar, gen * gridDim.x, ctrl, timeout_ns, 0xffffffffu);
-    __threadfence();
     *s_flag = ok ? 1u : 0u;
   }
   __syncthreads();
@@ -74,15 +82,24 @@ __global__ void __launch_bounds__(THREADS, MINB)
   for (int i = tid; i < passes * RADIX; i += THREADS) s_hist[i] = 0u;
   __syncthreads();
   auto count_all = [&](auto XF) {
-    for (uint32_t i = blockIdx.x * THREADS + tid; i < n; i += gridDim.x * THREADS) {
-      K k = k0[i];
-      if constexpr (decltype(XF)::value) k = xf_fwd(k, xf);
+    constexpr int LOADS = 4;  // in flight per thread
+    const uint32_t stride = gridDim.x * THREADS;
+    for (uint32_t i0 = blockIdx.x * THREADS + tid; i0 < n; i0 += stride * LOADS) {
+      K k[LOADS];
 #pragma unroll
-      for (int p = 0; p < MAXP; ++p) {
-        if (p < passes) {
-          const int lo = begin_bit + p * RADIX_BITS;
-          const uint32_t mask = (1u << min(RADIX_BITS, end_bit - lo)) - 1u;
-          atomicAdd(&s_hist[p * RADIX + int(digit_of(k, uint32_t(lo), mask))], 1u);
+      for (uint32_t u = 0; u < LOADS; ++u)
+        if (i0 + u * stride < n) k[u] = k0[i0 + u * stride];
+#pragma unroll
+      for (uint32_t u = 0; u < LOADS; ++u) {
+        if (i0 + u * stride >= n) break;
+        if constexpr (decltype(XF)::value) k[u] = xf_fwd(k[u], xf);
+#pragma unroll
+        for (int p = 0; p < MAXP; ++p) {
+          if (p < passes) {
+            const int lo = begin_bit + p * RADIX_BITS;
+            const uint32_t mask = (1u << min(RADIX_BITS, end_bit - lo)) - 1u;
+            atomicAdd(&s_hist[p * RADIX + int(digit_of(k[u], uint32_t(lo), mask))], 1u);
+          }
         }
       }
     }
@@ -101,14 +118,34 @@ __global__ void __launch_bounds__(THREADS, MINB)
   uint32_t gen = 1;
   if (!grid_barrier(ctrl, gen, knobs.timeout_ns, s_flag)) return;
 
-  // ---- 2. scans and moving passes, in every CTA
-  uint32_t exec = 0u;
-  for (int p = 0; p < passes; ++p) {
-    const uint32_t c = tid < RADIX ? ld_relaxed(&counts[p * RADIX + tid]) : 0u;
-    const uint32_t e = block_exclusive_scan<THREADS>(c, s_tot);
-    if (tid < RADIX) s_off[p * RADIX + tid] = e;
-    if (!__syncthreads_or(tid < RADIX && c == n)) exec |= 1u << p;
+  // ---- 2. scans and moving passes, in every CTA: a digit a thread, all
+  // passes at once
+  static_assert(THREADS >= RADIX && THREADS / 32 <= 32, "one thread per digit");
+  const int lane = tid & 31, warp = tid >> 5;
+  uint32_t* s_sum = s_hist;  // [MAXP][32] the warps' sums (the histograms are added up)
+  uint32_t cnt[MAXP], inc[MAXP];
+  uint32_t one = 0u;  // passes in which my digit holds every key
+#pragma unroll
+  for (int p = 0; p < MAXP; ++p)
+    cnt[p] = p < passes && tid < RADIX ? ld_relaxed(&counts[p * RADIX + tid]) : 0u;
+#pragma unroll
+  for (int p = 0; p < MAXP; ++p) {
+    if (p < passes && tid < RADIX && cnt[p] == n) one |= 1u << p;
+    inc[p] = warp_inclusive_scan(cnt[p], lane);
+    if (lane == 31) s_sum[p * 32 + warp] = inc[p];
   }
+  one = __reduce_or_sync(kFull, one);
+  if (tid == 0) *s_flag = 0u;
+  __syncthreads();
+  if (lane == 0 && one != 0u) atomicOr(s_flag, one);
+#pragma unroll
+  for (int p = 0; p < MAXP; ++p) {
+    const uint32_t before =
+        __reduce_add_sync(kFull, lane < THREADS / 32 && lane < warp ? s_sum[p * 32 + lane] : 0u);
+    if (p < passes && tid < RADIX) s_off[p * RADIX + tid] = before + inc[p] - cnt[p];
+  }
+  __syncthreads();
+  uint32_t exec = ~*s_flag & ((1u << passes) - 1u);
   if ((__popc(exec) & 1) != (passes & 1)) {  // keep the result in buffer (passes mod 2)
     const uint32_t skipped = ~exec & ((1u << passes) - 1u);
     exec |= skipped & (0u - skipped);
@@ -131,17 +168,24 @@ __global__ void __launch_bounds__(THREADS, MINB)
       t->bad_tile = -1;
     }
     if (rec) ctrl->t_pass[p][0] = stat_now(ctrl);
-    for (;;) {
-      __syncthreads();  // the previous tile is done with s_misc
-      if (tid == 0) {
-        s_misc[2] = ld_relaxed(&ctrl->error);
-        s_misc[0] = s_misc[2] ? tiles : atomicAdd(&ctrl->tile_counter[p], 1u);
+    if (tiles <= gridDim.x) {
+      __syncthreads();  // the operands are in place
+      if (blockIdx.x < tiles)
+        onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, true>(blockIdx.x, ctrl,
+                                                                      knobs.timeout_ns, smem);
+    } else {
+      for (;;) {
+        __syncthreads();  // the previous tile is done with s_misc
+        if (tid == 0) {
+          s_misc[2] = ld_relaxed(&ctrl->error);
+          s_misc[0] = s_misc[2] ? tiles : atomicAdd(&ctrl->tile_counter[p], 1u);
+        }
+        __syncthreads();
+        const uint32_t tile = s_misc[0];
+        if (tile >= tiles) break;  // CTA-uniform
+        onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, true>(tile, ctrl,
+                                                                      knobs.timeout_ns, smem);
       }
-      __syncthreads();
-      const uint32_t tile = s_misc[0];
-      if (tile >= tiles) break;  // CTA-uniform
-      onesweep_tile<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX, true>(tile, ctrl, knobs.timeout_ns,
-                                                                    smem);
     }
     ++gen;
     if (!grid_barrier(ctrl, gen, knobs.timeout_ns, s_flag)) return;

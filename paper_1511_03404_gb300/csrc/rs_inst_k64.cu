@@ -20,6 +20,7 @@ const Variant* variants_k64(int* count) {
       OnesweepSort<uint64_t, 0, 8, 256, 11, 4, true>::describe(),
       OnesweepSort<uint64_t, 0, 8, 512, 11, 2, true>::describe(),
       ClusterSort<uint64_t, 0, 8, 512, 16, 16>::describe(),
+      FusedSort<uint64_t, 0, 8, 256, 8, 4>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;
