@@ -31,6 +31,12 @@ TYPES = ((4, 0), (4, 4), (8, 0), (8, 8))
 SIZES = tuple(sorted({2**e for e in range(12, 27)} | {2**e + 2**(e - 1) for e in range(12, 26)}))
 
 
+# one launch: preferred within 2 %, which is what a run's times scatter by, as
+# the host is free earlier (a launch costs it about 4 us, a multi-launch sort
+# of 32-bit keys has six)
+ONE_LAUNCH = (1, 3, 4)
+
+
 def _time_variant(torch, kb, vb, n, variant, keys, vals, reps):
     dk = torch.empty_like(keys)
     ka = torch.empty_like(keys)
@@ -62,7 +68,7 @@ def _time_variant(torch, kb, vb, n, variant, keys, vals, reps):
     return statistics.median(times)
 
 
-def tune(sizes=SIZES, types=TYPES, reps=5, log=print, verbose=False) -> dict:
+def tune(sizes=SIZES, types=TYPES, reps=11, log=print, verbose=False) -> dict:
     import torch
 
     rs.load()
@@ -92,7 +98,8 @@ def tune(sizes=SIZES, types=TYPES, reps=5, log=print, verbose=False) -> dict:
                     continue
                 if ms is not None:
                     results[i] = ms
-            best = min(results, key=results.get)
+            best = min(results, key=lambda i: results[i] * (1.0 if infos[i]["kind"] in ONE_LAUNCH
+                                                            else 1.02))
             entries.append({"key_bytes": kb, "val_bytes": vb, "n_max": n, "variant": best,
                             "ms": results[best],
                             "gkeys_per_s": n / (results[best] / 1e3) / 1e9,
@@ -129,7 +136,7 @@ def main(argv=None):
     ap.add_argument("--verbose", action="store_true", help="name each variant before timing it")
     args = ap.parse_args(argv)
     sizes = (2**12, 2**16, 2**20, 2**24) if args.quick else SIZES
-    table = tune(sizes=sizes, reps=3 if args.quick else 5, verbose=args.verbose)
+    table = tune(sizes=sizes, reps=3 if args.quick else 11, verbose=args.verbose)
     with open(args.out, "w") as f:
         json.dump(table, f, indent=1)
         f.write("\n")

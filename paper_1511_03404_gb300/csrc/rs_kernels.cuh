@@ -1469,12 +1469,15 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
       }
       __syncthreads();
       // per digit: the count, its start, and from there the warps' starts
-      uint32_t c[WARPS], cnt = 0u;
+      // (32 warps' counts are read twice: in registers they would spill)
+      constexpr bool KEEP = WARPS <= 16;
+      uint32_t c[KEEP ? WARPS : 1], cnt = 0u;
       if (tid < RADIX) {
 #pragma unroll
         for (int w = 0; w < WARPS; ++w) {
-          c[w] = s_wh[w * RADIX + tid];
-          cnt += c[w];
+          const uint32_t x = s_wh[w * RADIX + tid];
+          if constexpr (KEEP) c[w] = x;
+          cnt += x;
         }
       }
       const uint32_t inc = warp_inclusive_scan(cnt, lane);
@@ -1484,10 +1487,13 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
         uint32_t run =
             __reduce_add_sync(kFull, lane < RADIX / 32 && lane < warp ? s_tot[lane] : 0u) + inc -
             cnt;
-#pragma unroll
+#pragma unroll(KEEP ? WARPS : 8)
         for (int w = 0; w < WARPS; ++w) {
+          uint32_t x;
+          if constexpr (KEEP) x = c[w];
+          else x = s_wh[w * RADIX + tid];
           s_wh[w * RADIX + tid] = run;
-          run += c[w];
+          run += x;
         }
       }
       __syncthreads();

@@ -1,6 +1,6 @@
 // Host side of the batched segmented sort (each of the four data types):
 // workspace sizing and the launch sequence memset -> k_seg_plan ->
-// k_seg_small -> k_seg_hist -> k_seg_persistent, all on the caller's stream
+// k_seg_small (short, then medium) -> k_seg_hist -> k_seg_persistent, all on the caller's stream
 // (capturable in a CUDA graph).
 #include <algorithm>
 
@@ -14,10 +14,11 @@ namespace {
 
 // MINB: resident CTAs per SM the short-segment kernel is compiled for (its
 // register budget); PASS_MINB: the same for the pass kernel.
-template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS, int MINB = 4, int PASS_MINB = MINB>
+template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS, int MEDIUM_ITEMS, int MINB = 4,
+          int PASS_MINB = MINB>
 struct SegSort {
   using C = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, SMALL_ITEMS>;
-  static constexpr int PLAN_THREADS = 256;
+  static constexpr int PLAN_THREADS = 256, MEDIUM_THREADS = 1024;
 
   static SegLayout layout(size_t n, size_t nseg, int passes) {
     return seg_layout(n, nseg, passes, R, C::TILE, C::CHUNK);
@@ -43,6 +44,17 @@ struct SegSort {
     }
     const int occ_small = prepare_kernel(reinterpret_cast<const void*>(small), THREADS, smem_small);
     if (occ_small <= 0) return cudaErrorInvalidConfiguration;
+    auto medium = &k_seg_small<K, VB, R, MEDIUM_THREADS, MEDIUM_ITEMS, true, 1, true>;
+    int smem_medium = SmallSmem<K, VB, R, MEDIUM_THREADS, MEDIUM_ITEMS, true>::BYTES;
+    if constexpr (VB == 0) {
+      if (begin_bit == 0 && end_bit == 8 * int(sizeof(K))) {
+        medium = &k_seg_small<K, VB, R, MEDIUM_THREADS, MEDIUM_ITEMS, false, 1, true>;
+        smem_medium = SmallSmem<K, VB, R, MEDIUM_THREADS, MEDIUM_ITEMS, false>::BYTES;
+      }
+    }
+    const int occ_medium =
+        prepare_kernel(reinterpret_cast<const void*>(medium), MEDIUM_THREADS, smem_medium);
+    if (occ_medium <= 0) return cudaErrorInvalidConfiguration;
     auto hist = &k_seg_hist<K, R, C::HIST_THREADS, C::MAXP, C::HIST_SLOTS, C::CHUNK, C::TILE,
                             CHUNK_TILES, C::HIST_MINB>;
     const int occ_hist =
@@ -65,6 +77,7 @@ struct SegSort {
     a.passes = passes;
     a.ctrl = ctrl;
     a.small_ids = reinterpret_cast<const uint32_t*>(w + L.small_ids);
+    a.medium_ids = reinterpret_cast<const uint32_t*>(w + L.medium_ids);
     a.descs = reinterpret_cast<const SegDesc*>(w + L.descs);
     a.tdesc = reinterpret_cast<TileDesc*>(w + L.tdesc);
     a.chunk_seg = reinterpret_cast<const uint32_t*>(w + L.chunk_seg);
@@ -78,8 +91,10 @@ struct SegSort {
     using V = ValT<VB>;
     k_seg_plan<PLAN_THREADS, C::RADIX>
         <<<unsigned((nseg + PLAN_THREADS - 1) / PLAN_THREADS), PLAN_THREADS, 0, s>>>(
-            n, uint32_t(C::SMALL_TILE), uint32_t(C::TILE), uint32_t(C::CHUNK), L.chunks_max,
-            reinterpret_cast<uint32_t*>(w + L.small_ids), reinterpret_cast<SegDesc*>(w + L.descs),
+            n, uint32_t(C::SMALL_TILE), uint32_t(MEDIUM_THREADS * MEDIUM_ITEMS), uint32_t(C::TILE),
+            uint32_t(C::CHUNK), L.chunks_max, reinterpret_cast<uint32_t*>(w + L.small_ids),
+            reinterpret_cast<uint32_t*>(w + L.medium_ids),
+            reinterpret_cast<SegDesc*>(w + L.descs),
             reinterpret_cast<uint32_t*>(w + L.chunk_seg), a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -94,15 +109,36 @@ struct SegSort {
         unsigned(std::max<size_t>(1, std::min<size_t>(sms * occ_hist, L.chunks_max)));
     const unsigned grid_small =
         unsigned(std::max<size_t>(1, std::min<size_t>(nseg, sms * occ_small)));
+    const unsigned grid_medium = unsigned(std::max<size_t>(
+        1, std::min<size_t>(sms * occ_medium, n / (size_t(C::SMALL_TILE) + 1))));
     prof_before(s);
-    small<<<grid_small, THREADS, smem_small, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
-                                                 static_cast<K*>(keys_alt),
-                                                 static_cast<V*>(vals_alt), a);
-    hist<<<grid_hist, C::HIST_THREADS,
-           passes * C::RADIX * C::HIST_SLOTS * 4, s>>>(static_cast<const K*>(keys), a);
-    kern<<<grid, THREADS, smem, s>>>(static_cast<K*>(keys), static_cast<V*>(vals),
-                                         static_cast<K*>(keys_alt), static_cast<V*>(vals_alt), a);
-    e = cudaGetLastError();
+    // each kernel waits for the one before it (pdl_wait), so that it may be
+    // launched as that one exits
+    auto launch = [&](auto kernel, unsigned blocks, int threads, int smem_bytes, auto... args) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(blocks);
+      cfg.blockDim = dim3(unsigned(threads));
+      cfg.dynamicSmemBytes = size_t(smem_bytes);
+      cfg.stream = s;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = pdl_enabled() ? 1 : 0;
+      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    };
+    K *k0 = static_cast<K*>(keys), *k1 = static_cast<K*>(keys_alt);
+    V *v0 = static_cast<V*>(vals), *v1 = static_cast<V*>(vals_alt);
+    launch(small, grid_small, THREADS, smem_small, k0, v0, k1, v1, a);
+    // (no segment is longer than the array)
+    if (n > size_t(C::SMALL_TILE))
+      launch(medium, grid_medium, MEDIUM_THREADS, smem_medium, k0, v0, k1, v1, a);
+    if (n > size_t(MEDIUM_THREADS) * MEDIUM_ITEMS) {
+      launch(hist, grid_hist, C::HIST_THREADS, passes * C::RADIX * C::HIST_SLOTS * 4,
+             static_cast<const K*>(k0), a);
+      launch(kern, grid, THREADS, smem, k0, v0, k1, v1, a);
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
     prof_after(s, RS_KERNEL_SEGMENTED,
                double(n) * (sizeof(K) + passes * 2.0 * (sizeof(K) + VB)));
     return e;
@@ -111,14 +147,14 @@ struct SegSort {
 
 // u32 pairs: pass tiles of 256 x 45 keys ranked in half-warp units, two CTAs
 // per SM; short segments up to 4096 elements sorted whole by one CTA
-using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 41, 12, 16, 4, 2>;
+using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 41, 12, 16, 16, 4, 2>;
 // u32 keys: 256 x 37 keys in half-warp units, two CTAs per SM; short
 // segments up to 4096
-using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 45, 14, 16, 4, 2>;
+using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 45, 14, 16, 16, 4, 2>;
 // 64-bit keys and pairs: 256 x 23 elements in half-warp units, two CTAs per
 // SM; short segments up to 2048 (pairs: that kernel at three CTAs per SM)
-using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 8, 4, 2>;
-using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 8, 3, 2>;
+using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 8, 8, 4, 2>;
+using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 8, 8, 3, 2>;
 
 bool seg_types(int kb, int vb) { return (kb == 4 || kb == 8) && (vb == 0 || vb == kb); }
 

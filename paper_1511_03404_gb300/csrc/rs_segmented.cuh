@@ -6,7 +6,8 @@
 //                     one CTA, long ones are tiled), numbers the work items
 //                     and maps every histogram chunk to its segment.
 //   k_seg_small       short segments, each sorted whole in one CTA's shared
-//                     memory (every pass) or by one warp;
+//                     memory (every pass) or by one warp; once more, with
+//                     larger CTAs, for the medium ones;
 //   k_seg_hist        the digit histograms of the long segments, chunk by
 //                     chunk; each segment's last chunk scans them and writes
 //                     the descriptors of the segment's pass tiles;
@@ -65,12 +66,14 @@ enum SegCtrlField {
   kNTiles = 3,   // pass tiles of all long segments (one pass)
   kNChunks = 4,  // histogram chunks of all long segments
   kNTiny = 6,    // segments of 1 to 32 elements
-  kSmallQueue = 7  // work-queue ticket of the short segments
+  kSmallQueue = 7,  // work-queue ticket of the short segments
+  kNMedium = 8,
+  kMediumQueue = 9  // and of the medium ones
 };
 constexpr uint32_t kTinyMax = 32;
 
 struct SegLayout {
-  size_t small_ids, descs, tdesc, chunk_seg, state, counts, offsets, status, total;
+  size_t small_ids, medium_ids, descs, tdesc, chunk_seg, state, counts, offsets, status, total;
   size_t tiles_max, chunks_max;
 };
 
@@ -84,7 +87,8 @@ inline SegLayout seg_layout(size_t n, size_t nseg, int passes, int radix_bits, i
   L.counts = align_up(L.state + nseg * kSegStateWords * 4, 256);
   L.offsets = align_up(L.counts + nseg * passes * radix * 4, 256);
   L.small_ids = align_up(L.offsets + nseg * passes * radix * 4, 256);
-  L.descs = align_up(L.small_ids + nseg * 4, 256);
+  L.medium_ids = align_up(L.small_ids + nseg * 4, 256);
+  L.descs = align_up(L.medium_ids + nseg * 4, 256);
   L.tdesc = align_up(L.descs + nseg * sizeof(SegDesc), 256);
   L.chunk_seg = align_up(L.tdesc + L.tiles_max * sizeof(TileDesc), 256);
   L.status = align_up(L.chunk_seg + L.chunks_max * 4, 256);
@@ -97,6 +101,7 @@ struct SegArgs {
   int begin_bit, end_bit, passes;
   Ctrl* ctrl;
   const uint32_t* small_ids;
+  const uint32_t* medium_ids;
   const SegDesc* descs;
   TileDesc* tdesc;    // [tiles_max]
   const uint32_t* chunk_seg;
@@ -109,9 +114,10 @@ struct SegArgs {
   Knobs knobs;
 };
 
-// Numbers the work, one segment a thread.  Segments longer than small_max are
+// Numbers the work, one segment a thread.  Segments longer than medium_max are
 // "long"; of the others, those of 1 to 32 elements are "tiny" (listed from the
-// end of small_ids), the rest "small"; empty ones are left out.  The order
+// end of small_ids), those of up to small_max "small", the rest "medium"; empty
+// ones are left out.  The order
 // inside the lists is of no consequence, so each CTA takes its places from
 // global counters: with one CTA scanning all segments in order, 20,000 of them
 // took 87 us.  The state of long segments, and the digit counts of those of
@@ -120,11 +126,11 @@ struct SegArgs {
 // do nothing.
 template <int THREADS, int RADIX>
 __global__ void __launch_bounds__(THREADS)
-    k_seg_plan(uint64_t n, uint32_t small_max, uint32_t tile, uint32_t chunk, uint64_t chunks_max,
-               uint32_t* __restrict__ small_ids, SegDesc* __restrict__ descs,
-               uint32_t* __restrict__ chunk_seg, SegArgs a) {
-  constexpr int COUNTS = 5, WARPS = THREADS / 32;
-  const int field[COUNTS] = {kNTiny, kNSmall, kNLarge, kNTiles, kNChunks};
+    k_seg_plan(uint64_t n, uint32_t small_max, uint32_t medium_max, uint32_t tile, uint32_t chunk, uint64_t chunks_max,
+               uint32_t* __restrict__ small_ids, uint32_t* __restrict__ medium_ids,
+               SegDesc* __restrict__ descs, uint32_t* __restrict__ chunk_seg, SegArgs a) {
+  constexpr int COUNTS = 6, WARPS = THREADS / 32;
+  const int field[COUNTS] = {kNTiny, kNSmall, kNLarge, kNTiles, kNChunks, kNMedium};
   __shared__ uint32_t s_tot[COUNTS][WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t s = uint64_t(blockIdx.x) * THREADS + tid;
@@ -137,10 +143,10 @@ __global__ void __launch_bounds__(THREADS)
     if (to < from || to > n || to - from > uint64_t((1u << 30) - 1u)) bad = true;
     else len = uint32_t(to - from);
   }
-  const bool tiny = len >= 1u && len <= kTinyMax, lng = len > small_max;
-  const bool small = len > kTinyMax && !lng;
+  const bool tiny = len >= 1u && len <= kTinyMax, lng = len > medium_max;
+  const bool small = len > kTinyMax && len <= small_max, medium = len > small_max && !lng;
   const uint32_t nt = lng ? (len + tile - 1u) / tile : 0u, nc = lng ? (len + chunk - 1u) / chunk : 0u;
-  const uint32_t mine[COUNTS] = {tiny, small, lng, nt, nc};
+  const uint32_t mine[COUNTS] = {tiny, small, lng, nt, nc, medium};
   uint32_t at[COUNTS];
 #pragma unroll
   for (int q = 0; q < COUNTS; ++q) {
@@ -164,6 +170,7 @@ __global__ void __launch_bounds__(THREADS)
   for (int q = 0; q < COUNTS; ++q) at[q] += s_tot[q][warp];
   const uint64_t slot = tiny ? a.nseg - 1u - at[0] : at[1];
   if ((tiny || small) && dbg_ok(slot, a.nseg, kSiteSegPlan)) small_ids[slot] = uint32_t(s);
+  if (medium && dbg_ok(at[5], a.nseg, kSiteSegPlan)) medium_ids[at[5]] = uint32_t(s);
   const uint32_t li = at[2], c0 = at[4];
   bool map_ok = false;
   if (lng) {
@@ -246,8 +253,12 @@ __device__ __forceinline__ void seg_warp_sort(const K* kin, const ValT<VB>* vin,
 
 // The short segments: those of up to 32 elements one warp each, the others
 // one CTA each, taken from a queue (the next one is asked for while the
-// current one is sorted), so that long and short ones even out.
-template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX, int MINB>
+// current one is sorted), so that long and short ones even out.  MEDIUM: the
+// medium list alone, on CTAs of 1024 threads: one read and one write of a
+// segment instead of a histogram and a tile or two in every pass (20,000
+// log-uniform segments of 2^26 pairs: the tiled passes take 28 % less).
+template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX, int MINB,
+          bool MEDIUM = false>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_seg_small(K* __restrict__ k0, ValT<VB>* __restrict__ v0, K* __restrict__ k1,
                 ValT<VB>* __restrict__ v1, SegArgs a) {
@@ -256,19 +267,22 @@ __global__ void __launch_bounds__(THREADS, MINB)
   const int passes = a.passes;
   K* kout = (passes & 1) ? k1 : k0;  // where the pass count parity puts the result
   ValT<VB>* vout = (passes & 1) ? v1 : v0;
+  pdl_wait();  // the planner (and what is before this kernel) is complete
   if (a.ctrl->error != 0u) return;  // bad offsets: nothing is written
-  const uint32_t n_small = a.ctrl->tile_counter[kNSmall];
-  const uint32_t n_tiny = a.ctrl->tile_counter[kNTiny];
+  constexpr int QUEUE = MEDIUM ? kMediumQueue : kSmallQueue;
+  const uint32_t* ids = MEDIUM ? a.medium_ids : a.small_ids;
+  const uint32_t n_small = a.ctrl->tile_counter[MEDIUM ? kNMedium : kNSmall];
+  const uint32_t n_tiny = MEDIUM ? 0u : a.ctrl->tile_counter[kNTiny];
   const K looked = (a.end_bit - a.begin_bit == 8 * int(sizeof(K)))
                        ? ~K(0)
                        : K(((K(1) << (a.end_bit - a.begin_bit)) - K(1)) << a.begin_bit);
-  if (threadIdx.x == 0) s_next[0] = atomicAdd(&a.ctrl->tile_counter[kSmallQueue], 1u);
+  if (threadIdx.x == 0) s_next[0] = atomicAdd(&a.ctrl->tile_counter[QUEUE], 1u);
   __syncthreads();
   for (uint32_t it = 0;; ++it) {
     const uint32_t i = s_next[it & 1u];
     if (i >= n_small) break;
-    if (threadIdx.x == 0) s_next[(it + 1u) & 1u] = atomicAdd(&a.ctrl->tile_counter[kSmallQueue], 1u);
-    const uint32_t s = a.small_ids[i];
+    if (threadIdx.x == 0) s_next[(it + 1u) & 1u] = atomicAdd(&a.ctrl->tile_counter[QUEUE], 1u);
+    const uint32_t s = ids[i];
     const uint64_t b = a.off[s];
     const uint32_t len = uint32_t(a.off[s + 1] - b);
     cta_sort<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>(k0 + b, v0 + b, kout + b, vout + b, len,
@@ -326,6 +340,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
         atomicAdd(&sh[(p * RADIX + int(digit_of(k, shiftp[p], maskp[p]))) * SLOTS + int(slot)],
                   1u);
   };
+  pdl_wait();
   if (a.ctrl->error != 0u) return;  // bad offsets
   const uint32_t n_chunks = a.ctrl->tile_counter[kNChunks];
   const int words = passes * RADIX * SLOTS;
@@ -492,6 +507,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
   Ctrl* ctrl = a.ctrl;
   const int passes = a.passes;
 
+  pdl_wait();
   const uint32_t n_tiles = ctrl->tile_counter[kNTiles];
   const uint32_t q_end = uint32_t(passes) * n_tiles;
 
