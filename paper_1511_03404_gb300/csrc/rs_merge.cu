@@ -7,8 +7,9 @@
 //               output tile of the merged pair begins in the left run (the
 //               merge path), one warp a tile: 32 probes of the tile's diagonal
 //               at a time;
-//   k_ms_merge  merges one output tile per CTA from the two input ranges its
-//               split delimits.
+//   k_ms_merge  merges one output tile (kOutTile) per CTA from the two input
+//               ranges its split delimits.
+// The merge kernels are launched as the one before exits (pdl_wait).
 // Ties always take the element of the left run, which holds the earlier
 // input positions, so every merge (and the whole sort) is stable.  Values do
 // not take part: 16-bit source positions are sorted and merged, and the values
@@ -24,9 +25,18 @@ namespace rs {
 
 namespace {
 
-constexpr int kMsThreads = 256;  // of a merge
-constexpr int kMsItems = 16;
-constexpr int kTile = kMsThreads * kMsItems;
+constexpr int kMsItems = 16;  // outputs a thread of a merge
+constexpr int kTile = 4096;   // of the tile sort: the first runs
+
+// Threads of a merge CTA, and its output tile.  Few 128-bit tiles fit an SM at
+// once, so that the last wave of an array of a few million is mostly empty:
+// tiles half the size lose half as much (4e6 keys with values, a pass: 54 us ->
+// 51).
+template <class K>
+constexpr int kMsThreads = sizeof(K) == 16 ? 128 : 256;
+template <class K>
+constexpr int kOutTile = kMsThreads<K> * kMsItems;
+constexpr int kOutTileLeast = 128 * kMsItems;
 
 // A 128-bit unsigned key: value = lo + 2^64 * hi (little-endian words).
 struct alignas(16) Key128 {
@@ -106,16 +116,16 @@ __device__ __forceinline__ void merge_items(const K* sk, Run a, Run b, K (&k)[kM
 // positions, the values as loaded.
 template <class K, class V, bool HAS_V>
 struct MsSmem {
-  static constexpr int SLOTS = kTile + kTile / 32;
+  static constexpr int SLOTS = kOutTile<K> + kOutTile<K> / 32;
   static constexpr int KEYS = 0;
   static constexpr int POS = (SLOTS * int(sizeof(K)) + 15) / 16 * 16;
   static constexpr int VALS = POS + (HAS_V ? SLOTS * 2 + 15 : 0) / 16 * 16;
-  static constexpr int BYTES = VALS + (HAS_V ? kTile * int(sizeof(V)) : 0);
+  static constexpr int BYTES = VALS + (HAS_V ? kOutTile<K> * int(sizeof(V)) : 0);
   // resident CTAs to leave registers for: as many as the shared memory takes,
   // up to what 16 keys in registers allow.  (At two, with the registers that
   // allows, merges of 32- and 64-bit keys took 1.4 times as long.)
   static constexpr int FIT = 226 * 1024 / (BYTES + 1024);
-  static constexpr int MOST = sizeof(K) == 4 ? 5 : 4;
+  static constexpr int MOST = sizeof(K) == 4 ? 5 : sizeof(K) == 8 ? 4 : 6;
   static constexpr int MINB = FIT < MOST ? FIT : MOST;
 };
 
@@ -313,14 +323,15 @@ __device__ __forceinline__ uint32_t merge_path_warp(const K* __restrict__ a, uin
 }
 
 // Runs of width w (a multiple of kTile) are merged in pairs; output tile c
-// starts at p = c * kTile inside the pair [base, base + 2w).  split[c] = how
+// starts at p = c * kOutTile inside the pair [base, base + 2w).  split[c] = how
 // many of the pair's left-run elements precede that tile.  One warp a tile.
 template <class K>
 __global__ void k_ms_split(const K* __restrict__ src, uint32_t n, uint32_t w,
                            uint32_t* __restrict__ split, uint32_t tiles) {
+  pdl_wait();
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) / 32u;
   if (c >= tiles) return;
-  const uint64_t p = uint64_t(c) * kTile;
+  const uint64_t p = uint64_t(c) * kOutTile<K>;
   const uint64_t base = p / (2ull * w) * (2ull * w);
   const uint32_t na = uint32_t(min(uint64_t(w), n - base));
   const uint32_t nb = uint32_t(n - base - na < w ? n - base - na : w);
@@ -331,10 +342,10 @@ __global__ void k_ms_split(const K* __restrict__ src, uint32_t n, uint32_t w,
 // Bound by latency: loads, a search of 12 dependent steps, 16 outputs one
 // after another, each a shared-memory read.  2^24 u32 keys a pass: 46 us with
 // the loads one after another and two reads an output, 41 now (u32 pairs 70 ->
-// 55, u64 keys 81 -> 60, 2^22 128-bit keys with values 67 -> 54); the split
+// 55, u64 keys 81 -> 60, 2^22 128-bit keys with values 67 -> 52); the split
 // 10-21 us a pass with one thread a tile, 5-8 now.
 template <class K, class V, bool HAS_V>
-__global__ void __launch_bounds__(kMsThreads, MsSmem<K, V, HAS_V>::MINB) k_ms_merge(const K* __restrict__ src,
+__global__ void __launch_bounds__(kMsThreads<K>, MsSmem<K, V, HAS_V>::MINB) k_ms_merge(const K* __restrict__ src,
                                                             const V* __restrict__ vsrc,
                                                             K* __restrict__ dst,
                                                             V* __restrict__ vdst, uint32_t n,
@@ -345,10 +356,11 @@ __global__ void __launch_bounds__(kMsThreads, MsSmem<K, V, HAS_V>::MINB) k_ms_me
   K* sk = reinterpret_cast<K*>(smem + S::KEYS);
   uint16_t* sp = reinterpret_cast<uint16_t*>(smem + S::POS);
   V* sv = reinterpret_cast<V*>(smem + S::VALS);
+  pdl_wait();
   const uint32_t c = blockIdx.x;
-  const uint64_t p0 = uint64_t(c) * kTile;
-  const uint64_t p1 = min(p0 + kTile, uint64_t(n));
-  const uint64_t base = p0 / (2ull * w) * (2ull * w);  // kTile divides 2w: one pair per CTA
+  const uint64_t p0 = uint64_t(c) * kOutTile<K>;
+  const uint64_t p1 = min(p0 + kOutTile<K>, uint64_t(n));
+  const uint64_t base = p0 / (2ull * w) * (2ull * w);  // kOutTile<K> divides 2w: one pair per CTA
   const uint32_t na = uint32_t(min(uint64_t(w), n - base));
   const uint32_t nb = uint32_t(n - base - na < w ? n - base - na : w);
   const uint32_t d0 = uint32_t(p0 - base), d1 = uint32_t(p1 - base);
@@ -366,7 +378,7 @@ __global__ void __launch_bounds__(kMsThreads, MsSmem<K, V, HAS_V>::MINB) k_ms_me
     V v[HAS_V ? kMsItems : 1];
 #pragma unroll
     for (int t = 0; t < kMsItems; ++t) {
-      const uint32_t i = uint32_t(t * kMsThreads + tid);
+      const uint32_t i = uint32_t(t * kMsThreads<K> + tid);
       const uint64_t at = (i < la ? from_a : from_b) + i;
       if (i < total) {
         k[t] = src[at];
@@ -375,7 +387,7 @@ __global__ void __launch_bounds__(kMsThreads, MsSmem<K, V, HAS_V>::MINB) k_ms_me
     }
 #pragma unroll
     for (int t = 0; t < kMsItems; ++t) {
-      const uint32_t i = uint32_t(t * kMsThreads + tid);
+      const uint32_t i = uint32_t(t * kMsThreads<K> + tid);
       if (i < total) {
         sk[pad(i)] = k[t];
         if constexpr (HAS_V) sv[i] = v[t];
@@ -396,7 +408,7 @@ __global__ void __launch_bounds__(kMsThreads, MsSmem<K, V, HAS_V>::MINB) k_ms_me
   __syncthreads();
 #pragma unroll
   for (int t = 0; t < kMsItems; ++t) {
-    const uint32_t i = uint32_t(t * kMsThreads + tid);
+    const uint32_t i = uint32_t(t * kMsThreads<K> + tid);
     if (i >= total || !dbg_ok(p0 + i, n, kSiteMergeOut)) continue;
     dst[p0 + i] = sk[pad(i)];
     if constexpr (HAS_V) vdst[p0 + i] = sv[sp[pad(i)]];
@@ -407,8 +419,11 @@ template <class K, class V, bool HAS_V>
 struct MergeSort {
   using S = MsSmem<K, V, HAS_V>;
 
-  static uint32_t tiles(size_t n) { return uint32_t((n + kTile - 1) / kTile); }
-  static size_t workspace(size_t n) { return align_up((size_t(tiles(n)) + 1) * 4, 256); }
+  static uint32_t tiles(size_t n) { return uint32_t((n + kOutTile<K> - 1) / kOutTile<K>); }
+  // for every type alike: the smallest tiles
+  static size_t workspace(size_t n) {
+    return align_up(((n + kOutTileLeast - 1) / kOutTileLeast + 1) * 4, 256);
+  }
 
   static cudaError_t run(void* keys, void* vals, void* keys_alt, void* vals_alt, size_t n,
                          void* ws, cudaStream_t s, int* in_alt) {
@@ -416,13 +431,13 @@ struct MergeSort {
     auto merge_k = &k_ms_merge<K, V, HAS_V>;
     using T = MsTileSmem<K>;
     if (prepare_kernel(reinterpret_cast<const void*>(tile_k), T::THREADS, T::BYTES) <= 0 ||
-        prepare_kernel(reinterpret_cast<const void*>(merge_k), kMsThreads, S::BYTES) <= 0)
+        prepare_kernel(reinterpret_cast<const void*>(merge_k), kMsThreads<K>, S::BYTES) <= 0)
       return cudaErrorInvalidConfiguration;
     K* bufk[2] = {static_cast<K*>(keys), static_cast<K*>(keys_alt)};
     V* bufv[2] = {static_cast<V*>(vals), static_cast<V*>(vals_alt)};
     const uint32_t nt = tiles(n);
     prof_before(s);
-    tile_k<<<nt, T::THREADS, T::BYTES, s>>>(bufk[0], bufv[0], bufk[0], bufv[0], uint32_t(n),
+    tile_k<<<unsigned((n + kTile - 1) / kTile), T::THREADS, T::BYTES, s>>>(bufk[0], bufv[0], bufk[0], bufv[0], uint32_t(n),
                                             knobs_now().mirror != 0);
     cudaError_t e = cudaGetLastError();
     prof_after(s, RS_KERNEL_MERGE, 2.0 * double(n) * double(sizeof(K) + (HAS_V ? sizeof(V) : 0)));
@@ -430,11 +445,26 @@ struct MergeSort {
     int cur = 0;
     uint32_t* split = static_cast<uint32_t*>(ws);
     for (uint64_t w = kTile; w < n; w *= 2) {
-      k_ms_split<K><<<(nt + 7) / 8, 256, 0, s>>>(bufk[cur], uint32_t(n), uint32_t(w), split, nt);
+      auto launch = [&](auto kernel, unsigned blocks, int threads, int smem_bytes, auto... args) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(unsigned(threads));
+        cfg.dynamicSmemBytes = size_t(smem_bytes);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = pdl_enabled() ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kernel, args...);
+      };
+      const K* from = bufk[cur];
+      const V* vfrom = bufv[cur];
+      e = launch(&k_ms_split<K>, (nt + 7) / 8, 256, 0, from, uint32_t(n), uint32_t(w), split, nt);
+      if (e != cudaSuccess) return e;
       prof_before(s);
-      merge_k<<<nt, kMsThreads, S::BYTES, s>>>(bufk[cur], bufv[cur], bufk[cur ^ 1],
-                                                bufv[cur ^ 1], uint32_t(n), uint32_t(w), split);
-      e = cudaGetLastError();
+      e = launch(merge_k, nt, kMsThreads<K>, S::BYTES, from, vfrom, bufk[cur ^ 1], bufv[cur ^ 1],
+                 uint32_t(n), uint32_t(w), static_cast<const uint32_t*>(split));
       prof_after(s, RS_KERNEL_MERGE,
                  2.0 * double(n) * double(sizeof(K) + (HAS_V ? sizeof(V) : 0)));
       if (e != cudaSuccess) return e;
