@@ -15,8 +15,8 @@ const Variant* variants_k32(int* count) {
       SmallSort<uint32_t, 0, 8, 1024, 8>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 16, 4, true>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 8, 4>::describe(),
-      FusedSort<uint32_t, 0, 8, 256, 16, 4>::describe(),
-      FusedSort<uint32_t, 0, 8, 256, 8, 4>::describe(),
+      FusedSort<uint32_t, 0, 8, 256, 16, 2>::describe(),
+      FusedSort<uint32_t, 0, 8, 256, 8, 3>::describe(),
       ClusterSort<uint32_t, 0, 8, 512, 16, 8>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 22, 4, true>::describe(),
       OnesweepSort<uint32_t, 0, 8, 256, 45, 2, true>::describe(),

@@ -12,7 +12,7 @@ const Variant* variants_k64(int* count) {
       OnesweepSort<uint64_t, 0, 8, 256, 8, 4>::describe(),
       SmallSort<uint64_t, 0, 8, 1024, 8>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 12, 3, true>::describe(),
-      FusedSort<uint64_t, 0, 8, 256, 12, 3>::describe(),
+      FusedSort<uint64_t, 0, 8, 256, 12, 2>::describe(),
       ClusterSort<uint64_t, 0, 8, 512, 16, 8>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 16, 3, true>::describe(),
       OnesweepSort<uint64_t, 0, 8, 256, 25, 2, true>::describe(),
@@ -20,7 +20,7 @@ const Variant* variants_k64(int* count) {
       OnesweepSort<uint64_t, 0, 8, 256, 11, 4, true>::describe(),
       OnesweepSort<uint64_t, 0, 8, 512, 11, 2, true>::describe(),
       ClusterSort<uint64_t, 0, 8, 512, 16, 16>::describe(),
-      FusedSort<uint64_t, 0, 8, 256, 8, 4>::describe(),
+      FusedSort<uint64_t, 0, 8, 256, 8, 3>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;

@@ -14,8 +14,8 @@ const Variant* variants_kv32(int* count) {
       OnesweepSort<uint32_t, 4, 7, 256, 16, 4>::describe(),
       SmallSort<uint32_t, 4, 8, 1024, 8>::describe(),
       OnesweepSort<uint32_t, 4, 8, 256, 16, 4, true>::describe(),
-      FusedSort<uint32_t, 4, 8, 256, 16, 4>::describe(),
-      FusedSort<uint32_t, 4, 8, 256, 8, 4>::describe(),
+      FusedSort<uint32_t, 4, 8, 256, 16, 2>::describe(),
+      FusedSort<uint32_t, 4, 8, 256, 8, 3>::describe(),
       ClusterSort<uint32_t, 4, 8, 512, 16, 8>::describe(),
       OnesweepSort<uint32_t, 4, 8, 256, 18, 4, true>::describe(),
       OnesweepSort<uint32_t, 4, 8, 256, 41, 2, true>::describe(),

@@ -19,7 +19,7 @@ const Variant* variants_kv64(int* count) {
       OnesweepSort<uint64_t, 8, 8, 384, 14, 2, true>::describe(),
       OnesweepSort<uint64_t, 8, 8, 512, 10, 2, true>::describe(),
       ClusterSort<uint64_t, 8, 8, 512, 16, 16>::describe(),
-      FusedSort<uint64_t, 8, 8, 256, 8, 3>::describe(),
+      FusedSort<uint64_t, 8, 8, 256, 8, 2>::describe(),
   };
   *count = int(sizeof(table) / sizeof(table[0]));
   return table;
