@@ -235,6 +235,16 @@ rs_status rs_sort(int key_bytes, int val_bytes, void* keys, void* vals, void* ke
                   void* ws, size_t ws_bytes, rs_stream_t stream, int* result_in_alt);
 
 /*
+ * rs_sort whose result is always in keys / vals, whatever the number of digit
+ * passes; the contents of keys_alt / vals_alt afterwards are not specified.
+ * Arguments, errors and device-side status as for rs_sort.
+ */
+rs_status rs_sort_in_place(int key_bytes, int val_bytes, void* keys, void* vals, void* keys_alt,
+                           void* vals_alt, size_t n, int begin_bit, int end_bit,
+                           const rs_config* cfg, void* ws, size_t ws_bytes,
+                           rs_stream_t stream);
+
+/*
  * End-to-end form of rs_sort for data in host memory: copies the caller's
  * host arrays into the device buffers, sorts them (Sec. 2.6, as rs_sort) and
  * copies the sorted arrays back, all enqueued on `stream` in that order.

@@ -378,9 +378,10 @@ rs_status rs_workspace_bytes(int key_bytes, int val_bytes, size_t n, int begin_b
   return RS_OK;
 }
 
-rs_status rs_sort(int key_bytes, int val_bytes, void* keys, void* vals, void* keys_alt,
-                  void* vals_alt, size_t n, int begin_bit, int end_bit, const rs_config* cfg,
-                  void* ws, size_t ws_bytes, rs_stream_t stream, int* result_in_alt) {
+static rs_status sort_impl(int key_bytes, int val_bytes, void* keys, void* vals, void* keys_alt,
+                           void* vals_alt, size_t n, int begin_bit, int end_bit,
+                           const rs_config* cfg, void* ws, size_t ws_bytes, rs_stream_t stream,
+                           bool in_place, int* result_in_alt) {
   if (!result_in_alt || !valid_types(key_bytes, val_bytes)) return RS_ERR_INVALID;
   if (n > RS_MAX_N || begin_bit < 0 || begin_bit > end_bit || end_bit > 8 * key_bytes)
     return RS_ERR_INVALID;
@@ -413,6 +414,7 @@ rs_status rs_sort(int key_bytes, int val_bytes, void* keys, void* vals, void* ke
              reinterpret_cast<cudaStream_t>(stream), knobs_now()};
   a.key_kind = key_kind;
   a.descending = descending;
+  a.in_place = in_place;
   int in_alt = 0;
   nvtx_push("rs_sort");
   const cudaError_t e = v->run(a, &in_alt);
@@ -420,6 +422,22 @@ rs_status rs_sort(int key_bytes, int val_bytes, void* keys, void* vals, void* ke
   if (e != cudaSuccess) return RS_ERR_CUDA;
   *result_in_alt = in_alt;
   return RS_OK;
+}
+
+rs_status rs_sort(int key_bytes, int val_bytes, void* keys, void* vals, void* keys_alt,
+                  void* vals_alt, size_t n, int begin_bit, int end_bit, const rs_config* cfg,
+                  void* ws, size_t ws_bytes, rs_stream_t stream, int* result_in_alt) {
+  return sort_impl(key_bytes, val_bytes, keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit,
+                   cfg, ws, ws_bytes, stream, false, result_in_alt);
+}
+
+rs_status rs_sort_in_place(int key_bytes, int val_bytes, void* keys, void* vals, void* keys_alt,
+                           void* vals_alt, size_t n, int begin_bit, int end_bit,
+                           const rs_config* cfg, void* ws, size_t ws_bytes,
+                           rs_stream_t stream) {
+  int in_alt = 0;
+  return sort_impl(key_bytes, val_bytes, keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit,
+                   cfg, ws, ws_bytes, stream, true, &in_alt);
 }
 
 rs_status rs_sort_host(int key_bytes, int val_bytes, const void* h_keys, const void* h_vals,

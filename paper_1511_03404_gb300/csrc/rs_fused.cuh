@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
             ValT<VB>* __restrict__ v1, uint32_t n, int begin_bit, int end_bit, int passes,
             uint32_t* __restrict__ counts, Layout lay, uint32_t tiles,
             uint4* __restrict__ zero_base, uint64_t zero_vec4, Ctrl* __restrict__ ctrl, Knobs knobs, KeyXf<K> xf,
-            uint32_t shape) {
+            uint32_t shape, bool copy) {
   using F = FusedSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   using S = typename F::S;
   constexpr int RADIX = F::RADIX, MAXP = F::MAXP;
@@ -81,6 +81,13 @@ __global__ void __launch_bounds__(THREADS, MINB)
   // ---- 1. histograms of every pass, and the look-back words cleared
   for (int i = tid; i < passes * RADIX; i += THREADS) s_hist[i] = 0u;
   __syncthreads();
+  // copy: the input is in k1 and v1 and the passes start from a copy in k0 and
+  // v0, so that an odd number of them ends where the input was
+  const K* kin = copy ? k1 : k0;
+  if constexpr (VB > 0) {
+    if (copy)
+      for (uint32_t i = blockIdx.x * THREADS + tid; i < n; i += gridDim.x * THREADS) v0[i] = v1[i];
+  }
   auto count_all = [&](auto XF) {
     constexpr int LOADS = 4;  // in flight per thread
     const uint32_t stride = gridDim.x * THREADS;
@@ -88,10 +95,11 @@ __global__ void __launch_bounds__(THREADS, MINB)
       K k[LOADS];
 #pragma unroll
       for (uint32_t u = 0; u < LOADS; ++u)
-        if (i0 + u * stride < n) k[u] = k0[i0 + u * stride];
+        if (i0 + u * stride < n) k[u] = kin[i0 + u * stride];
 #pragma unroll
       for (uint32_t u = 0; u < LOADS; ++u) {
         if (i0 + u * stride >= n) break;
+        if (copy) k0[i0 + u * stride] = k[u];
         if constexpr (decltype(XF)::value) k[u] = xf_fwd(k[u], xf);
 #pragma unroll
         for (int p = 0; p < MAXP; ++p) {

@@ -25,6 +25,9 @@ struct SortArgs {
   Knobs knobs;
   int key_kind = 0;    // 0 unsigned, 1 signed, 2 float (see KeyXf)
   int descending = 0;
+  // the result has to end in keys / vals: a form that would leave it in the
+  // alternate buffers (an odd number of passes) starts from a copy there
+  bool in_place = false;
 };
 
 enum VariantKind { kOnesweep = 0, kSmall = 1, kOnesweepPersist = 2, kFused = 3, kCluster = 4 };

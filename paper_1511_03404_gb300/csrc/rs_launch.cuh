@@ -49,15 +49,17 @@ struct OnesweepSort {
   // early: the kernel after this one (the first pass) may be scheduled as
   // soon as this one starts, because its grid fills the GPU anyway
   // shape: the per-call record of rs_workspace_stats (0: none)
+  // copy: the keys and values are copied to the alternate buffers
   static cudaError_t upsweep(const SortArgs& a, int passes, const Layout& L, bool clear_status,
-                             bool early = false, uint32_t shape = 0u) {
+                             bool early = false, uint32_t shape = 0u, bool copy = false) {
     char* ws = static_cast<char*>(a.ws);
     Ctrl* ctrl = reinterpret_cast<Ctrl*>(ws);
     cudaError_t e = cudaMemsetAsync(ws, 0, L.memset_bytes, a.stream);
     if (e != cudaSuccess) return e;
-    const bool full = R == 8 && a.begin_bit == 0 && a.end_bit == 8 * int(sizeof(K));
-    auto kern = full ? &k_upsweep<K, R, UP_THREADS, MAXP, (R == 8)>
-                     : &k_upsweep<K, R, UP_THREADS, MAXP, false>;
+    const bool full = !copy && R == 8 && a.begin_bit == 0 && a.end_bit == 8 * int(sizeof(K));
+    auto kern = full   ? &k_upsweep<K, R, UP_THREADS, MAXP, (R == 8), false>
+                : copy ? &k_upsweep<K, R, UP_THREADS, MAXP, false, true>
+                       : &k_upsweep<K, R, UP_THREADS, MAXP, false, false>;
     constexpr int SLOTS = sizeof(K) == 4 ? 32 : 16;
     const int max_smem = MAXP * RADIX * SLOTS * 4;
     const int occ = prepare_kernel(reinterpret_cast<const void*>(kern), UP_THREADS, max_smem);
@@ -73,9 +75,11 @@ struct OnesweepSort {
         static_cast<const K*>(a.keys), a.n, a.begin_bit, a.end_bit, passes,
         reinterpret_cast<uint32_t*>(ws + L.counts), reinterpret_cast<uint32_t*>(ws + L.offsets),
         ctrl, reinterpret_cast<uint4*>(ws + L.status), zero_vec4,
-        make_key_xf<K>(a.key_kind, a.descending), early, shape);
+        make_key_xf<K>(a.key_kind, a.descending), early, shape,
+        copy ? static_cast<K*>(a.keys_alt) : nullptr, static_cast<const K*>(a.vals),
+        copy && VB > 0 ? static_cast<K*>(a.vals_alt) : nullptr);
     e = cudaGetLastError();
-    prof_after(a.stream, 0, double(a.n) * sizeof(K));
+    prof_after(a.stream, 0, double(a.n) * (copy ? 2 * (sizeof(K) + VB) : sizeof(K)));
     return e;
   }
 
@@ -85,6 +89,9 @@ struct OnesweepSort {
     const size_t nt = tiles(a.n);
     const Layout L = onesweep_layout(passes, R, nt);
     using V = ValT<VB>;
+    // passes from the copy in the alternate buffers end in keys / vals
+    const bool copy = a.in_place && (passes & 1) != 0;
+    if (copy) *in_alt = 0;
     auto kern = kernel<true>();
     int smem = Smem<true>::BYTES;
     if constexpr (VB == 0) {
@@ -104,7 +111,7 @@ struct OnesweepSort {
     const uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 |
                            1u << 24;
     nvtx_push("rs upsweep");
-    cudaError_t e = upsweep(a, passes, L, true, fills, shape);
+    cudaError_t e = upsweep(a, passes, L, true, fills, shape, copy);
     nvtx_pop();
     if (e != cudaSuccess) return e;
     char* ws = static_cast<char*>(a.ws);
@@ -134,8 +141,10 @@ struct OnesweepSort {
       cfg.numAttrs = pdl ? 1 : 0;
       nvtx_push(kPassNames[p]);
       e = cudaLaunchKernelEx(
-          &cfg, kern, static_cast<K*>(a.keys), static_cast<K*>(a.keys_alt),
-          static_cast<V*>(a.vals), static_cast<V*>(a.vals_alt), a.n, p, uint32_t(lo), mask,
+          &cfg, kern, static_cast<K*>(copy ? a.keys_alt : a.keys),
+          static_cast<K*>(copy ? a.keys : a.keys_alt),
+          static_cast<V*>(copy ? a.vals_alt : a.vals),
+          static_cast<V*>(copy ? a.vals : a.vals_alt), a.n, p, uint32_t(lo), mask,
           static_cast<const uint32_t*>(reinterpret_cast<const uint32_t*>(ws + L.offsets) +
                                        size_t(p) * RADIX),
           L.words(ws, p), uint32_t(nt),
@@ -201,10 +210,12 @@ struct FusedSort {
     if (occ <= 0) return cudaErrorInvalidConfiguration;
     const unsigned grid =
         unsigned(std::max<size_t>(1, std::min<size_t>(nt, size_t(device_info().sms) * occ)));
-    K* k0 = static_cast<K*>(a.keys);
-    K* k1 = static_cast<K*>(a.keys_alt);
-    V* v0 = static_cast<V*>(a.vals);
-    V* v1 = static_cast<V*>(a.vals_alt);
+    bool copy = a.in_place && (passes & 1) != 0;
+    if (copy) *in_alt = 0;
+    K* k0 = static_cast<K*>(copy ? a.keys_alt : a.keys);
+    K* k1 = static_cast<K*>(copy ? a.keys : a.keys_alt);
+    V* v0 = static_cast<V*>(copy ? a.vals_alt : a.vals);
+    V* v1 = static_cast<V*>(copy ? a.vals : a.vals_alt);
     uint32_t n = a.n;
     int begin = a.begin_bit, end = a.end_bit, np = passes;
     uint32_t* counts = reinterpret_cast<uint32_t*>(ws + L.counts);
@@ -216,7 +227,7 @@ struct FusedSort {
     KeyXf<K> xf = make_key_xf<K>(a.key_kind, a.descending);
     uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 | 2u << 24;
     void* args[] = {&k0, &k1, &v0, &v1, &n, &begin, &end, &np, &counts, &lay, &tiles, &zero_base,
-                    &zero_vec4, &ctrl, &knobs, &xf, &shape};
+                    &zero_vec4, &ctrl, &knobs, &xf, &shape, &copy};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(THREADS);

@@ -111,6 +111,7 @@ _SIGS = {
                       _vp, _vp], _i),
     "rs_workspace_stats": ([_vp, _vp, _vp], _i),
     "rs_sort": ([_i, _i, _vp, _vp, _vp, _vp, _sz, _i, _i, _vp, _vp, _sz, _vp, _vp], _i),
+    "rs_sort_in_place": ([_i, _i, _vp, _vp, _vp, _vp, _sz, _i, _i, _vp, _vp, _sz, _vp], _i),
     "rs_digit_counts": ([_i, _vp, _sz, _i, _i, _i, _vp, _vp, _vp, _vp, _sz, _vp], _i),
     "rs_workspace_status": ([_vp, _vp, _vp], _i),
     "rs_segmented_sort_pairs": ([_vp, _vp, _vp, _vp, _sz, _vp, _sz, _i, _i, _vp, _sz, _vp, _vp],
@@ -323,6 +324,15 @@ def rs_sort(key_bytes, val_bytes, keys, vals, keys_alt, vals_alt, n, begin_bit, 
                         end_bit, _cfg(radix_bits, variant, key_kind, descending), ws, ws_bytes,
                         stream, ctypes.byref(r))
     return st, r.value
+
+
+def rs_sort_in_place(key_bytes, val_bytes, keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit,
+                     ws, ws_bytes, stream, radix_bits=0, variant=-1, key_kind=RS_KEY_UNSIGNED,
+                     descending=False):
+    return load().rs_sort_in_place(key_bytes, val_bytes, keys, vals, keys_alt, vals_alt, n,
+                                   begin_bit, end_bit,
+                                   _cfg(radix_bits, variant, key_kind, descending), ws, ws_bytes,
+                                   stream)
 
 
 def rs_digit_counts(key_bytes, keys, n, begin_bit, end_bit, radix_bits, d_counts, d_offsets,
@@ -585,15 +595,10 @@ def sort(keys, vals=None, begin_bit=0, end_bit=None, radix_bits=0, variant=-1, s
         va = torch.empty_like(vals) if vals is not None else None
     else:
         ka, va = alt
-    st, in_alt = rs_sort(kb, vb, keys.data_ptr(), vals.data_ptr() if vals is not None else None,
-                         ka.data_ptr(), va.data_ptr() if va is not None else None, n, begin_bit,
-                         end_bit, ws.data_ptr(), ws.numel(), _stream_handle(stream), radix_bits,
-                         variant, kind, descending)
-    check(st, "rs_sort")
-    if in_alt:
-        keys.copy_(ka)
-        if vals is not None:
-            vals.copy_(va)
+    check(rs_sort_in_place(kb, vb, keys.data_ptr(), vals.data_ptr() if vals is not None else None,
+                           ka.data_ptr(), va.data_ptr() if va is not None else None, n, begin_bit,
+                           end_bit, ws.data_ptr(), ws.numel(), _stream_handle(stream), radix_bits,
+                           variant, kind, descending), "rs_sort")
     return keys, vals
 
 

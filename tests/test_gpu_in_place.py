@@ -1,0 +1,64 @@
+"""A sort whose result has to end where its input was starts, when its number
+of passes is odd, from a copy that the counting kernel makes.  Bit ranges of
+one, two and three passes, in every form that can end in the alternate
+buffers, with the four arrays starting at 16-byte boundaries, all one element
+past one, or each at its own offset (the copy then goes by elements), against
+the oracle; nothing around the arrays may change."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+from gpu_util import from_dev, to_dev  # noqa: E402
+
+from paper_1511_03404_gb300 import rs  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+GUARD = 8
+
+
+def forms(kb, vb):
+    """One variant of each kind with global passes: the first compiled."""
+    out = {}
+    for i in range(rs.rs_num_variants(kb, vb)):
+        out.setdefault(rs.rs_variant_info(kb, vb, i)["kind"], i)
+    return [out[k] for k in (0, 2, 3) if k in out]
+
+
+@pytest.mark.parametrize("dt", [np.uint32, np.uint64])
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("offsets", [(0, 0, 0, 0), (1, 1, 1, 1), (0, 1, 3, 0)])
+@pytest.mark.parametrize("bits", [(0, 20), (3, 8), (5, 21)])
+def test_in_place(dt, pairs, offsets, bits):
+    rng = np.random.default_rng(11)
+    kb = np.dtype(dt).itemsize
+    vb = kb if pairs else 0
+    stream = torch.cuda.current_stream().cuda_stream
+    for variant in forms(kb, vb):
+        for n in (2, 33, 4099, 300007):
+            def buffer(off):
+                return to_dev(rng.integers(0, 2 ** 32, off + n + GUARD, dtype=dt), torch)
+            bk, bv, bka, bva = (buffer(o) for o in offsets)
+            before = [from_dev(b, dt) for b in (bk, bv)]
+            k, v, ka, va = (b.data_ptr() + o * kb for b, o in zip((bk, bv, bka, bva), offsets))
+            alts = [from_dev(b, dt) for b in (bka, bva)]
+            ws = rs.workspace(kb, vb, n, *bits, variant=variant)
+            rs.check(rs.rs_sort_in_place(kb, vb, k, v if pairs else None, ka,
+                                         va if pairs else None, n, *bits, ws.data_ptr(),
+                                         ws.numel(), stream, variant=variant))
+            st, info = rs.rs_workspace_status(ws.data_ptr(), stream)
+            rs.check(st)
+            ok, ov = offsets[0], offsets[1]
+            ek, ev = oracle.lsd_sort(before[0][ok:ok + n].copy(), before[1][ov:ov + n].copy(),
+                                     begin_bit=bits[0], end_bit=bits[1])
+            before[0][ok:ok + n] = ek
+            if pairs:
+                before[1][ov:ov + n] = ev
+            what = (variant, n)
+            assert np.array_equal(from_dev(bk, dt), before[0]), what
+            assert np.array_equal(from_dev(bv, dt), before[1]), what
+            for b, a, o in zip((bka, bva), alts, offsets[2:]):
+                got = from_dev(b, dt)
+                assert np.array_equal(got[:o], a[:o]) and np.array_equal(got[o + n:], a[o + n:]), what
