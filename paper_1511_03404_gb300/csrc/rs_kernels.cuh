@@ -1438,10 +1438,11 @@ struct SmallSmem {
   static constexpr int KEYS = TOT + 32 * 4;                              // K [TILE]
   static constexpr int IDX = KEYS + TILE * int(sizeof(K));               // u16 [TILE]
   static constexpr int END = (IDX + (INDEX ? TILE * 2 : 0) + 15) / 16 * 16;
-  // the values, in the end: where the counters were if they fit
+  static constexpr int BYTES = END;
+  // the values, in the end, go where the counters were if they fit, else
+  // where the keys were
   static constexpr bool VALS_FIT = TILE * VB <= TOT;
-  static constexpr int VALS = VALS_FIT ? 0 : END;                        // V [TILE]
-  static constexpr int BYTES = VALS_FIT ? END : END + TILE * VB;
+  static_assert(VB == 0 || VB == int(sizeof(K)), "the values fit the keys' place");
 };
 
 // All digit passes of one array of len <= TILE elements inside one CTA.  The
@@ -1467,7 +1468,6 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
   uint32_t* s_tot = reinterpret_cast<uint32_t*>(smem + S::TOT);
   K* s_k = reinterpret_cast<K*>(smem + S::KEYS);
   uint16_t* s_i = reinterpret_cast<uint16_t*>(smem + S::IDX);
-  V* s_v = reinterpret_cast<V*>(smem + S::VALS);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int items = int((len + THREADS - 1) / THREADS);
   constexpr int BATCH = ITEMS < 4 ? ITEMS : 4;
@@ -1576,14 +1576,25 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
     }
     if (!__syncthreads_or(bad)) break;
   }
-  if constexpr (VB > 0) {
+  // (a test of the length instead left the 1024 x 16 form for 64-bit pairs 40
+  // bytes of spills and 5 % slower)
+  constexpr bool fit = VB > 0 && S::VALS_FIT;
+  V* s_v = reinterpret_cast<V*>(smem + (fit ? S::WH : S::KEYS));
+  if (fit) {
     for (uint32_t i = tid; i < len; i += THREADS) s_v[i] = vin[i];
     __syncthreads();
   }
   for (uint32_t i = tid; i < len; i += THREADS) {
     if (!dbg_ok(i, len, kSiteSmallOut)) continue;
     kout[i] = xf.on ? xf_inv(s_k[i], xf) : s_k[i];
-    if constexpr (VB > 0) vout[i] = s_v[s_i[i]];
+    if (fit) vout[i] = s_v[s_i[i]];
+  }
+  if (VB > 0 && !fit) {
+    __syncthreads();  // the keys have left
+    for (uint32_t i = tid; i < len; i += THREADS) s_v[i] = vin[i];
+    __syncthreads();
+    for (uint32_t i = tid; i < len; i += THREADS)
+      if (dbg_ok(i, len, kSiteSmallOut)) vout[i] = s_v[s_i[i]];
   }
 }
 

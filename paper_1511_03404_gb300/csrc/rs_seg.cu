@@ -1,7 +1,7 @@
 // Host side of the batched segmented sort (each of the four data types):
 // workspace sizing and the launch sequence memset -> k_seg_plan ->
-// k_seg_small (short, then medium) -> k_seg_hist -> k_seg_persistent, all on the caller's stream
-// (capturable in a CUDA graph).
+// k_seg_small (short, then medium) -> k_seg_hist -> k_seg_persistent, all on
+// the caller's stream (capturable in a CUDA graph).
 #include <algorithm>
 
 #include "../../include/rs.h"
@@ -14,8 +14,8 @@ namespace {
 
 // MINB: resident CTAs per SM the short-segment kernel is compiled for (its
 // register budget); PASS_MINB: the same for the pass kernel.
-template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS, int MEDIUM_ITEMS, int MINB = 4,
-          int PASS_MINB = MINB>
+template <class K, int VB, int R, int THREADS, int ITEMS, int CHUNK_TILES, int SMALL_ITEMS,
+          int MEDIUM_ITEMS, int MINB, int PASS_MINB>
 struct SegSort {
   using C = SegKernelCfg<K, VB, R, THREADS, ITEMS, CHUNK_TILES, SMALL_ITEMS>;
   static constexpr int PLAN_THREADS = 256, MEDIUM_THREADS = 1024;
@@ -145,16 +145,22 @@ struct SegSort {
   }
 };
 
-// u32 pairs: pass tiles of 256 x 45 keys ranked in half-warp units, two CTAs
-// per SM; short segments up to 4096 elements sorted whole by one CTA
-using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 41, 12, 16, 16, 4, 2>;
-// u32 keys: 256 x 37 keys in half-warp units, two CTAs per SM; short
-// segments up to 4096
-using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 45, 14, 16, 16, 4, 2>;
-// 64-bit keys and pairs: 256 x 23 elements in half-warp units, two CTAs per
-// SM; short segments up to 2048 (pairs: that kernel at three CTAs per SM)
-using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 8, 8, 4, 2>;
-using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 8, 8, 3, 2>;
+// Short segments are sorted by a CTA of 256 threads up to 256 x SMALL_ITEMS
+// elements, medium ones by one of 1024 threads up to 1024 x MEDIUM_ITEMS (its
+// counters, keys and positions fill the shared memory of an SM), longer ones in
+// passes over tiles of 256 x ITEMS, two CTAs an SM.  The lines lie where the
+// next form becomes the faster one: 20,000 log-uniform segments of 2^26 u32
+// pairs / keys take 1405 / 1048 us with medium segments up to 16 items a
+// thread, 1363 / 1004 up to 20, 1403 / 1052 up to 24; of 2^25 u64 pairs / keys
+// 2049 / 1666 up to 8, 1827 / 1441 up to 12, 1715 / 1372 up to 16.  10,000 rows
+// of up to 3,000 u64 pairs / keys take 773 / 664 us with short segments up to
+// 8 items a thread, 489 / 366 up to 12, 510 / 390 up to 16; rows of up to
+// 2,047 take 364 / 285, 388 / 298 and 413 / 320, for the registers; u32 ones
+// are the same at 16 and 24.
+using SegU32Pairs = SegSort<uint32_t, 4, 8, 256, 41, 12, 16, 20, 4, 2>;
+using SegU32Keys = SegSort<uint32_t, 0, 8, 256, 45, 14, 16, 20, 4, 2>;
+using SegU64Keys = SegSort<uint64_t, 0, 8, 256, 23, 24, 12, 16, 4, 2>;
+using SegU64Pairs = SegSort<uint64_t, 8, 8, 256, 23, 24, 12, 16, 3, 2>;
 
 bool seg_types(int kb, int vb) { return (kb == 4 || kb == 8) && (vb == 0 || vb == kb); }
 

@@ -256,7 +256,7 @@ __device__ __forceinline__ void seg_warp_sort(const K* kin, const ValT<VB>* vin,
 // current one is sorted), so that long and short ones even out.  MEDIUM: the
 // medium list alone, on CTAs of 1024 threads: one read and one write of a
 // segment instead of a histogram and a tile or two in every pass (20,000
-// log-uniform segments of 2^26 pairs: the tiled passes take 28 % less).
+// log-uniform segments of 2^26 pairs: the tiled passes take 36 % less).
 template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX, int MINB,
           bool MEDIUM = false>
 __global__ void __launch_bounds__(THREADS, MINB)

@@ -103,10 +103,13 @@ def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
 def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
     """Empty, one-warp (up to 32), one-CTA (every number of items a thread, and
-    the larger CTAs of medium ones) and tiled segments, more of them than one round of the planner takes."""
+    the larger CTAs of medium ones) and tiled segments, more of them than one
+    round of the planner takes."""
     rng = np.random.default_rng(7)
-    lengths = [0, 1, 2, 31, 32, 33, 255, 256, 257, 1023, 1025, 2047, 2048, 2049, 3841, 4096, 4097,
-               8191, 8192, 8193, 12000, 0, 16383, 16384, 16385, 30011, 70001]
+    lengths = [0, 1, 2, 31, 32, 33, 255, 256, 257, 1023, 1025, 2047, 2048, 2049, 3071,
+               3072, 3073, 3841, 4096, 4097,
+               8191, 8192, 8193, 12000, 0, 16383, 16384, 16385, 20479, 20480, 20481, 30011,
+               70001]
     lengths += list(rng.integers(0, 70, 9000)) + [5, 0, 4096, 0]
     off = inputs.offsets_from_lengths(np.asarray(lengths, dtype=np.uint64))
     n = int(off[-1])
