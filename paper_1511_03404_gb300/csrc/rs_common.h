@@ -7,11 +7,11 @@
 
 namespace rs {
 
-// Look-back status word of one (tile, digit): 2 flag bits + a 30-bit count.
+// Look-back status word of one (tile, digit) of a segment: 2 flag bits + a
+// 30-bit count.
 constexpr uint32_t kFlagShift = 30;
 constexpr uint32_t kFlagAgg = 1u << kFlagShift;  // count of this tile only
 constexpr uint32_t kFlagInc = 2u << kFlagShift;  // count of all tiles up to and including this one
-constexpr uint32_t kFlagErr = 3u << kFlagShift;  // this tile gave up; successors give up too
 constexpr uint32_t kFlagMask = 3u << kFlagShift;
 constexpr uint32_t kValueMask = (1u << kFlagShift) - 1u;
 
@@ -122,7 +122,7 @@ inline KeyXf<K> make_key_xf(int kind, int descending) {
   return x;
 }
 
-// Word of (tile or group t, digit d) in a [t/4][radix][4] look-back array.
+// Word of (tile t, digit d) in a segment's [t/4][radix][4] look-back array.
 template <int RADIX>
 __host__ __device__ __forceinline__ size_t lb_index(uint32_t t, uint32_t d) {
   return ((size_t(t >> 2) * RADIX + d) << 2) | (t & 3u);

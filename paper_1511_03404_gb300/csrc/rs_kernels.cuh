@@ -485,8 +485,10 @@ __device__ __forceinline__ void trace_add(uint64_t* tr, int k, uint64_t v) {
 // side by side.  Under load such a round trip takes 1-2 us, and how many
 // follow one another is what a look-back costs: a walk over groups of 32
 // tiles, 8 tiles at a time, took 3.8 of them a tile (5.9 of its 10.5 us, keys
-// alone at 2^26); this one takes 1.7, the first under the stage, and leaves
-// 2.8 of 9.2 us.
+// alone at 2^26); this one takes 1.4 to 1.7, the first under the stage, and
+// leaves 2.5 of 9.5 us.  What is left waits for tiles in flight: windows of 4
+// and 6 supers (1.04 round trips) took u32 pairs from 1.012 to 1.057 and
+// 1.088 ms, for their words.
 template <class K, int VB, int RADIX>
 struct TreeLookBack {
   uint32_t excl = 0u;
@@ -879,10 +881,10 @@ struct Prefetch {
 // after item, a chain of three of them; the returning atomic ranks 2.58e12
 // digits a second on the whole GPU, the masks 0.91e12 (random digits in
 // registers; all 32 lanes on one digit: 0.297e12 and 0.267e12).  Measured at
-// 2^26, a whole sort, before -> now, ms: u32 keys 1.09 -> 0.777, u32 pairs
-// 1.31 -> 1.075, u64 keys 3.04 -> 2.32, u64 pairs 4.08 -> 3.74; pipe busy
-// (2^24) 68 % -> 68 % (keys), 79 % (pairs) at 25.5 -> 19.0 and 34 -> 30.5
-// wavefronts per 32 elements.
+// 2^26, a whole sort, before -> now, ms: u32 keys 1.09 -> 0.726, u32 pairs
+// 1.31 -> 1.012, u64 keys 3.04 -> 2.285, u64 pairs 4.08 -> 3.51; pipe busy
+// 68 % -> 76 % (u32 keys) and 80 % (u32 pairs) at 25.5 -> 16.8 and 29.6 ->
+// 25.5 wavefronts per 32 elements.
 //
 // PERSIST: the calling kernel keeps the CTA resident over many tiles.  The
 // barriers are initialised once by the kernel, this tile's keys were staged
