@@ -62,3 +62,38 @@ def test_in_place(dt, pairs, offsets, bits):
             for b, a, o in zip((bka, bva), alts, offsets[2:]):
                 got = from_dev(b, dt)
                 assert np.array_equal(got[:o], a[:o]) and np.array_equal(got[o + n:], a[o + n:]), what
+
+
+@pytest.mark.parametrize("n", [5000, 300007, 3000001])
+def test_in_place_captured(n):
+    """Captured once, replayed on new inputs in the same buffers: the copy is
+    part of the graph."""
+    rng = np.random.default_rng(5)
+    k = torch.empty(n, dtype=torch.int32, device="cuda")
+    v, ka, va = (torch.empty_like(k) for _ in range(3))
+    ws = rs.workspace(4, 4, n, 0, 20)
+    side = torch.cuda.Stream()
+
+    def sort():
+        rs.check(rs.rs_sort_in_place(4, 4, k.data_ptr(), v.data_ptr(), ka.data_ptr(),
+                                     va.data_ptr(), n, 0, 20, ws.data_ptr(), ws.numel(),
+                                     torch.cuda.current_stream().cuda_stream))
+
+    with torch.cuda.stream(side):
+        k.zero_()
+        v.zero_()
+        sort()
+    side.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        sort()
+    for _ in range(2):
+        hk, hv = (rng.integers(0, 2 ** 32, n, dtype=np.uint32) for _ in range(2))
+        k.copy_(to_dev(hk, torch))
+        v.copy_(to_dev(hv, torch))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        ek, ev = oracle.lsd_sort(hk, hv, begin_bit=0, end_bit=20)
+        assert np.array_equal(from_dev(k, np.uint32), ek)
+        assert np.array_equal(from_dev(v, np.uint32), ev)
