@@ -36,13 +36,16 @@ struct FusedSmem {
   static constexpr int MAXP = (8 * int(sizeof(K)) + RADIX_BITS - 1) / RADIX_BITS;
   static constexpr int OFF = (S::BYTES + 15) / 16 * 16;  // u32 [MAXP][RADIX] digit offsets
   static constexpr int FLAG = OFF + MAXP * RADIX * 4;    // u32: barrier outcome
+  static constexpr int ONE = FLAG + 4;                   // u32: passes with one digit value
   static constexpr int BYTES = FLAG + 16;
   // the histograms of step 1 use the warp-counter region of the tile
   static_assert(MAXP <= S::WARPS, "histograms fit the warp counters");
 };
 
 // All CTAs of the grid meet; false if the wait ran out or an error was
-// reported (CTA-uniform).
+// reported (CTA-uniform).  Nothing else may write *s_flag: no barrier stands
+// between the threads' reads of it here and what thread 0 does next, and a
+// thread that read another word's zero would leave the kernel alone.
 __device__ __forceinline__ bool grid_barrier(Ctrl* ctrl, uint32_t gen, uint64_t timeout_ns,
                                              uint32_t* s_flag) {
   __syncthreads();
@@ -55,6 +58,13 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* ctrl, uint32_t gen, uint64_t 
     *s_flag = ok ? 1u : 0u;
   }
   __syncthreads();
+  if constexpr (kDebugChecks) {
+    // debug builds: all warps but the first read late, so that a store to the
+    // word before they have read it shows
+    const uint64_t t0 = global_ns();
+    while (threadIdx.x >= 32 && global_ns() - t0 < 20000u) {
+    }
+  }
   return *s_flag != 0u;
 }
 
@@ -74,12 +84,14 @@ __global__ void __launch_bounds__(THREADS, MINB)
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + S::MISC);
   uint32_t* s_off = reinterpret_cast<uint32_t*>(smem + F::OFF);
   uint32_t* s_flag = reinterpret_cast<uint32_t*>(smem + F::FLAG);
+  uint32_t* s_one = reinterpret_cast<uint32_t*>(smem + F::ONE);
   const int tid = threadIdx.x;
   const bool rec = blockIdx.x == 0 && tid == 0;  // keeps the per-call record
   if (rec) stat_begin(ctrl, n, shape);
 
   // ---- 1. histograms of every pass, and the look-back words cleared
   for (int i = tid; i < passes * RADIX; i += THREADS) s_hist[i] = 0u;
+  if (tid == 0) *s_one = 0u;
   __syncthreads();
   // copy: the input is in k1 and v1 and the passes start from a copy in k0 and
   // v0, so that an odd number of them ends where the input was
@@ -143,9 +155,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     if (lane == 31) s_sum[p * 32 + warp] = inc[p];
   }
   one = __reduce_or_sync(kFull, one);
-  if (tid == 0) *s_flag = 0u;
   __syncthreads();
-  if (lane == 0 && one != 0u) atomicOr(s_flag, one);
+  if (lane == 0 && one != 0u) atomicOr(s_one, one);
 #pragma unroll
   for (int p = 0; p < MAXP; ++p) {
     const uint32_t before =
@@ -153,7 +164,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     if (p < passes && tid < RADIX) s_off[p * RADIX + tid] = before + inc[p] - cnt[p];
   }
   __syncthreads();
-  uint32_t exec = ~*s_flag & ((1u << passes) - 1u);
+  uint32_t exec = ~*s_one & ((1u << passes) - 1u);
   if ((__popc(exec) & 1) != (passes & 1)) {  // keep the result in buffer (passes mod 2)
     const uint32_t skipped = ~exec & ((1u << passes) - 1u);
     exec |= skipped & (0u - skipped);
