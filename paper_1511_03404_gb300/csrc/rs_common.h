@@ -141,10 +141,11 @@ __host__ __device__ __forceinline__ size_t lb_index(uint32_t t, uint32_t d) {
 // stores, atomics and loads is one line.  (Four groups of one digit side by
 // side, fetched by one 16-byte load, took 2.5 times the sectors.)  The words
 // are one range, zeroed by the upsweep.  The size asked of the caller is what
-// 32-bit tile words with two words per 32 tiles would take: somewhat more.
+// 32-bit tile words with two words per 32 tiles would take, both counts rounded
+// up to 4: more than the words take, whatever the number of tiles.
 struct Layout {
   size_t counts, offsets, status, gagg, sagg, sinc, status_bytes, total, memset_bytes;
-  size_t tiles, groups, supers;  // rounded up
+  size_t tiles, groups, supers;
   size_t radix;
 
   // the words of pass p
@@ -162,9 +163,9 @@ inline Layout onesweep_layout(int passes, int radix_bits, size_t tiles) {
   Layout L;
   const size_t radix = size_t(1) << radix_bits;
   L.radix = radix;
-  L.tiles = align_up(tiles, 8);
-  L.groups = align_up((tiles + kGroupTiles - 1) / kGroupTiles, 4);
-  L.supers = align_up((tiles + kSuperTiles - 1) / kSuperTiles, 4);
+  L.tiles = tiles;
+  L.groups = (tiles + kGroupTiles - 1) / kGroupTiles;
+  L.supers = (tiles + kSuperTiles - 1) / kSuperTiles;
   L.counts = 256;
   L.offsets = align_up(L.counts + size_t(passes) * radix * 4, 256);
   L.status = align_up(L.offsets + size_t(passes) * radix * 4, 256);
@@ -174,7 +175,7 @@ inline Layout onesweep_layout(int passes, int radix_bits, size_t tiles) {
   L.status_bytes = align_up(L.sinc + size_t(passes) * L.supers * radix * 4 - L.status, 256);
   const size_t asked = size_t(passes) * radix * 4 *
                        (align_up(tiles, 4) + 2 * align_up((tiles + 31) / 32, 4));
-  L.total = L.status + (asked > L.status_bytes ? align_up(asked, 256) : L.status_bytes);
+  L.total = L.status + align_up(asked, 256);
   L.memset_bytes = L.offsets;  // Ctrl + counts
   return L;
 }
