@@ -145,8 +145,11 @@ rs_status rs_tune_clear(void);
 
 /*
  * Workspace bytes a sort of n elements over [begin_bit, end_bit) needs with
- * configuration cfg (NULL = library choice).  The sort entry points with the
- * same arguments accept any workspace at least this large.
+ * configuration cfg (NULL = library choice).  The sort entry points accept any
+ * workspace at least this large with the same arguments, and with a smaller n
+ * or fewer bits: one workspace of the longest array serves a program that sorts
+ * several lengths (a shorter one whose own choice takes more is sorted with the
+ * longer one's).
  */
 rs_status rs_workspace_bytes(int key_bytes, int val_bytes, size_t n, int begin_bit, int end_bit,
                              const rs_config* cfg, size_t* bytes);

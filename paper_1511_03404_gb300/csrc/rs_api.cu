@@ -288,6 +288,21 @@ static int tuned_variant(int kb, int vb, size_t n) {
 
 // -------------------------------------------------------------- choosing
 
+static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
+
+// Without a table: one CTA when the array fits a small-sort tile, else onesweep.
+static const Variant* default_variant(const Variant* v, int count, size_t n, int want_r) {
+  const Variant* best = nullptr;
+  for (int i = 0; i < count; ++i) {
+    const Variant* c = &v[i];
+    if (want_r && c->radix_bits != want_r) continue;
+    if (n > c->max_n) continue;
+    if (c->kind == kSmall && (!best || best->kind != kSmall)) best = c;
+    if ((c->kind == kOnesweep || c->kind == kOnesweepPersist) && !best) best = c;
+  }
+  return best;
+}
+
 static const Variant* choose(int kb, int vb, size_t n, const rs_config* cfg) {
   int count = 0;
   const Variant* v = variants(kb, vb, &count);
@@ -303,23 +318,74 @@ static const Variant* choose(int kb, int vb, size_t n, const rs_config* cfg) {
     const int tv = tuned_variant(kb, vb, n);
     if (tv >= 0 && tv < count && n <= v[tv].max_n) return &v[tv];
   }
-  // default: one CTA when the array fits a small-sort tile, else onesweep
-  const Variant* best = nullptr;
-  for (int i = 0; i < count; ++i) {
-    const Variant* c = &v[i];
-    if (want_r && c->radix_bits != want_r) continue;
-    if (n > c->max_n) continue;
-    if (c->kind == kSmall && (!best || best->kind != kSmall)) best = c;
-    if ((c->kind == kOnesweep || c->kind == kOnesweepPersist) && !best) best = c;
+  return default_variant(v, count, n, want_r);
+}
+
+static size_t variant_bytes(const Variant& v, size_t n, int begin_bit, int end_bit) {
+  return v.workspace(uint32_t(n), num_passes(begin_bit, end_bit, v.radix_bits));
+}
+
+// The library's choice for n elements when `room` bytes of workspace are less
+// than it takes: the choice for a longer array, nearest first, if the room is
+// what the shortest array with that choice would be asked for.  Tile sizes do
+// not only grow with n (smaller tiles take over at some lengths, and take more
+// words), and a workspace sized for a program's longest array has to serve the
+// shorter ones.  Null where no longer array's workspace would be this small.
+static const Variant* choose_within(int kb, int vb, size_t n, int begin_bit, int end_bit,
+                                    size_t room) {
+  int count = 0;
+  const Variant* v = variants(kb, vb, &count);
+  std::lock_guard<std::mutex> g(g_tune_mu);
+  auto fits = [&](const Variant* c, size_t shortest) {
+    return c && n <= c->max_n && shortest <= c->max_n &&
+           variant_bytes(*c, shortest, begin_bit, end_bit) <= room;
+  };
+  size_t from = 0;  // the band of an entry is (from, n_max]
+  auto it = g_tune.find(kb * 16 + vb);
+  if (it != g_tune.end()) {
+    for (const TuneEntry& e : it->second) {
+      if (e.n_max >= n) {
+        const size_t shortest = std::max(n, from + 1);
+        const Variant* c = &v[e.variant];
+        if (fits(c, shortest)) return c;
+        // the part of the band that its variant does not take
+        const size_t past = std::max(shortest, size_t(c->max_n) + 1);
+        if (past <= e.n_max) {
+          const Variant* d = default_variant(v, count, past, 0);
+          if (fits(d, past)) return d;
+        }
+      }
+      from = e.n_max;
+    }
   }
-  return best;
+  const size_t past = std::max(n, from + 1);
+  const Variant* d = past <= RS_MAX_N ? default_variant(v, count, past, 0) : nullptr;
+  return fits(d, past) ? d : nullptr;
+}
+
+// The variant of a sort that is given this workspace, and what it takes of it:
+// the choice, or if that takes more, one that fits (in a workspace that starts
+// where it may).
+static const Variant* choose_for(int kb, int vb, size_t n, int begin_bit, int end_bit,
+                                 const rs_config* cfg, const void* ws, size_t ws_bytes,
+                                 size_t* need) {
+  const Variant* v = choose(kb, vb, n, cfg);
+  if (!v) return nullptr;
+  *need = variant_bytes(*v, n, begin_bit, end_bit);
+  const size_t room = ws ? ws_bytes : 0;
+  if (*need > room && aligned(ws, 256) && !(cfg && (cfg->variant >= 0 || cfg->radix_bits > 0))) {
+    const Variant* w = choose_within(kb, vb, n, begin_bit, end_bit, room);
+    if (w) {
+      v = w;
+      *need = variant_bytes(*v, n, begin_bit, end_bit);
+    }
+  }
+  return v;
 }
 
 static bool valid_types(int kb, int vb) {
   return (kb == 4 || kb == 8) && (vb == 0 || vb == kb);
 }
-
-static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 }  // namespace rs
 
@@ -374,7 +440,7 @@ rs_status rs_workspace_bytes(int key_bytes, int val_bytes, size_t n, int begin_b
   if (n <= 1 || begin_bit == end_bit) return RS_OK;
   const Variant* v = choose(key_bytes, val_bytes, n, cfg);
   if (!v) return RS_ERR_INVALID;
-  *bytes = v->workspace(uint32_t(n), num_passes(begin_bit, end_bit, v->radix_bits));
+  *bytes = variant_bytes(*v, n, begin_bit, end_bit);
   return RS_OK;
 }
 
@@ -405,10 +471,10 @@ static rs_status sort_impl(int key_bytes, int val_bytes, void* keys, void* vals,
     if (!vals || !vals_alt || vals == vals_alt) return RS_ERR_INVALID;
     if (!aligned(vals, val_bytes) || !aligned(vals_alt, val_bytes)) return RS_ERR_INVALID;
   }
-  const Variant* v = choose(key_bytes, val_bytes, n, cfg);
+  size_t need = 0;
+  const Variant* v =
+      choose_for(key_bytes, val_bytes, n, begin_bit, end_bit, cfg, ws, ws_bytes, &need);
   if (!v) return RS_ERR_INVALID;
-  const int passes = num_passes(begin_bit, end_bit, v->radix_bits);
-  const size_t need = v->workspace(uint32_t(n), passes);
   if (need > 0 && (!ws || ws_bytes < need || !aligned(ws, 256))) return RS_ERR_WORKSPACE;
   SortArgs a{keys, vals, keys_alt, vals_alt, uint32_t(n), begin_bit, end_bit, ws, ws_bytes,
              reinterpret_cast<cudaStream_t>(stream), knobs_now()};
@@ -468,6 +534,7 @@ rs_status rs_sort_host(int key_bytes, int val_bytes, const void* h_keys, const v
     if (cfg && (cfg->key_kind < RS_KEY_UNSIGNED || cfg->key_kind > RS_KEY_FLOAT ||
                 (cfg->descending & ~1)))
       return RS_ERR_INVALID;
+    choose_for(key_bytes, val_bytes, n, begin_bit, end_bit, cfg, ws, ws_bytes, &need);
     if (need > 0 && (!ws || ws_bytes < need || !aligned(ws, 256))) return RS_ERR_WORKSPACE;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
