@@ -617,7 +617,9 @@ typedef enum rs_debug_knob {
   RS_DEBUG_TRACE_PASS = 5,        /* the digit pass whose tiles are traced */
   RS_DEBUG_LB_SMALL = 6,          /* accepted, without effect */
   RS_DEBUG_MIRROR_LANES = 8,      /* 1: lanes take their keys in reverse, so that equal digits
-                                     draw their ranks out of turn and every tile needs repair */
+                                     draw their ranks out of turn and every tile needs repair;
+                                     2: in the digit passes of a debug build a warp's keys of
+                                     one digit come wholly reversed (else as 1) */
   RS_DEBUG_BAD_INDEX_TILE = 7     /* debug build only (else RS_ERR_INVALID): this tile of
                                      digit pass 0 of a multi-launch sort computes scatter
                                      indices past the array, so that the bounds checks of

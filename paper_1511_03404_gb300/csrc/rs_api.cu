@@ -165,7 +165,7 @@ Knobs knobs_now() {
   k.trace = reinterpret_cast<uint64_t*>(g_trace_ptr.load());
   k.trace_tiles = uint32_t(g_trace_tiles.load());
   k.trace_pass = int32_t(g_trace_pass.load());
-  k.mirror = int32_t(g_mirror.load() != 0);
+  k.mirror = int32_t(g_mirror.load());
   k.dbg_bad_tile = int32_t(g_dbg_bad_tile.load());
   return k;
 }
@@ -800,7 +800,11 @@ rs_status rs_debug_set(rs_debug_knob knob, long long value) {
     case RS_DEBUG_LB_SMALL:
       return RS_OK;  // accepted, without effect
     case RS_DEBUG_MIRROR_LANES:
-      g_mirror.store(value);
+#ifdef RS_DEBUG
+      g_mirror.store(value == 2 ? 2 : value != 0);
+#else
+      g_mirror.store(value != 0);
+#endif
       return RS_OK;
     case RS_DEBUG_BAD_INDEX_TILE:
 #ifdef RS_DEBUG

@@ -66,8 +66,9 @@ struct Knobs {
   uint64_t* trace;         // device [trace_tiles][16] phase timestamps (ns) and counters, or null
   uint32_t trace_tiles;    // tiles 0 .. trace_tiles-1 of trace_pass are recorded
   int32_t trace_pass;
-  int32_t mirror;          // test-only: every warp's lanes take their keys in reverse, so that
-                           // equal digits draw their ranks out of turn
+  int32_t mirror;          // test-only: 1, every warp's lanes take their keys in reverse, so that
+                           // equal digits draw their ranks out of turn; 2 (digit passes of
+                           // debug builds), out of turn from item to item too
   int32_t dbg_bad_tile;    // debug builds only: this tile of pass 0 computes scatter
                            // indices past the array, which the bounds checks drop (-1: off)
 };

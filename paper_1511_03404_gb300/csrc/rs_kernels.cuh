@@ -451,7 +451,8 @@ struct TileArgs {
   int32_t drop_tile;            // test-only: this tile publishes nothing (-1: none)
   int32_t bad_tile;             // debug builds, test-only: this tile's scatter indices are
                                 // pushed past n (-1: none)
-  bool mirror;                  // test-only: lanes take their keys in reverse
+  int32_t mirror;               // test-only: 1, lanes take their keys in reverse; 2 (debug
+                                // builds), a warp's slots of a digit are taken in reverse
   bool xin;                     // the source holds untransformed keys: apply xf on load
   bool xout;                    // write untransformed keys (apply xf's inverse)
 };
@@ -871,8 +872,8 @@ struct Prefetch {
 //     key's bits): the bits up to this digit ascend over the whole stage.
 //     Keys that agree in all of them need no order: later passes tell them
 //     apart, or they are equal.
-// A tile that fails is put in order (a slot drawn out of turn is less than a
-// warp away from its place) and scattered again to the same destinations.
+// A tile that fails is put in order, whatever order its draws took, and
+// scattered again to the same destinations.
 //
 // What bounds it: the shared-memory pipe.  Each of the accesses by a random
 // digit or slot costs 3.1-3.6 wavefronts a warp: the count, the draw, the
@@ -950,10 +951,10 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   stamp(trace(), 1);
 
   // ---- 1. count.  Warp w owns tile slots [w*ITEMS*32, (w+1)*ITEMS*32); item j
-  // of lane l is slot w*ITEMS*32 + j*32 + l.  mirror (test-only): the lanes
+  // of lane l is slot w*ITEMS*32 + j*32 + l.  mirror 1 (test-only): the lanes
   // are taken in reverse, so that every repeated digit draws out of turn.
   K* s_kin = Stage<K>(t.ksrc + tile_base, tile_len).at(smem + S::KIN);
-  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (t.mirror ? 31 - lane : lane));
+  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (t.mirror == 1 ? 31 - lane : lane));
   uint32_t* wh = s_wh + warp * RADIX;
   // a tile's keys are its first tile_len slots; the rest draw nothing
   const uint32_t lim = tile_len - min(slot0, tile_len);  // item j is a key if j * 32 < lim
@@ -1082,6 +1083,30 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
     stage(std::true_type{});
   else
     stage(std::false_type{});
+  if constexpr (kDebugChecks) {
+    if (t.mirror == 2) {  // test-only: as if each warp's draws had come last item first
+      __syncthreads();
+      if (tid < RADIX) {
+        uint32_t at = my_start;
+        for (int w = 0; w < WARPS; ++w) {
+          const uint32_t end = s_wh[w * RADIX + tid];  // one past the slots drawn
+          for (uint32_t a = at, b = end; a + 1u < b; ++a) {
+            --b;
+            if constexpr (INDEX) {
+              const uint16_t x = s_idx[a];
+              s_idx[a] = s_idx[b];
+              s_idx[b] = x;
+            } else {
+              const K x = s_out[a];
+              s_out[a] = s_out[b];
+              s_out[b] = x;
+            }
+          }
+          at = end;
+        }
+      }
+    }
+  }
   // past the end, and one more: what the scatter may read, and ascends to
   for (uint32_t i = tile_len + tid; i <= uint32_t(TILE); i += THREADS) {
     if constexpr (INDEX) s_idx[i] = uint16_t(tile_len - 1u);
@@ -1210,8 +1235,12 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   bool ok = check(bad, 5) == 0u;
   const bool repaired = !ok;
   if (!ok) {
-    // out of turn: at most 31 places off, so 32 rounds of odd-even
-    // transposition put every digit run in order; then the scatter again
+    // out of turn.  A warp draws a digit's slots from a range that no other
+    // warp draws from, and the ranges are in order, so that no element is further
+    // from its place than such a range is long (at most ITEMS * 32): that many
+    // rounds of odd-even transposition, and one for the first parity, put
+    // every digit run in order.  Two rounds without an exchange end them
+    // early (draws out of turn within one item take up to 32).
     auto wrong = [&](uint32_t i) {  // stage slots i and i + 1 are out of order
       if constexpr (INDEX) {
         const uint32_t a = s_idx[i], b = s_idx[i + 1];
@@ -1220,9 +1249,11 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
         return (s_out[i] & upto_bits()) > (s_out[i + 1] & upto_bits());
       }
     };
-    for (int r = 0; r < 32; ++r) {
+    for (int r = 0, go = 2; r <= ITEMS * 32 && go > 0; ++r) {
+      bool moved = false;
       for (uint32_t i = uint32_t(2 * tid + (r & 1)); i + 1u < tile_len; i += 2 * THREADS) {
         if (!wrong(i)) continue;
+        moved = true;
         if constexpr (INDEX) {
           const uint16_t a = s_idx[i];
           s_idx[i] = s_idx[i + 1];
@@ -1233,7 +1264,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
           s_out[i + 1] = a;
         }
       }
-      __syncthreads();
+      go = __syncthreads_or(moved) ? 2 : go - 1;
     }
     bad = 0u;
     for (uint32_t i = tid; i < tile_len; i += THREADS) {
@@ -1310,7 +1341,7 @@ __device__ __forceinline__ void pass_args(
   t->tiles = tiles;
   t->xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
   t->xout = xf.on && pass == 31 - __clz(exec);
-  t->mirror = knobs.mirror != 0;
+  t->mirror = knobs.mirror;
   t->drop_tile = pass == knobs.drop_pass ? knobs.drop_tile : -1;
   t->bad_tile = kDebugChecks && pass == 0 ? knobs.dbg_bad_tile : -1;
   t->trace = pass == knobs.trace_pass ? knobs.trace : nullptr;

@@ -6,6 +6,10 @@ repair; the result must still be the oracle's, bit for bit.  Keys of few
 values make long runs of one digit, partial bit ranges take the slot-indexed
 stage for keys too, and the sizes lie around one tile and around the groups
 of 8 and 64 tiles of the look-back."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -153,3 +157,47 @@ def test_merge_tiles_by_bytes(kb, vb, mirror):
                 assert not vb or np.array_equal(gv, ev), (n, mask)
     finally:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
+
+
+@pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
+def test_any_order_of_a_warps_draws_is_repaired(dtype, pairs):
+    """A warp's keys of one digit in reverse, across its items: up to all the
+    keys of a warp are out of place, and by as many places."""
+    if not rs.debug_library():
+        pytest.skip("the reversal is in the debug build")
+    kb = np.dtype(dtype).itemsize
+    try:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 2))
+        for var in variants(kb, kb if pairs else 0, (0, 2, 3)):
+            tile = var["threads"] * var["items"]
+            for n in (33, tile - 1, 3 * tile + 5):
+                v = inputs.values(dtype, n) if pairs else None
+                for name, mask in (("uniform", None), ("few", 0x0303), ("two", 0x10001)):
+                    k = inputs.keys(dtype, "uniform", n)
+                    k = k if mask is None else k & dtype(mask)
+                    check(k, v, (name, n, var), variant=var["index"])
+                    check(k, v, (name, "bits", n, var), variant=var["index"], begin_bit=3,
+                          end_bit=17)
+        rng = np.random.default_rng(5)
+        off = inputs.offsets_from_lengths(np.asarray([30011, 70001, 20481, 5, 100000], np.uint64))
+        n = int(off[-1])
+        k = rng.integers(0, 4, n).astype(dtype)
+        v = inputs.values(dtype, n) if pairs else None
+        dk, dv = to_dev(k, torch), to_dev(v, torch) if pairs else None
+        rs.segmented_sort(dk, to_dev(off, torch), dv)
+        ek, ev = oracle.segmented_sort(k, v, off)
+        assert np.array_equal(from_dev(dk, dtype), ek)
+        assert not pairs or np.array_equal(from_dev(dv, dtype), ev)
+    finally:
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
+
+
+def test_any_order_under_the_debug_build():
+    if rs.debug_library():
+        pytest.skip("already the debug build")
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.abspath(__file__), "-m", "gpu",
+                        "-x", "-q", "-p", "no:cacheprovider", "-k", "any_order_of"],
+                       env=dict(os.environ, RS_LIBRARY="debug"), capture_output=True, text=True,
+                       timeout=900)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
+    assert "4 passed" in r.stdout and "skipped" not in r.stdout
