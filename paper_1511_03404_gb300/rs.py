@@ -518,9 +518,15 @@ def _torch():
     return torch
 
 
-def _stream_handle(stream=None) -> int:
-    if stream is not None:
-        return stream.cuda_stream
+def _on_stream(stream):
+    """The context in which ``stream`` is the current one."""
+    torch = _torch()
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(stream.cuda_stream)
+    return torch.cuda.stream(stream)
+
+
+def _stream_handle() -> int:
     # the handle without a Stream object around it (2.8 us of a small sort's 10
     # on the host, 0.4 this way)
     torch = _torch()
@@ -578,6 +584,10 @@ def sort(keys, vals=None, begin_bit=0, end_bit=None, radix_bits=0, variant=-1, s
     torch = _torch()
     if not keys.is_cuda or not keys.is_contiguous():
         raise ValueError("keys must be a contiguous CUDA tensor")
+    if stream is not None:  # the buffers allocated here are that stream's as well
+        with _on_stream(stream):
+            return sort(keys, vals, begin_bit, end_bit, radix_bits, variant, None, ws, alt,
+                        descending, key_kind)
     kb, kind = _key_type(keys)
     if key_kind is not None:
         kind = key_kind
@@ -597,7 +607,7 @@ def sort(keys, vals=None, begin_bit=0, end_bit=None, radix_bits=0, variant=-1, s
         ka, va = alt
     check(rs_sort_in_place(kb, vb, keys.data_ptr(), vals.data_ptr() if vals is not None else None,
                            ka.data_ptr(), va.data_ptr() if va is not None else None, n, begin_bit,
-                           end_bit, ws.data_ptr(), ws.numel(), _stream_handle(stream), radix_bits,
+                           end_bit, ws.data_ptr(), ws.numel(), _stream_handle(), radix_bits,
                            variant, kind, descending), "rs_sort")
     return keys, vals
 
@@ -614,6 +624,9 @@ def segmented_sort(keys, offsets, vals=None, begin_bit=0, end_bit=None, stream=N
     torch = _torch()
     if not keys.is_cuda or not keys.is_contiguous():
         raise ValueError("keys must be a contiguous CUDA tensor")
+    if stream is not None:  # the buffers allocated here and the copies back are that stream's
+        with _on_stream(stream):
+            return segmented_sort(keys, offsets, vals, begin_bit, end_bit, None, ws)
     kb = _key_bytes(keys)
     vb = 0
     if vals is not None:
@@ -633,7 +646,7 @@ def segmented_sort(keys, offsets, vals=None, begin_bit=0, end_bit=None, stream=N
     ptr = lambda t: None if t is None else t.data_ptr()  # noqa: E731
     st, in_alt = rs_segmented_sort(kb, vb, ptr(keys), ptr(vals), ptr(ka), ptr(va), n,
                                    offsets.data_ptr(), nseg, begin_bit, end_bit, ws.data_ptr(),
-                                   ws.numel(), _stream_handle(stream))
+                                   ws.numel(), _stream_handle())
     check(st, "rs_segmented_sort")
     if in_alt:
         keys.copy_(ka)
