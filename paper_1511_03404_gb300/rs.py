@@ -171,8 +171,10 @@ def load():
                 fn = getattr(lib, name)
                 fn.argtypes = args
                 fn.restype = res
-            _lib = lib
-            _apply_tuned_table(lib)
+            try:
+                _apply_tuned_table(lib)
+            finally:  # (a table that cannot be read is reported once)
+                _lib = lib  # from here on other threads use it, without the lock
     return _lib
 
 
