@@ -278,8 +278,8 @@ rs_status rs_sort_host(int key_bytes, int val_bytes, const void* h_keys, const v
  * is done: the digit passes that moved the data and those skipped because
  * one digit value held every key (Sec. 2.6's counting sort of that digit is
  * then the identity), the device time of each kernel phase, and the
- * algorithmic bytes.  Recorded by rs_sort, the four typed sorts,
- * rs_sort_host and rs_sort_keys_u32_noalloc (whose array has no public
+ * algorithmic bytes.  Recorded by rs_sort, rs_sort_in_place, the four typed
+ * sorts, rs_sort_host and rs_sort_keys_u32_noalloc (whose array has no public
  * address: its record is not readable).  A segmented sort's workspace gives
  * form 0; a workspace last used by the sample-sort, merge-sort or server
  * entry points holds no record.  Times come from the GPU's global timer and
@@ -301,7 +301,9 @@ typedef struct rs_sort_stats {
                             last CTA finished; 0 for skipped passes */
   double total_ms;       /* first kernel's start until the last recorded time */
   double bytes;          /* algorithmic bytes: n K for the histograms plus
-                            2 n (K + V) per moving pass (form 3: 2 n (K + V)) */
+                            2 n (K + V) per moving pass (form 3: 2 n (K + V)); an odd
+                            number of passes of rs_sort_in_place starts from a copy:
+                            n (K + 2 V) more */
 } rs_sort_stats;
 
 /* Synchronizes `stream`, then fills *out.  RS_ERR_INVALID for out NULL;

@@ -652,7 +652,7 @@ rs_status rs_workspace_stats(const void* ws, rs_stream_t stream, rs_sort_stats* 
   out->form = form;
   out->key_bytes = int(c.stat_shape & 0xffu);
   out->val_bytes = int((c.stat_shape >> 8) & 0xffu);
-  out->passes = int((c.stat_shape >> 16) & 0xffu);
+  out->passes = int((c.stat_shape >> 16) & 0x7fu);
   out->n = c.stat_n;
   if (out->passes < 1 || out->passes > kMaxPasses) {
     out->form = 0;
@@ -673,7 +673,8 @@ rs_status rs_workspace_stats(const void* ws, rs_stream_t stream, rs_sort_stats* 
   if (form == 3)
     out->bytes = 2.0 * n * (kb + vb);  // one read and one write; the passes stay on chip
   else
-    out->bytes = n * kb + double(__builtin_popcount(out->moved_mask)) * 2.0 * n * (kb + vb);
+    out->bytes = n * kb + ((c.stat_shape & kShapeCopied) ? n * (kb + 2.0 * vb) : 0.0) +
+                 double(__builtin_popcount(out->moved_mask)) * 2.0 * n * (kb + vb);
   return RS_OK;
 }
 

@@ -50,13 +50,16 @@ struct Ctrl {
   // block at the start of every multi-launch sort).  Times are %globaltimer
   // nanoseconds after t0, the upsweep's start.
   uint32_t stat_n;       // elements sorted
-  uint32_t stat_shape;   // key bytes | value bytes << 8 | passes << 16 | 1 << 24 (recorded)
+  uint32_t stat_shape;   // key bytes | value bytes << 8 | passes << 16 | form << 24, and
+                         // kShapeCopied if the passes started from a copy
   uint32_t t0_lo, t0_hi; // %globaltimer when the upsweep started
   uint32_t t_upsweep;    // upsweep's last CTA done
   uint32_t t_pass[kMaxPasses][2];  // per pass: first tile taken, last CTA done
   uint32_t reserved[64 - 5 - kMaxPasses - 5 - 2 * kMaxPasses];
 };
 static_assert(sizeof(Ctrl) == 256, "Ctrl must be 256 bytes");
+
+constexpr uint32_t kShapeCopied = 1u << 23;
 
 // Test-only fault injection and the bound on every device-side wait.
 struct Knobs {

@@ -109,7 +109,7 @@ struct OnesweepSort {
     const bool pdl = pdl_enabled();
     const bool fills = pdl && (PERSIST || nt > size_t(device_info().sms) * occ);
     const uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 |
-                           1u << 24;
+                           1u << 24 | (copy ? kShapeCopied : 0u);
     nvtx_push("rs upsweep");
     cudaError_t e = upsweep(a, passes, L, true, fills, shape, copy);
     nvtx_pop();
@@ -225,7 +225,8 @@ struct FusedSort {
     uint64_t zero_vec4 = L.status_bytes / 16;
     Knobs knobs = a.knobs;
     KeyXf<K> xf = make_key_xf<K>(a.key_kind, a.descending);
-    uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 | 2u << 24;
+    uint32_t shape = uint32_t(sizeof(K)) | uint32_t(VB) << 8 | uint32_t(passes) << 16 |
+                     2u << 24 | (copy ? kShapeCopied : 0u);
     void* args[] = {&k0, &k1, &v0, &v1, &n, &begin, &end, &np, &counts, &lay, &tiles, &zero_base,
                     &zero_vec4, &ctrl, &knobs, &xf, &shape, &copy};
     cudaLaunchConfig_t cfg = {};
@@ -240,7 +241,8 @@ struct FusedSort {
     cfg.numAttrs = 1;
     prof_before(a.stream);
     e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), args);
-    prof_after(a.stream, 1, double(a.n) * (sizeof(K) + passes * 2.0 * (sizeof(K) + VB)));
+    prof_after(a.stream, 1, double(a.n) * (sizeof(K) + (copy ? sizeof(K) + 2.0 * VB : 0.0) +
+                                           passes * 2.0 * (sizeof(K) + VB)));
     return e;
   }
 

@@ -97,3 +97,28 @@ def test_in_place_captured(n):
         ek, ev = oracle.lsd_sort(hk, hv, begin_bit=0, end_bit=20)
         assert np.array_equal(from_dev(k, np.uint32), ek)
         assert np.array_equal(from_dev(v, np.uint32), ev)
+
+
+@pytest.mark.parametrize("dt", [np.uint32, np.uint64])
+@pytest.mark.parametrize("pairs", [False, True])
+def test_the_record_counts_the_copy(dt, pairs):
+    """rs_workspace_stats: n K for the histograms, 2 n (K + V) per moving pass,
+    and n (K + 2 V) for the copy that an odd number of passes starts from."""
+    kb = np.dtype(dt).itemsize
+    vb = kb if pairs else 0
+    n = 100003
+    stream = torch.cuda.current_stream().cuda_stream
+    hk = np.random.default_rng(3).integers(0, 2 ** 32, n, dtype=dt)
+    for variant in forms(kb, vb):
+        for end, passes in ((24, 3), (32, 4), (5, 1)):
+            k = to_dev(hk, torch)
+            v, ka, va = (torch.zeros_like(k) for _ in range(3))
+            ws = rs.workspace(kb, vb, n, 0, end, variant=variant)
+            rs.check(rs.rs_sort_in_place(kb, vb, k.data_ptr(), v.data_ptr() if pairs else None,
+                                         ka.data_ptr(), va.data_ptr() if pairs else None, n, 0,
+                                         end, ws.data_ptr(), ws.numel(), stream, variant=variant))
+            st, s = rs.rs_workspace_stats(ws.data_ptr(), stream)
+            rs.check(st)
+            assert s["passes"] == passes and s["moved_mask"] == (1 << passes) - 1
+            copy = n * (kb + 2 * vb) if passes & 1 else 0
+            assert s["bytes"] == n * kb + copy + passes * 2 * n * (kb + vb), (variant, passes)
