@@ -28,7 +28,8 @@ enum DbgSite : uint32_t {
   kSiteGroupInc, kSiteKeyScatter, kSiteValScatter, kSiteFusedCounts, kSiteFusedClear,
   kSiteClusterOut, kSiteSmallOut, kSiteSegPlan, kSiteSegCounts, kSiteSegClear, kSiteSegState,
   kSiteSegSmallOut, kSiteMergeTile, kSiteMergeSplit, kSiteMergeOut, kSiteSampleOff,
-  kSiteSampleSample, kSiteSampleSplitter, kSiteSampleCount, kSiteSampleOut, kSiteSampleBucket
+  kSiteSampleSample, kSiteSampleSplitter, kSiteSampleCount, kSiteSampleOut, kSiteSampleBucket,
+  kSiteCopyKeys, kSiteCopyVals
 };
 
 namespace {

@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
   const K* kin = copy ? k1 : k0;
   if constexpr (VB > 0) {
     if (copy)
-      for (uint32_t i = blockIdx.x * THREADS + tid; i < n; i += gridDim.x * THREADS) v0[i] = v1[i];
+      for (uint32_t i = blockIdx.x * THREADS + tid; i < n; i += gridDim.x * THREADS)
+        if (dbg_ok(i, n, kSiteCopyVals)) v0[i] = v1[i];
   }
   auto count_all = [&](auto XF) {
     constexpr int LOADS = 4;  // in flight per thread
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
 #pragma unroll
       for (uint32_t u = 0; u < LOADS; ++u) {
         if (i0 + u * stride >= n) break;
-        if (copy) k0[i0 + u * stride] = k[u];
+        if (copy && dbg_ok(i0 + u * stride, n, kSiteCopyKeys)) k0[i0 + u * stride] = k[u];
         if constexpr (decltype(XF)::value) k[u] = xf_fwd(k[u], xf);
 #pragma unroll
         for (int p = 0; p < MAXP; ++p) {

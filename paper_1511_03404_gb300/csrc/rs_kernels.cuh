@@ -275,7 +275,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (((va ^ reinterpret_cast<uintptr_t>(vals_to)) & 15u) == 0u) {
         const uint32_t vhead = min(uint32_t(((16u - (va & 15u)) & 15u) / sizeof(K)), n);
         const uint32_t nv = (n - vhead) / VEC;
-        if (blockIdx.x == 0 && uint32_t(tid) < vhead) vals_to[tid] = vals[tid];
+        if (blockIdx.x == 0 && uint32_t(tid) < vhead && dbg_ok(tid, n, kSiteCopyVals))
+          vals_to[tid] = vals[tid];
         const uint4* src = reinterpret_cast<const uint4*>(vals + vhead);
         uint4* dst = reinterpret_cast<uint4*>(vals_to + vhead);
         for (uint32_t base = blockIdx.x * THREADS + tid; base < nv; base += stride * UNROLL) {
@@ -285,23 +286,28 @@ __global__ void __launch_bounds__(THREADS, 1)
             if (base + uint32_t(u) * stride < nv) buf[u] = src[base + uint32_t(u) * stride];
 #pragma unroll
           for (int u = 0; u < UNROLL; ++u)
-            if (base + uint32_t(u) * stride < nv) dst[base + uint32_t(u) * stride] = buf[u];
+            if (base + uint32_t(u) * stride < nv &&
+                dbg_ok(vhead + uint64_t(base + uint32_t(u) * stride) * VEC + (VEC - 1), n,
+                       kSiteCopyVals))
+              dst[base + uint32_t(u) * stride] = buf[u];
         }
         done = vhead + nv * VEC;
       }
       for (uint32_t i = done + blockIdx.x * THREADS + tid; i < n; i += stride)
-        vals_to[i] = vals[i];
+        if (dbg_ok(i, n, kSiteCopyVals)) vals_to[i] = vals[i];
     }
   }
   auto count_all = [&](auto XF) {
     if (blockIdx.x == 0) {
       if (uint32_t(tid) < head) {
         count_key(keys[tid], XF);
-        if constexpr (COPY) keys_to[tid] = keys[tid];
+        if constexpr (COPY)
+          if (dbg_ok(tid, n, kSiteCopyKeys)) keys_to[tid] = keys[tid];
       }
       if (uint32_t(tid) < n - tail) {
         count_key(keys[tail + tid], XF);
-        if constexpr (COPY) keys_to[tail + tid] = keys[tail + tid];
+        if constexpr (COPY)
+          if (dbg_ok(tail + tid, n, kSiteCopyKeys)) keys_to[tail + tid] = keys[tail + tid];
       }
     }
     for (uint32_t base = blockIdx.x * THREADS + tid; base < nvec; base += stride * UNROLL) {
@@ -317,9 +323,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (i < nvec) {
           const K* ks = reinterpret_cast<const K*>(&buf[u]);
           if constexpr (COPY) {
-            if (kvec) {
+            const bool in = dbg_ok(head + uint64_t(i) * VEC + (VEC - 1), n, kSiteCopyKeys);
+            if (in && kvec) {
               reinterpret_cast<uint4*>(keys_to + head)[i] = buf[u];
-            } else {
+            } else if (in) {
 #pragma unroll
               for (int e = 0; e < VEC; ++e) keys_to[head + i * VEC + e] = ks[e];
             }

@@ -4,6 +4,10 @@ one, two and three passes, in every form that can end in the alternate
 buffers, with the four arrays starting at 16-byte boundaries, all one element
 past one, or each at its own offset (the copy then goes by elements), against
 the oracle; nothing around the arrays may change."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -57,6 +61,9 @@ def test_in_place(dt, pairs, offsets, bits):
             if pairs:
                 before[1][ov:ov + n] = ev
             what = (variant, n)
+            if rs.debug_library():
+                st, is_debug, site, index = rs.rs_debug_status()
+                assert is_debug and st == rs.RS_OK, (what, site, index)
             assert np.array_equal(from_dev(bk, dt), before[0]), what
             assert np.array_equal(from_dev(bv, dt), before[1]), what
             for b, a, o in zip((bka, bva), alts, offsets[2:]):
@@ -122,3 +129,15 @@ def test_the_record_counts_the_copy(dt, pairs):
             assert s["passes"] == passes and s["moved_mask"] == (1 << passes) - 1
             copy = n * (kb + 2 * vb) if passes & 1 else 0
             assert s["bytes"] == n * kb + copy + passes * 2 * n * (kb + vb), (variant, passes)
+
+
+def test_in_place_under_the_debug_build():
+    """The same calls with every store's index checked, those of the copy among them."""
+    if rs.debug_library():
+        pytest.skip("already the debug build")
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.abspath(__file__), "-m", "gpu",
+                        "-x", "-q", "-p", "no:cacheprovider", "-k", "not under_the_debug_build"],
+                       env=dict(os.environ, RS_LIBRARY="debug"), capture_output=True, text=True,
+                       timeout=900)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
+    assert " passed" in r.stdout and "failed" not in r.stdout
