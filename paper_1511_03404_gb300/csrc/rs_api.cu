@@ -132,6 +132,7 @@ static std::atomic<long long> g_trace_ptr{0};
 static std::atomic<long long> g_trace_tiles{0};
 static std::atomic<long long> g_trace_pass{0};
 static std::atomic<long long> g_mirror{0};
+static std::atomic<long long> g_repairs_ptr{0};
 static std::atomic<long long> g_dbg_bad_tile{-1};
 
 bool pdl_enabled() {
@@ -165,7 +166,8 @@ Knobs knobs_now() {
   k.trace = reinterpret_cast<uint64_t*>(g_trace_ptr.load());
   k.trace_tiles = uint32_t(g_trace_tiles.load());
   k.trace_pass = int32_t(g_trace_pass.load());
-  k.mirror = int32_t(g_mirror.load());
+  k.order.mirror = int32_t(g_mirror.load());
+  k.order.repairs = reinterpret_cast<uint32_t*>(g_repairs_ptr.load());
   k.dbg_bad_tile = int32_t(g_dbg_bad_tile.load());
   return k;
 }
@@ -806,6 +808,9 @@ rs_status rs_debug_set(rs_debug_knob knob, long long value) {
 #else
       g_mirror.store(value != 0);
 #endif
+      return RS_OK;
+    case RS_DEBUG_REPAIRS_PTR:
+      g_repairs_ptr.store(value);
       return RS_OK;
     case RS_DEBUG_BAD_INDEX_TILE:
 #ifdef RS_DEBUG

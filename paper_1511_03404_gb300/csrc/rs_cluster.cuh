@@ -89,7 +89,7 @@ struct ClusterSmem {
 template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 __global__ void __launch_bounds__(THREADS, 1)
     k_cluster_sort(K* __restrict__ keys, ValT<VB>* __restrict__ vals, uint32_t n, uint32_t slice,
-                   int begin_bit, int end_bit, Ctrl* ctrl, KeyXf<K> xf, bool mirror) {
+                   int begin_bit, int end_bit, Ctrl* ctrl, KeyXf<K> xf, OrderTest order) {
   using V = ValT<VB>;
   using S = ClusterSmem<K, RADIX_BITS, THREADS, ITEMS, INDEX>;
   constexpr int RADIX = S::RADIX, WARPS = S::WARPS;
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   int src = 0;
   for (int attempt = 0; attempt < 2; ++attempt) {
     const bool careful = attempt != 0;
-    const uint32_t slot0 = uint32_t(warp * items * 32 + (mirror && !careful ? 31 - lane : lane));
+    const uint32_t slot0 = uint32_t(warp * items * 32 + (order.mirror && !careful ? 31 - lane : lane));
     src = 0;
     {
       K* ks = reinterpret_cast<K*>(smem + S::KEYS);
@@ -284,6 +284,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t found = 0u;
     for (uint32_t q = 0; q < ncta; ++q) found |= s_flags[q];
     if (!found) break;  // the same in every CTA
+    if (!careful && rank == 0u && tid == 0 && order.repairs != nullptr)
+      atomicAdd(order.repairs, 1u);
   }
 
   // write this CTA's slice out (untransformed): everything is read before the

@@ -61,6 +61,15 @@ static_assert(sizeof(Ctrl) == 256, "Ctrl must be 256 bytes");
 
 constexpr uint32_t kShapeCopied = 1u << 23;
 
+// Test-only: the order in which ranks are drawn.
+struct OrderTest {
+  uint32_t* repairs;       // device counter of tiles put in order and of sorts inside a CTA or
+                           // cluster done again, or null
+  int32_t mirror;          // 1: every warp's lanes take their keys in reverse, so that equal
+                           // digits draw their ranks out of turn; 2 (digit passes of debug
+                           // builds): out of turn from item to item too
+};
+
 // Test-only fault injection and the bound on every device-side wait.
 struct Knobs {
   uint64_t timeout_ns;     // a look-back wait gives up after this long
@@ -69,9 +78,7 @@ struct Knobs {
   uint64_t* trace;         // device [trace_tiles][16] phase timestamps (ns) and counters, or null
   uint32_t trace_tiles;    // tiles 0 .. trace_tiles-1 of trace_pass are recorded
   int32_t trace_pass;
-  int32_t mirror;          // test-only: 1, every warp's lanes take their keys in reverse, so that
-                           // equal digits draw their ranks out of turn; 2 (digit passes of
-                           // debug builds), out of turn from item to item too
+  OrderTest order;
   int32_t dbg_bad_tile;    // debug builds only: this tile of pass 0 computes scatter
                            // indices past the array, which the bounds checks drop (-1: off)
 };

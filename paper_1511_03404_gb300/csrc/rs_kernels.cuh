@@ -458,8 +458,7 @@ struct TileArgs {
   int32_t drop_tile;            // test-only: this tile publishes nothing (-1: none)
   int32_t bad_tile;             // debug builds, test-only: this tile's scatter indices are
                                 // pushed past n (-1: none)
-  int32_t mirror;               // test-only: 1, lanes take their keys in reverse; 2 (debug
-                                // builds), a warp's slots of a digit are taken in reverse
+  OrderTest order;              // test-only
   bool xin;                     // the source holds untransformed keys: apply xf on load
   bool xout;                    // write untransformed keys (apply xf's inverse)
 };
@@ -961,7 +960,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   // of lane l is slot w*ITEMS*32 + j*32 + l.  mirror 1 (test-only): the lanes
   // are taken in reverse, so that every repeated digit draws out of turn.
   K* s_kin = Stage<K>(t.ksrc + tile_base, tile_len).at(smem + S::KIN);
-  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (t.mirror == 1 ? 31 - lane : lane));
+  const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (t.order.mirror == 1 ? 31 - lane : lane));
   uint32_t* wh = s_wh + warp * RADIX;
   // a tile's keys are its first tile_len slots; the rest draw nothing
   const uint32_t lim = tile_len - min(slot0, tile_len);  // item j is a key if j * 32 < lim
@@ -1091,7 +1090,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   else
     stage(std::false_type{});
   if constexpr (kDebugChecks) {
-    if (t.mirror == 2) {  // test-only: as if each warp's draws had come last item first
+    if (t.order.mirror == 2) {  // test-only: as if each warp's draws had come last item first
       __syncthreads();
       if (tid < RADIX) {
         uint32_t at = my_start;
@@ -1242,6 +1241,7 @@ __device__ __forceinline__ bool onesweep_tile(uint32_t tile, Ctrl* ctrl, uint64_
   bool ok = check(bad, 5) == 0u;
   const bool repaired = !ok;
   if (!ok) {
+    if (tid == 0 && t.order.repairs != nullptr) atomicAdd(t.order.repairs, 1u);
     // out of turn.  A warp draws a digit's slots from a range that no other
     // warp draws from, and the ranges are in order, so that no element is further
     // from its place than such a range is long (at most ITEMS * 32): that many
@@ -1348,7 +1348,7 @@ __device__ __forceinline__ void pass_args(
   t->tiles = tiles;
   t->xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
   t->xout = xf.on && pass == 31 - __clz(exec);
-  t->mirror = knobs.mirror;
+  t->order = knobs.order;
   t->drop_tile = pass == knobs.drop_pass ? knobs.drop_tile : -1;
   t->bad_tile = kDebugChecks && pass == 0 ? knobs.dbg_bad_tile : -1;
   t->trace = pass == knobs.trace_pass ? knobs.trace : nullptr;
@@ -1499,7 +1499,7 @@ template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* kout,
                                          ValT<VB>* vout, uint32_t len, int begin_bit,
                                          int end_bit, unsigned char* smem, const KeyXf<K>& xf,
-                                         bool mirror) {
+                                         const OrderTest& order) {
   using V = ValT<VB>;
   using S = SmallSmem<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>;
   constexpr int RADIX = S::RADIX, WARPS = S::WARPS;
@@ -1524,7 +1524,7 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
     const bool careful = attempt != 0;
     // item j of lane l of warp w is element (w * items + j) * 32 + l
     const uint32_t slot0 =
-        uint32_t(warp * items * 32 + (mirror && !careful ? 31 - lane : lane));
+        uint32_t(warp * items * 32 + (order.mirror && !careful ? 31 - lane : lane));
     for (uint32_t i = tid; i < len; i += THREADS) {
       const K k = kin[i];
       s_k[i] = xf.on ? xf_fwd(k, xf) : k;
@@ -1615,6 +1615,7 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
       else bad = bad || a > b;
     }
     if (!__syncthreads_or(bad)) break;
+    if (!careful && tid == 0 && order.repairs != nullptr) atomicAdd(order.repairs, 1u);
   }
   // (a test of the length instead left the 1024 x 16 form for 64-bit pairs 40
   // bytes of spills and 5 % slower)
@@ -1643,7 +1644,7 @@ __device__ __forceinline__ void cta_sort(const K* kin, const ValT<VB>* vin, K* k
 template <class K, int VB, int RADIX_BITS, int THREADS, int ITEMS, bool INDEX>
 __global__ void __launch_bounds__(THREADS, 1)
     k_small_sort(K* keys, ValT<VB>* vals, uint32_t n, int begin_bit, int end_bit, Ctrl* ctrl,
-                 KeyXf<K> xf, bool mirror) {
+                 KeyXf<K> xf, OrderTest order) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int passes = (end_bit - begin_bit + RADIX_BITS - 1) / RADIX_BITS;
   if (ctrl != nullptr && threadIdx.x == 0) {
@@ -1655,7 +1656,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                             3u << 24);
   }
   cta_sort<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>(keys, vals, keys, vals, n, begin_bit, end_bit,
-                                                     smem, xf, mirror);
+                                                     smem, xf, order);
   __syncthreads();
   if (ctrl != nullptr && threadIdx.x == 0) ctrl->t_upsweep = stat_now(ctrl);
 }

@@ -289,8 +289,8 @@ struct ClusterSort {
     uint32_t n = a.n;
     int begin = a.begin_bit, end = a.end_bit;
     KeyXf<K> xf = make_key_xf<K>(a.key_kind, a.descending);
-    bool mirror = a.knobs.mirror != 0;
-    void* args[] = {&keys, &vals, &n, &slice, &begin, &end, &ctrl, &xf, &mirror};
+    OrderTest order = a.knobs.order;
+    void* args[] = {&keys, &vals, &n, &slice, &begin, &end, &ctrl, &xf, &order};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncta);
     cfg.blockDim = dim3(THREADS);
@@ -352,7 +352,7 @@ struct SmallSort {
     kern<<<1, THREADS, S::BYTES, a.stream>>>(static_cast<K*>(a.keys), static_cast<V*>(a.vals),
                                              a.n, a.begin_bit, a.end_bit, ctrl,
                                              make_key_xf<K>(a.key_kind, a.descending),
-                                             a.knobs.mirror != 0);
+                                             a.knobs.order);
     const cudaError_t e = cudaGetLastError();
     prof_after(a.stream, 2, 2.0 * double(a.n) * double(sizeof(K) + VB));
     return e;

@@ -160,7 +160,8 @@ struct MsTileSmem {
 // pass, but leave one CTA an SM for 128-bit keys: 275 us instead of 203.
 template <class K, class V, bool HAS_V>
 __global__ void __launch_bounds__(MsTileSmem<K>::THREADS, MsTileSmem<K>::MINB)
-    k_ms_tile(const K* src, const V* vsrc, K* dst, V* vdst, uint32_t n, bool mirror) {
+    k_ms_tile(const K* src, const V* vsrc, K* dst, V* vdst, uint32_t n,
+              OrderTest order) {
   using S = MsTileSmem<K>;
   constexpr int THREADS = S::THREADS, ITEMS = S::ITEMS, WARPS = S::WARPS, WORDS = S::WORDS;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(MsTileSmem<K>::THREADS, MsTileSmem<K>::MINB)
   for (int attempt = 0; attempt < 2; ++attempt) {
     const bool careful = attempt != 0;
     // item j of lane l of warp w is place (w * ITEMS + j) * 32 + l
-    const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (mirror && !careful ? 31 - lane : lane));
+    const uint32_t slot0 = uint32_t(warp * ITEMS * 32 + (order.mirror && !careful ? 31 - lane : lane));
 #pragma unroll
     for (int t = 0; t < ITEMS; ++t) s_pos[t * THREADS + tid] = uint16_t(t * THREADS + tid);
     for (int i = tid; i < WARPS * 256 / 4; i += THREADS)
@@ -273,6 +274,7 @@ __global__ void __launch_bounds__(MsTileSmem<K>::THREADS, MsTileSmem<K>::MINB)
       bad = bad || !ordered;
     }
     if (!__syncthreads_or(bad)) break;
+    if (!careful && tid == 0 && order.repairs != nullptr) atomicAdd(order.repairs, 1u);
   }
   // in place: every value is read before the first is written
   V v[HAS_V ? ITEMS : 1];
@@ -438,7 +440,7 @@ struct MergeSort {
     const uint32_t nt = tiles(n);
     prof_before(s);
     tile_k<<<unsigned((n + kTile - 1) / kTile), T::THREADS, T::BYTES, s>>>(bufk[0], bufv[0], bufk[0], bufv[0], uint32_t(n),
-                                            knobs_now().mirror != 0);
+                                            knobs_now().order);
     cudaError_t e = cudaGetLastError();
     prof_after(s, RS_KERNEL_MERGE, 2.0 * double(n) * double(sizeof(K) + (HAS_V ? sizeof(V) : 0)));
     if (e != cudaSuccess) return e;

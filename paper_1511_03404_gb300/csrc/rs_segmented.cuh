@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     const uint32_t len = uint32_t(a.off[s + 1] - b);
     cta_sort<K, VB, RADIX_BITS, THREADS, ITEMS, INDEX>(k0 + b, v0 + b, kout + b, vout + b, len,
                                                        a.begin_bit, a.end_bit, smem,
-                                                       KeyXf<K>{}, a.knobs.mirror != 0);
+                                                       KeyXf<K>{}, a.knobs.order);
     __syncthreads();
   }
   const uint32_t warps = gridDim.x * (THREADS / 32);

@@ -36,7 +36,7 @@ KERNEL_NAMES = ("upsweep", "onesweep", "small", "segmented", "merge", "sample")
 
 (RS_DEBUG_TIMEOUT_NS, RS_DEBUG_DROP_PUBLISH_TILE, RS_DEBUG_DROP_PUBLISH_PASS, RS_DEBUG_TRACE_PTR,
  RS_DEBUG_TRACE_TILES, RS_DEBUG_TRACE_PASS, RS_DEBUG_LB_SMALL, RS_DEBUG_BAD_INDEX_TILE,
- RS_DEBUG_MIRROR_LANES) = range(9)
+ RS_DEBUG_MIRROR_LANES, RS_DEBUG_REPAIRS_PTR) = range(10)
 
 
 class RsError(RuntimeError):

@@ -56,6 +56,26 @@ def merge_via_abi(k, v, kb, vb):
             from_dev(va if alt else dv, v.dtype) if vb else None)
 
 
+class Repairs:
+    """The library's count of tiles put in order and of sorts done again."""
+
+    def __init__(self):
+        self.count = torch.zeros(1, dtype=torch.int32, device="cuda")
+        rs.check(rs.rs_debug_set(rs.RS_DEBUG_REPAIRS_PTR, self.count.data_ptr()))
+
+    def take(self):
+        n = int(self.count.item())
+        self.count.zero_()
+        return n
+
+
+@pytest.fixture
+def repairs():
+    yield Repairs()
+    torch.cuda.synchronize()
+    rs.check(rs.rs_debug_set(rs.RS_DEBUG_REPAIRS_PTR, 0))
+
+
 @pytest.fixture
 def mirrored():
     rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 1))
@@ -64,7 +84,7 @@ def mirrored():
 
 
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
-def test_out_of_turn_ranks_are_repaired(dtype, pairs, mirrored):
+def test_out_of_turn_ranks_are_repaired(dtype, pairs, mirrored, repairs):
     kb = np.dtype(dtype).itemsize
     for var in variants(kb, kb if pairs else 0, (0, 1, 2, 3, 4)):
         tile = var["threads"] * var["items"]
@@ -78,13 +98,28 @@ def test_out_of_turn_ranks_are_repaired(dtype, pairs, mirrored):
                             ("few", inputs.keys(dtype, "uniform", n) & dtype(0x0303)),
                             ("sorted_desc", inputs.keys(dtype, "sorted_desc", n))):
                 check(k, v, (name, n, var), variant=var["index"])
+                # every digit has repeats in some warp from here on
+                assert repairs.take() > 0 or name != "uniform" or n < 1000, (n, var)
             check(inputs.keys(dtype, "uniform", n), v, ("bits", n, var), variant=var["index"],
                   begin_bit=3, end_bit=17)
+            assert repairs.take() > 0 or n < 1000, ("bits", n, var)
+
+
+@pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
+def test_how_often_the_hardware_draws_out_of_turn(dtype, pairs, repairs):
+    """Without the knob: the count of repairs is printed (-s), any is allowed."""
+    kb = np.dtype(dtype).itemsize
+    for var in variants(kb, kb if pairs else 0, (0, 1, 2, 3, 4)):
+        n = min(var["max_n"], 40 * var["threads"] * var["items"] + 3)
+        check(inputs.keys(dtype, "gaussian", n), inputs.values(dtype, n) if pairs else None, var,
+              variant=var["index"])
+        print(f"k{kb} v{kb if pairs else 0} variant {var['index']}, {n} elements: "
+              f"{repairs.take()} repairs")
 
 
 @pytest.mark.parametrize("mirror", [0, 1])
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
-def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
+def test_tiles_around_the_look_back_levels(dtype, pairs, mirror, repairs):
     kb = np.dtype(dtype).itemsize
     try:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, mirror))
@@ -96,6 +131,7 @@ def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
                 n = tiles * tile - 3
                 v = inputs.values(dtype, n) if pairs else None
                 check(inputs.keys(dtype, "gaussian", n), v, (n, var), variant=var["index"])
+                assert not mirror or repairs.take() >= tiles, (n, var)  # in some pass each tile
                 if not pairs and not mirror:
                     check(inputs.keys(dtype, "gaussian", n), v, (n, var, "bits"),
                           variant=var["index"], begin_bit=0, end_bit=20)
@@ -105,7 +141,7 @@ def test_tiles_around_the_look_back_levels(dtype, pairs, mirror):
 
 @pytest.mark.parametrize("mirror", [0, 1])
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
-def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
+def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror, repairs):
     """Empty, one-warp (up to 32), one-CTA (every number of items a thread, and
     the larger CTAs of medium ones) and tiled segments, more of them than one
     round of the planner takes."""
@@ -119,6 +155,8 @@ def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
     n = int(off[-1])
     kb = np.dtype(dtype).itemsize
     v = inputs.values(dtype, n) if pairs else None
+    # segments of a CTA or more with keys enough for repeats in some warp
+    certain = sum(int(x) >= 1000 for x in lengths)
     try:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, mirror))
         for k in (inputs.keys(dtype, "uniform", n), inputs.keys(dtype, "uniform", n) & dtype(0x303)):
@@ -129,13 +167,14 @@ def test_segments_around_the_one_warp_and_one_cta_forms(dtype, pairs, mirror):
                 ek, ev = oracle.segmented_sort(k, v, off, begin_bit=begin, end_bit=end)
                 assert np.array_equal(from_dev(dk, dtype), ek), (begin, end)
                 assert not pairs or np.array_equal(from_dev(dv, dtype), ev), (begin, end)
+                assert not mirror or repairs.take() >= certain, (begin, end)
     finally:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
 
 
 @pytest.mark.parametrize("mirror", [0, 1])
 @pytest.mark.parametrize("kb,vb", [(4, 0), (4, 4), (8, 0), (8, 8), (16, 0), (16, 8)])
-def test_merge_tiles_by_bytes(kb, vb, mirror):
+def test_merge_tiles_by_bytes(kb, vb, mirror, repairs):
     """The merge sort's tiles: bytes that are the same in a whole tile are
     left out, few-valued ones repeat in every warp."""
     rng = np.random.default_rng(3)
@@ -155,12 +194,14 @@ def test_merge_tiles_by_bytes(kb, vb, mirror):
                 ek, ev = oracle.sort_wide(k, v) if kb == 16 else oracle.lsd_sort(k, v)
                 assert np.array_equal(gk, ek), (n, mask)
                 assert not vb or np.array_equal(gv, ev), (n, mask)
+                # equal keys are out of turn everywhere, distinct ones in some byte
+                assert not mirror or repairs.take() >= n // 4096 or mask == 0, (n, mask)
     finally:
         rs.check(rs.rs_debug_set(rs.RS_DEBUG_MIRROR_LANES, 0))
 
 
 @pytest.mark.parametrize("dtype,pairs", TYPES, ids=TYPE_IDS)
-def test_any_order_of_a_warps_draws_is_repaired(dtype, pairs):
+def test_any_order_of_a_warps_draws_is_repaired(dtype, pairs, repairs):
     """A warp's keys of one digit in reverse, across its items: up to all the
     keys of a warp are out of place, and by as many places."""
     if not rs.debug_library():
@@ -178,6 +219,7 @@ def test_any_order_of_a_warps_draws_is_repaired(dtype, pairs):
                     check(k, v, (name, n, var), variant=var["index"])
                     check(k, v, (name, "bits", n, var), variant=var["index"], begin_bit=3,
                           end_bit=17)
+                    assert repairs.take() > 0 or n < 1000, (name, n, var)
         rng = np.random.default_rng(5)
         off = inputs.offsets_from_lengths(np.asarray([30011, 70001, 20481, 5, 100000], np.uint64))
         n = int(off[-1])
