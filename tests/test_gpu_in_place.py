@@ -106,6 +106,54 @@ def test_in_place_captured(n):
         assert np.array_equal(from_dev(v, np.uint32), ev)
 
 
+ORDERS = [(oracle.KEY_UNSIGNED, False), (oracle.KEY_UNSIGNED, True), (oracle.KEY_SIGNED, False),
+          (oracle.KEY_FLOAT, True)]
+ORDER_IDS = ["unsigned", "unsigned_desc", "signed", "float_desc"]
+
+
+@pytest.mark.parametrize("dt", [np.uint32, np.uint64])
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("kind,desc", ORDERS, ids=ORDER_IDS)
+def test_in_place_orders_and_skipped_passes(dt, pairs, kind, desc):
+    """Odd numbers of passes in every key order: the copy holds the keys as
+    they came, the first pass that moves data transforms them.  Whole 32-bit keys
+    at 7 bits a digit (five passes), where keys are staged themselves, and bit
+    ranges of three; keys of which every pass moves data, some, or none."""
+    rng = np.random.default_rng(13)
+    kb = np.dtype(dt).itemsize
+    vb = kb if pairs else 0
+    stream = torch.cuda.current_stream().cuda_stream
+    cases = [(i, bits) for i in forms(kb, vb) for bits in ((0, 20), (8 * kb - 20, 8 * kb))]
+    cases += [(i, (0, 32)) for i in range(rs.rs_num_variants(kb, vb)) if kb == 4
+              and rs.rs_variant_info(kb, vb, i)["radix_bits"] == 7]
+    assert len(cases) == 6 + (kb == 4)
+    for variant, bits in cases:
+        info = rs.rs_variant_info(kb, vb, variant)
+        assert -(-(bits[1] - bits[0]) // info["radix_bits"]) & 1
+        for n in (33, 100003):
+            for mask in (~0, 0xff << bits[0], 0x3 << (bits[1] - 2), 0):
+                hk = rng.integers(0, 2 ** (8 * kb) - 1, n, dtype=dt, endpoint=True)
+                hk &= dt(mask & (2 ** (8 * kb) - 1))
+                hv = rng.integers(0, 2 ** 32, n, dtype=dt)
+                k, v = to_dev(hk, torch), to_dev(hv, torch)
+                ka, va = torch.zeros_like(k), torch.zeros_like(k)
+                ws = rs.workspace(kb, vb, n, *bits, variant=variant)
+                rs.check(rs.rs_sort_in_place(kb, vb, k.data_ptr(), v.data_ptr() if pairs else None,
+                                             ka.data_ptr(), va.data_ptr() if pairs else None, n,
+                                             *bits, ws.data_ptr(), ws.numel(), stream,
+                                             variant=variant, key_kind=kind, descending=desc))
+                st, s = rs.rs_workspace_stats(ws.data_ptr(), stream)
+                rs.check(st)
+                what = (variant, bits, n, mask)
+                assert s["moved_mask"].bit_count() & 1, what  # from the copy back to the keys
+                if kind == oracle.KEY_UNSIGNED and mask == 0:
+                    assert s["moved_mask"] == 1, what
+                ek, ev = oracle.ordered_sort(hk, hv, kind=kind, descending=desc,
+                                             begin_bit=bits[0], end_bit=bits[1])
+                assert np.array_equal(from_dev(k, dt), ek), what
+                assert np.array_equal(from_dev(v, dt), ev if pairs else hv), what
+
+
 @pytest.mark.parametrize("dt", [np.uint32, np.uint64])
 @pytest.mark.parametrize("pairs", [False, True])
 def test_the_record_counts_the_copy(dt, pairs):
