@@ -1,7 +1,7 @@
 // The whole sort inside one thread-block cluster, for arrays up to
-// CL x THREADS x ITEMS elements: every digit pass (Sec. 2.6) runs on data held
-// in the cluster's shared memory, with no trip through global memory and no
-// kernel boundary between passes.
+// 8 x THREADS x ITEMS elements (65,536), whether on 8 CTAs or 16: every digit
+// pass (Sec. 2.6) runs on data held in the cluster's shared memory, with no
+// trip through global memory and no kernel boundary between passes.
 //
 // CTA c of the cluster owns positions [c * slice, (c + 1) * slice) of the
 // array; the slice follows the length, so that every CTA takes part.  One

@@ -80,7 +80,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
   constexpr int RADIX = F::RADIX, MAXP = F::MAXP;
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* s_hist = reinterpret_cast<uint32_t*>(smem + S::WH);
-  uint32_t* s_tot = reinterpret_cast<uint32_t*>(smem + S::TOT);
   uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + S::MISC);
   uint32_t* s_off = reinterpret_cast<uint32_t*>(smem + F::OFF);
   uint32_t* s_flag = reinterpret_cast<uint32_t*>(smem + F::FLAG);

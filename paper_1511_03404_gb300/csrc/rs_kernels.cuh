@@ -5,13 +5,14 @@
 //               pass (the "count" step of each counting sort); its last CTA
 //               takes the exclusive scan of each histogram (the "prefix"
 //               step) and decides which passes move data.
-//   k_onesweep  one digit pass: the tile's keys are ranked within the tile
-//               (stable: warp-major, then item, then lane order), the tile's
-//               digit counts are published for the following tiles, the
-//               tile's global digit offsets come from a decoupled look-back
-//               over the preceding tiles, and the tile is scattered through
-//               shared memory so that each digit run is written contiguously
-//               (the stable "scatter" step).
+//   k_onesweep  one digit pass: the tile's digit counts are published for the
+//               following tiles, then its keys draw their places in the tile
+//               (stable: warp-major, then item, then lane order, checked and
+//               put right where the draws came in another order), the tile's
+//               global digit offsets come from a look-back over the preceding
+//               tiles, and the tile is scattered through shared memory so that
+//               each digit run is written contiguously (the stable "scatter"
+//               step).
 //   k_small_sort  arrays that fit one tile: all passes in one CTA, in shared
 //               memory, in a single launch.
 // All arithmetic is on unsigned integers; results are exact.
@@ -128,10 +129,6 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-
-__device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Bounded wait until *p >= target.  False when it ran out or another CTA
@@ -453,7 +450,6 @@ struct TileArgs {
   uint32_t n;                   // elements of the array / segment
   uint32_t shift, mask;         // digit of this pass: (key >> shift) & mask
   uint32_t tile0;               // index of this array's tile 0 in status (a segment's first tile)
-  uint32_t tiles;               // tiles of this array
   uint32_t trace_tiles;         // test-only: tiles the trace holds
   int32_t drop_tile;            // test-only: this tile publishes nothing (-1: none)
   int32_t bad_tile;             // debug builds, test-only: this tile's scatter indices are
@@ -1345,7 +1341,6 @@ __device__ __forceinline__ void pass_args(
   t->shift = shift;
   t->mask = mask;
   t->tile0 = 0u;
-  t->tiles = tiles;
   t->xin = xf.on && pass == __ffs(int(exec)) - 1;  // first and last pass that move data
   t->xout = xf.on && pass == 31 - __clz(exec);
   t->order = knobs.order;

@@ -272,7 +272,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
   constexpr int QUEUE = MEDIUM ? kMediumQueue : kSmallQueue;
   const uint32_t* ids = MEDIUM ? a.medium_ids : a.small_ids;
   const uint32_t n_small = a.ctrl->tile_counter[MEDIUM ? kNMedium : kNSmall];
-  const uint32_t n_tiny = MEDIUM ? 0u : a.ctrl->tile_counter[kNTiny];
+  uint32_t n_tiny = 0u;
+  if constexpr (!MEDIUM) n_tiny = a.ctrl->tile_counter[kNTiny];
   const K looked = (a.end_bit - a.begin_bit == 8 * int(sizeof(K)))
                        ? ~K(0)
                        : K(((K(1) << (a.end_bit - a.begin_bit)) - K(1)) << a.begin_bit);
