@@ -92,3 +92,29 @@ def test_a_calls_buffers_are_its_streams(segmented, monkeypatch):
     ek, ev = expected(segmented)
     assert np.array_equal(from_dev(k, np.uint32), ek)
     assert np.array_equal(from_dev(v, np.uint32), ev)
+
+
+def test_sorts_of_several_streams_at_once():
+    """Eight streams, each with its own buffers and workspace, enqueue sorts of
+    every form side by side: one CTA, a cluster, one cooperative launch, ordinary
+    and resident passes, segments; each result against the oracle."""
+    streams = [torch.cuda.Stream() for _ in range(8)]
+    jobs = []
+    for i, n in enumerate([3000, 30000, 50000, 100003, 300007, 1 << 20, 3000017, 70001] * 3):
+        dtype = (np.uint32, np.uint64)[i % 2]
+        k, v = inputs.keys(dtype, "gaussian", n, seed=i + 1), inputs.values(dtype, n)
+        jobs.append((i, k, v, to_dev(k, torch), to_dev(v, torch), i % 3 == 2))
+    off = {n: np.asarray([0, n // 7, n // 2, n], np.uint64) for n in {j[1].size for j in jobs}}
+    doff = {n: to_dev(o, torch) for n, o in off.items()}
+    torch.cuda.synchronize()
+    for i, k, v, dk, dv, segmented in jobs:
+        if segmented:
+            rs.segmented_sort(dk, doff[k.size], dv, 0, 20, stream=streams[i % 8])
+        else:
+            rs.sort(dk, dv, stream=streams[i % 8], key_kind=rs.RS_KEY_UNSIGNED)
+    torch.cuda.synchronize()
+    for i, k, v, dk, dv, segmented in jobs:
+        ek, ev = (oracle.segmented_sort(k, v, off[k.size], begin_bit=0, end_bit=20) if segmented
+                  else oracle.lsd_sort(k, v))
+        assert np.array_equal(from_dev(dk, k.dtype), ek), (i, k.size)
+        assert np.array_equal(from_dev(dv, k.dtype), ev), (i, k.size)
