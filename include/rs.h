@@ -622,9 +622,10 @@ typedef enum rs_debug_knob {
                                      draw their ranks out of turn and every tile needs repair;
                                      2: in the digit passes of a debug build a warp's keys of
                                      one digit come wholly reversed (else as 1) */
-  RS_DEBUG_REPAIRS_PTR = 9,       /* device u32 that counts tiles whose ranks came out of turn
-                                     and were put in order, and sorts inside one CTA or
-                                     cluster done again for that; 0 off */
+  RS_DEBUG_REPAIRS_PTR = 9,       /* debug build only (else RS_ERR_INVALID): device u32 that
+                                     counts tiles whose ranks came out of turn and were put in
+                                     order, and sorts inside one CTA or cluster done again for
+                                     that; 0 off */
   RS_DEBUG_BAD_INDEX_TILE = 7     /* debug build only (else RS_ERR_INVALID): this tile of
                                      digit pass 0 of a multi-launch sort computes scatter
                                      indices past the array, so that the bounds checks of

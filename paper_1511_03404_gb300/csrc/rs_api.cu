@@ -810,8 +810,12 @@ rs_status rs_debug_set(rs_debug_knob knob, long long value) {
 #endif
       return RS_OK;
     case RS_DEBUG_REPAIRS_PTR:
+#ifdef RS_DEBUG
       g_repairs_ptr.store(value);
       return RS_OK;
+#else
+      return RS_ERR_INVALID;  // only a debug build counts
+#endif
     case RS_DEBUG_BAD_INDEX_TILE:
 #ifdef RS_DEBUG
       g_dbg_bad_tile.store(value < 0 ? -1 : value);

@@ -284,8 +284,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t found = 0u;
     for (uint32_t q = 0; q < ncta; ++q) found |= s_flags[q];
     if (!found) break;  // the same in every CTA
-    if (!careful && rank == 0u && tid == 0 && order.repairs != nullptr)
-      atomicAdd(order.repairs, 1u);
+    if (!careful && rank == 0u && tid == 0) count_repair(order);
   }
 
   // write this CTA's slice out (untransformed): everything is read before the

@@ -63,8 +63,8 @@ constexpr uint32_t kShapeCopied = 1u << 23;
 
 // Test-only: the order in which ranks are drawn.
 struct OrderTest {
-  uint32_t* repairs;       // device counter of tiles put in order and of sorts inside a CTA or
-                           // cluster done again, or null
+  uint32_t* repairs;       // debug builds: device counter of tiles put in order and of sorts
+                           // inside a CTA or cluster done again, or null
   int32_t mirror;          // 1: every warp's lanes take their keys in reverse, so that equal
                            // digits draw their ranks out of turn; 2 (digit passes of debug
                            // builds): out of turn from item to item too

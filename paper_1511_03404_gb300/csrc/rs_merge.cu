@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(MsTileSmem<K>::THREADS, MsTileSmem<K>::MINB)
       bad = bad || !ordered;
     }
     if (!__syncthreads_or(bad)) break;
-    if (!careful && tid == 0 && order.repairs != nullptr) atomicAdd(order.repairs, 1u);
+    if (!careful && tid == 0) count_repair(order);
   }
   // in place: every value is read before the first is written
   V v[HAS_V ? ITEMS : 1];
