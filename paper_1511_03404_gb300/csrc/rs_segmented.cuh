@@ -117,7 +117,12 @@ struct SegArgs {
 // Numbers the work, one segment a thread.  Segments longer than medium_max are
 // "long"; of the others, those of 1 to 32 elements are "tiny" (listed from the
 // end of small_ids), those of up to small_max "small", the rest "medium"; empty
-// ones are left out.  The order
+// ones are left out.  Where one CTA sees every segment (up to THREADS of them)
+// and one is long, none is medium: so few medium ones leave SMs idle, one
+// after the other with the long ones' tiles, which they can fill instead (108
+// segments of up to 24,000 u64 keys 175 us with medium ones and 115 without;
+// up to 18,000 u64 pairs 191 and 130; 300 and more took the same or less with
+// them).  The order
 // inside the lists is of no consequence, so each CTA takes its places from
 // global counters: with one CTA scanning all segments in order, 20,000 of them
 // took 87 us.  The state of long segments, and the digit counts of those of
@@ -143,7 +148,9 @@ __global__ void __launch_bounds__(THREADS)
     if (to < from || to > n || to - from > uint64_t((1u << 30) - 1u)) bad = true;
     else len = uint32_t(to - from);
   }
-  const bool tiny = len >= 1u && len <= kTinyMax, lng = len > medium_max;
+  const uint32_t line =
+      gridDim.x == 1u && __syncthreads_or(len > medium_max) ? small_max : medium_max;
+  const bool tiny = len >= 1u && len <= kTinyMax, lng = len > line;
   const bool small = len > kTinyMax && len <= small_max, medium = len > small_max && !lng;
   const uint32_t nt = lng ? (len + tile - 1u) / tile : 0u, nc = lng ? (len + chunk - 1u) / chunk : 0u;
   const uint32_t mine[COUNTS] = {tiny, small, lng, nt, nc, medium};

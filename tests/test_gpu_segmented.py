@@ -219,3 +219,29 @@ def test_torch_segmented_sort_helper():
         dk = to_dev(k, torch)
         rs.segmented_sort(dk, doff)
         assert np.array_equal(from_dev(dk, dt), oracle.segmented_sort(k, None, off)[0])
+
+
+@pytest.mark.parametrize("kb,vb", [(4, 0), (4, 4), (8, 0), (8, 8)],
+                         ids=["k32", "kv32", "k64", "kv64"])
+def test_medium_segments_beside_long_ones(kb, vb):
+    """Where one CTA plans all segments (up to 256) and one of them is long,
+    the medium ones are tiled with it; else they are sorted whole.  Segments
+    of every form on both sides of both lines, against the oracle."""
+    dt = np.uint32 if kb == 4 else np.uint64
+    rng = np.random.default_rng(9)
+    for nseg in (1, 3, 255, 256, 257, 300):
+        for longest in (20480 if kb == 4 else 16384, 20481 if kb == 4 else 16385, 70001):
+            L = rng.integers(0, 6000, nseg)
+            L[rng.integers(0, nseg)] = longest
+            if nseg > 3:
+                L[5:9] = (0, 32, 3072, 4097)
+            off = inputs.offsets_from_lengths(L.astype(np.uint64))
+            n = int(off[-1])
+            k = inputs.keys(dt, "gaussian", n)
+            v = inputs.values(dt, n) if vb else None
+            for begin, end in ((0, 8 * kb), (3, 20)):
+                dk, dv = to_dev(k, torch), to_dev(v, torch) if vb else None
+                rs.segmented_sort(dk, to_dev(off, torch), dv, begin, end)
+                ek, ev = oracle.segmented_sort(k, v, off, begin_bit=begin, end_bit=end)
+                assert np.array_equal(from_dev(dk, dt), ek), (nseg, longest, end)
+                assert not vb or np.array_equal(from_dev(dv, dt), ev), (nseg, longest, end)
