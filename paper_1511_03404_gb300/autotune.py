@@ -28,8 +28,9 @@ from . import rs
 TYPES = ((4, 0), (4, 4), (8, 0), (8, 8))
 # the lengths of the paper's grid (Sec. 3): 2^e and 2^e + 2^(e-1), so that no
 # length of the grid falls between two measured sizes; and the quarters of each
-# octave up to 2^22, where the forms take over from one another (50,000 u32
-# pairs, in a band measured at 2^16 alone, got a form 7 % slower than the best)
+# octave up to 2^22, where the forms take over from one another (in bands of
+# half an octave, lengths got a form measured at their band's top that was up to
+# 7 % slower there than the best)
 SIZES = tuple(sorted({2**e for e in range(12, 27)} | {2**e + 2**(e - 1) for e in range(12, 26)} |
                      {2**e + q * 2**(e - 2) for e in range(12, 22) for q in (1, 3)}))
 
